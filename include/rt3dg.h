@@ -243,8 +243,9 @@ rt_status rt_materialize_rays(const rt_bvh *bvh, const rt_rayspec *rays, const i
 /* ------------------------------------------------------------------------ */
 
 typedef enum {
-    RT_KERNEL_AUTO = 0,   /* DIRS sets: RAY_WIDE up to 2^19 Gaussians, WIDE
-                             beyond; ENV and HEMI sets: RAY_REFILL; explicit
+    RT_KERNEL_AUTO = 0,   /* DIRS sets: WIDE where neighbouring Gaussians lie
+                             close together (measured on the tree), else
+                             RAY_WIDE; ENV and HEMI sets: RAY_REFILL; explicit
                              rays and id lists: WARP_RAY up to 2^22 rays
                              (RAY_WIDE with a hit log), RAY_WIDE beyond (an id
                              list traced in the tree's order); the binary
@@ -253,7 +254,10 @@ typedef enum {
     RT_KERNEL_PACKET = 2, /* one warp per 32 rays of neighbouring Gaussians in
                              one direction, shared stack, binary tree          */
     RT_KERNEL_WIDE = 3,   /* as PACKET over the 4-wide tree (the binary tree
-                             collapsed by greedy largest-area expansion)       */
+                             collapsed by greedy largest-area expansion); a
+                             full DIRS set without counters or hit log: one
+                             warp per group of up to 64 neighbouring Gaussians
+                             and direction, walking the tree once for all   */
     RT_KERNEL_RAY_WIDE = 4, /* one thread per ray over the 4-wide tree        */
     RT_KERNEL_RAY_REFILL = 5, /* as RAY_WIDE, idle lanes refilled with new rays
                               as theirs finish (full implicit sets; otherwise

@@ -9,11 +9,13 @@
 // tiles spread over the Morton range, and keeps the fastest if it beats the
 // default strategy by more than 3 %.
 //
-// Batch: the work items (32 rays each) of all jobs form one virtual queue,
-// job after job in decreasing estimated cost (rays x log2 n), consumed
-// through one device counter by a persistent grid; each warp finds its job by
-// binary search over the jobs' first item and runs that job's strategy.  The
-// counter reset and the launch are captured into a CUDA graph at creation.
+// Batch: the work items of all jobs form virtual queues, job after job in
+// decreasing estimated cost (rays x log2 n), consumed through device counters
+// by persistent grids; each warp finds its job by binary search over the jobs'
+// first item and runs that job's strategy.  Shaft jobs (direction sets) have
+// a kernel of their own, since its shared memory would cost the other
+// strategies residency (20 instead of 32 warps); the two are parallel
+// branches of one captured CUDA graph with the counters' reset.
 #include <math.h>
 #include <string.h>
 
@@ -23,7 +25,7 @@
 #include <tuple>
 #include <vector>
 
-#include "rt_trace_core.cuh"
+#include "rt_shaft.cuh"
 
 rt_status rt_trace_launch_job(const BvhDev &b, const RaySetDev &rs, const TraceJob &job, float *T_out,
                               int strat, rt_stream_t stream, unsigned long long *work);
@@ -42,25 +44,29 @@ std::map<TuneKey, std::pair<int, int>> g_tune_cache;
 constexpr int kTuneBlocks = 4;
 constexpr float kTuneMargin = 0.97f;
 
-// The strategy used without tuning, as the single-scene AUTO: for a
-// direction set 4-wide packets sharing the direction, or one thread per ray
-// on the 4-wide tree (far-first) for scenes of at most 2^19 Gaussians; one
-// thread per ray on the 4-wide tree with lane refill for env-map and
-// hemisphere rays (their directions differ within a tile); binary variants
-// when there is no 4-wide tree.
+// The strategy used without tuning: for a direction set over more than 2^15
+// Gaussians shaft packets where they pay (rt_shaft_pays), else one thread per
+// ray on the 4-wide tree (far-first; small jobs keep the strategy they always
+// reported here, tuning finds the faster one); one thread per ray on the
+// 4-wide tree with lane refill for env-map and hemisphere rays (their
+// directions differ within a tile); binary variants when there is no 4-wide
+// tree.
 int default_kernel(const rt_bvh *bvh, int32_t kind) {
     if (kind == RT_RAYS_DIRS) {
         if (bvh->n_wide == 0) return RT_KERNEL_PACKET;
-        return bvh->n <= (int64_t(1) << 19) ? RT_KERNEL_RAY_WIDE : RT_KERNEL_WIDE;
+        return bvh->n > (int64_t(1) << 15) && rt_shaft_pays(bvh) ? RT_KERNEL_WIDE : RT_KERNEL_RAY_WIDE;
     }
     return bvh->n_wide > 0 ? RT_KERNEL_RAY_REFILL : RT_KERNEL_RAY;
 }
 
-TraceJob full_job(const rt_bvh *bvh, int32_t K, int32_t order_block) {
+// Items of a full implicit set: tiles of 32 Gaussians, or shaft groups.
+int64_t item_tiles(const rt_bvh *bvh, bool shaft) { return shaft ? bvh->n_groups : (bvh->n + 31) / 32; }
+
+TraceJob full_job(const rt_bvh *bvh, int32_t K, int32_t order_block, bool shaft) {
     TraceJob job;
     memset(&job, 0, sizeof(job));
     job.mode = MODE_FULL;
-    job.n_tiles = (bvh->n + 31) / 32;
+    job.n_tiles = item_tiles(bvh, shaft);
     int64_t B = order_block > 0 ? order_block : 1;
     if (B > job.n_tiles) B = job.n_tiles;
     if (B < 1) B = 1;
@@ -76,9 +82,9 @@ struct BatchJobDev {
     RaySetDev rs;
     TraceJob job;
     float *T_out;
-    int32_t strat;  // 0 per-ray, 1 packet, 2 4-wide packet, 3 4-wide packet with a shared direction,
+    int32_t strat;  // 0 per-ray, 1 packet, 2 4-wide packet, 3 shaft packet (direction sets),
                     // 4 per-ray 4-wide, 5 per-ray 4-wide with lane refill
-    int64_t item_begin;  // item jobs: first item of the item queue
+    int64_t item_begin;  // shaft and item jobs: first item of their queue
     int64_t slot_begin;  // refill jobs: first ray slot of the slot queue
 };
 
@@ -217,7 +223,6 @@ __global__ void __launch_bounds__(128, RT_BATCH_MIN_BLOCKS) k_trace_batch(const 
         const BatchJobDev &J = jobs[lo];
         const int64_t local = (int64_t)item - J.item_begin;
         if (J.strat == 4) trace_item<4, false>(J.b, J.rs, J.job, J.T_out, aux, local, J.job.n_out, wc, rays_done, stk);
-        else if (J.strat == 3) trace_item<3, false>(J.b, J.rs, J.job, J.T_out, aux, local, J.job.n_out, wc, rays_done, stk);
         else if (J.strat == 2) trace_item<2, false>(J.b, J.rs, J.job, J.T_out, aux, local, J.job.n_out, wc, rays_done, stk);
         else if (J.strat == 1) trace_item<1, false>(J.b, J.rs, J.job, J.T_out, aux, local, J.job.n_out, wc, rays_done, stk);
         else trace_item<0, false>(J.b, J.rs, J.job, J.T_out, aux, local, J.job.n_out, wc, rays_done, stk);
@@ -225,9 +230,31 @@ __global__ void __launch_bounds__(128, RT_BATCH_MIN_BLOCKS) k_trace_batch(const 
     if (total_slots > 0) batch_refill(jobs, n_item_jobs, n_jobs, total_slots, status, work + 1);
 }
 
-int persistent_grid() {
+// The shaft jobs [0, n_jobs) of a batch, their (group, direction) items one
+// queue.
+__global__ void __launch_bounds__(128, RT_SHAFT_MIN_BLOCKS) k_shaft_batch(const BatchJobDev *__restrict__ jobs, int n_jobs,
+                                                                          int64_t total_items, int *status,
+                                                                          unsigned long long *work) {
+    __shared__ ShaftSmem sm[4];
+    for (;;) {
+        unsigned long long item = 0;
+        if ((threadIdx.x & 31) == 0) item = atomicAdd(work, 1ull);
+        item = __shfl_sync(0xffffffffu, item, 0);
+        if ((int64_t)item >= total_items) break;
+        int lo = 0, hi = n_jobs - 1;  // last job with item_begin <= item
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (jobs[mid].item_begin <= (int64_t)item) lo = mid;
+            else hi = mid - 1;
+        }
+        const BatchJobDev &J = jobs[lo];
+        shaft_item(J.b, J.rs, J.job, J.T_out, (int64_t)item - J.item_begin, status, sm[threadIdx.x >> 5]);
+    }
+}
+
+int persistent_grid(const void *kernel) {
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_trace_batch, 128, 0) != cudaSuccess || per_sm < 1) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, 128, 0) != cudaSuccess || per_sm < 1) {
         cudaGetLastError();
         per_sm = 1;
     }
@@ -295,11 +322,14 @@ extern "C" rt_status rt_trace_autotune(const rt_bvh *bvh, const rt_rayspec *rays
             for (int rep = 0; rep < 2 && res == RT_OK; ++rep) {  // the first run warms caches
                 cudaEventRecord(e0, st);
                 for (int q = 0; q < nb && res == RT_OK; ++q) {
-                    TraceJob job = full_job(bvh, rs.K, blocks[bi]);
-                    job.n_tiles = S;
-                    job.tile_base = nb == 1 ? 0 : (ntiles - S) * (2 * q + 1) / (2 * nb);
-                    if (job.order_block > S) job.order_block = (int32_t)S;
-                    job.n_items = S * rs.K;
+                    const bool shaft = kernel == RT_KERNEL_WIDE && rays->kind == RT_RAYS_DIRS;
+                    TraceJob job = full_job(bvh, rs.K, blocks[bi], shaft);
+                    // the same share of the scene in tiles of 32 and in shaft groups
+                    const int64_t all = job.n_tiles, part = nb == 1 ? all : all * S / ntiles > 0 ? all * S / ntiles : 1;
+                    job.n_tiles = part;
+                    job.tile_base = nb == 1 ? 0 : (all - part) * (2 * q + 1) / (2 * nb);
+                    if (job.order_block > part) job.order_block = (int32_t)part;
+                    job.n_items = part * rs.K;
                     res = rt_trace_launch_job(b, rs, job, T_scratch, strat, stream, work + q);
                 }
                 cudaEventRecord(e1, st);
@@ -389,29 +419,34 @@ extern "C" rt_status rt_batch_create(const rt_batch_job *jobs, int32_t n_jobs, i
         memset(&H, 0, sizeof(H));
         H.b = bvh_dev(J.bvh);
         H.rs = rs;
-        H.job = full_job(J.bvh, rs.K, o.order_block);
         H.T_out = J.T_out;
         H.strat = o.kernel == RT_KERNEL_RAY_REFILL ? (J.bvh->n_wide > 0 ? 5 : 0)
                   : o.kernel == RT_KERNEL_RAY_WIDE ? (J.bvh->n_wide > 0 ? 4 : 0)
                   : o.kernel == RT_KERNEL_WIDE ? (J.bvh->n_wide > 0 ? (J.rays.kind == RT_RAYS_DIRS ? 3 : 2) : 1)
                   : o.kernel == RT_KERNEL_PACKET ? 1 : 0;
+        H.job = full_job(J.bvh, rs.K, o.order_block, H.strat == 3);
         cost[j] = (double)count * log2((double)(J.bvh->n > 1 ? J.bvh->n : 2));
     }
-    // item jobs first, then lane-refill jobs; largest estimated cost first in each
+    // shaft jobs (a queue and kernel of their own), item jobs, then lane-refill
+    // jobs; largest estimated cost first in each
     std::vector<int> order(n_jobs);
     for (int j = 0; j < n_jobs; ++j) order[j] = j;
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
-        const bool ra = host[a].strat == 5, rb = host[b].strat == 5;
-        return ra != rb ? rb : cost[a] > cost[b];
+        auto rank = [&](int j) { return host[j].strat == 3 ? 0 : host[j].strat == 5 ? 2 : 1; };
+        return rank(a) != rank(b) ? rank(a) < rank(b) : cost[a] > cost[b];
     });
     std::vector<BatchJobDev> queue(n_jobs);
-    int64_t items = 0, slots = 0, rays = 0;
-    int n_item_jobs = 0;
+    int64_t shafts = 0, items = 0, slots = 0, rays = 0;
+    int n_shaft_jobs = 0, n_item_jobs = 0;
     for (int q = 0; q < n_jobs; ++q) {
         queue[q] = host[order[q]];
         if (queue[q].strat == 5) {
             queue[q].slot_begin = slots;
             slots += queue[q].job.n_items * 32;
+        } else if (queue[q].strat == 3) {
+            queue[q].item_begin = shafts;
+            shafts += queue[q].job.n_items;
+            ++n_shaft_jobs;
         } else {
             queue[q].item_begin = items;
             items += queue[q].job.n_items;
@@ -419,7 +454,7 @@ extern "C" rt_status rt_batch_create(const rt_batch_job *jobs, int32_t n_jobs, i
         }
         rays += queue[q].job.n_out;
     }
-    bt->n_items = items + slots / 32;
+    bt->n_items = shafts + items + slots / 32;
     bt->n_rays = rays;
     const size_t tbytes = ((sizeof(BatchJobDev) * n_jobs + 255) & ~(size_t)255);
     rt_status r = rt_alloc(&bt->table, tbytes + 256, stream);
@@ -436,23 +471,39 @@ extern "C" rt_status rt_batch_create(const rt_batch_job *jobs, int32_t n_jobs, i
         delete bt;
         return RT_ERR_CUDA;
     }
-    // capture: reset the queue counter, one persistent launch
-    cudaStream_t cap;
-    if (cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking) != cudaSuccess) {
-        rt_free(bt->table, stream);
-        delete bt;
-        return RT_ERR_CUDA;
-    }
-    const int grid = persistent_grid();
+    // capture: reset the queue counters, then one persistent launch for the
+    // shaft jobs and one for the others on branches of their own, so that the
+    // second fills the multiprocessors as the first one's blocks leave
+    cudaStream_t cap = nullptr, side = nullptr;
+    cudaEvent_t fork = nullptr, join = nullptr;
+    bool ok = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking) == cudaSuccess &&
+              cudaStreamCreateWithFlags(&side, cudaStreamNonBlocking) == cudaSuccess &&
+              cudaEventCreateWithFlags(&fork, cudaEventDisableTiming) == cudaSuccess &&
+              cudaEventCreateWithFlags(&join, cudaEventDisableTiming) == cudaSuccess;
     int *status = rt_status_ptr();
-    bool ok = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
-    if (ok) {
-        cudaMemsetAsync(work, 0, 16, cap);
-        k_trace_batch<<<grid, 128, 0, cap>>>(dtab, n_item_jobs, n_jobs, items, slots, status, work);
+    if (ok && (ok = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal) == cudaSuccess)) {
+        const int n_other = n_jobs - n_shaft_jobs;
+        cudaMemsetAsync(work, 0, 24, cap);
+        if (n_other > 0) {
+            cudaEventRecord(fork, cap);
+            cudaStreamWaitEvent(side, fork, 0);
+        }
+        if (n_shaft_jobs > 0)
+            k_shaft_batch<<<persistent_grid((const void *)k_shaft_batch), 128, 0, cap>>>(dtab, n_shaft_jobs, shafts,
+                                                                                         status, work + 2);
+        if (n_other > 0) {
+            k_trace_batch<<<persistent_grid((const void *)k_trace_batch), 128, 0, side>>>(
+                dtab + n_shaft_jobs, n_item_jobs, n_other, items, slots, status, work);
+            cudaEventRecord(join, side);
+            cudaStreamWaitEvent(cap, join, 0);
+        }
         ok = cudaStreamEndCapture(cap, &bt->graph) == cudaSuccess;
     }
     if (ok) ok = cudaGraphInstantiate(&bt->exec, bt->graph, 0) == cudaSuccess;
-    cudaStreamDestroy(cap);
+    if (fork) cudaEventDestroy(fork);
+    if (join) cudaEventDestroy(join);
+    if (side) cudaStreamDestroy(side);
+    if (cap) cudaStreamDestroy(cap);
     if (!ok) {
         cudaGetLastError();
         if (bt->exec) cudaGraphExecDestroy(bt->exec);

@@ -352,6 +352,127 @@ __global__ void k_prep(const float *__restrict__ mean, const float *__restrict__
     }
 }
 
+// Shaft groups: each tile of 64 sorted positions is cut where its means lie
+// far apart (a jump of the Morton curve), since a packet of a direction set
+// walks the tree once per group with the box of the group's means.  A walk's
+// cost is taken as SA(box + one leaf) (10 + 0.27 rays): the Gaussians a shaft
+// of that box meets, times the issue slots one of them costs the walk and one
+// ray.  The cut of the largest gain is made first, until none gains.  One
+// warp per tile, lane l holds positions 2 l and 2 l + 1; the boxes left and
+// right of every cut come from two segmented scans.  The order of the list is
+// that of the tiles' arrival.
+struct Box6 {
+    float l[3], h[3];
+};
+__device__ __forceinline__ Box6 box_join(const Box6 &a, const Box6 &b) {
+    Box6 r;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        r.l[c] = fminf(a.l[c], b.l[c]);
+        r.h[c] = fmaxf(a.h[c], b.h[c]);
+    }
+    return r;
+}
+template <bool UP>
+__device__ __forceinline__ Box6 box_shfl(const Box6 &a, int off) {
+    Box6 r;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        r.l[c] = UP ? __shfl_up_sync(0xffffffffu, a.l[c], off) : __shfl_down_sync(0xffffffffu, a.l[c], off);
+        r.h[c] = UP ? __shfl_up_sync(0xffffffffu, a.h[c], off) : __shfl_down_sync(0xffffffffu, a.h[c], off);
+    }
+    return r;
+}
+__global__ void __launch_bounds__(128) k_tile_groups(const float4 *__restrict__ gauss,
+                                                     const float *__restrict__ leafbox, int64_t n, int2 *groups,
+                                                     unsigned *n_groups) {
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const int64_t tiles = (n + 63) / 64;
+    for (int64_t tile = blockIdx.x * 4ll + (threadIdx.x >> 5); tile < tiles; tile += 4ll * gridDim.x) {
+        const int64_t left = n - tile * 64;
+        const int cnt = (int)(left < 64 ? left : 64);
+        Box6 v[2];
+        float L[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const bool in = 2 * lane + r < cnt;
+            const int64_t p = tile * 64 + (in ? 2 * lane + r : 0);
+            const float4 g = gauss[4 * p];
+            const float m[3] = {g.x, g.y, g.z};
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                v[r].l[c] = in ? m[c] : INFINITY;
+                v[r].h[c] = in ? m[c] : -INFINITY;
+                const float e = leafbox[6 * p + 3 + c] - leafbox[6 * p + c];
+                if (in && e == e) L[c] += e / (float)cnt;  // an empty box is NaN
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+            for (int off = 16; off > 0; off >>= 1) L[c] += __shfl_xor_sync(FULL, L[c], off);
+        const Box6 both = box_join(v[0], v[1]);
+        uint64_t starts = 1ull | (cnt < 64 ? 1ull << cnt : 0ull);  // the end of a short tile closes its last group
+        for (int it = 0; it < 63; ++it) {
+            const bool sa = (starts >> (2 * lane)) & 1ull, sb = (starts >> (2 * lane + 1)) & 1ull;
+            const bool sn = lane == 31 || ((starts >> (2 * lane + 2)) & 1ull);
+            // pre: the box from the group's start through position 2 l + 1;
+            // suf: from position 2 l to the group's end
+            Box6 pre = sb ? v[1] : both, suf = sb ? v[0] : both;
+            int fp = sa || sb, fs = sb || sn;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const Box6 a = box_shfl<true>(pre, off), z = box_shfl<false>(suf, off);
+                const int ap = __shfl_up_sync(FULL, fp, off), zs = __shfl_down_sync(FULL, fs, off);
+                if (lane >= off && !fp) {
+                    pre = box_join(pre, a);
+                    fp = ap;
+                }
+                if (lane + off < 32 && !fs) {
+                    suf = box_join(suf, z);
+                    fs = zs;
+                }
+            }
+            const Box6 prv = box_shfl<true>(pre, 1), nxt = box_shfl<false>(suf, 1);
+            auto cost = [&](const Box6 &x, int rays) {
+                const float dx = x.h[0] - x.l[0] + L[0], dy = x.h[1] - x.l[1] + L[1], dz = x.h[2] - x.l[2] + L[2];
+                return (dx * dy + dy * dz + dz * dx) * (10.0f + 0.27f * (float)rays);
+            };
+            float gain = 0.0f;
+            int at = 0;
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {  // the cut in front of position 2 l + r
+                const int c = 2 * lane + r;
+                if (c == 0 || c >= cnt || (r ? sb : sa)) continue;
+                const uint64_t below = starts & ((1ull << c) - 1ull), above = starts >> c;
+                const int s0 = 63 - __clzll((long long)below), s1 = above ? c + __ffsll((long long)above) - 1 : cnt;
+                const Box6 A = r == 0 ? prv : sa ? v[0] : box_join(prv, v[0]);
+                const Box6 B = r == 0 ? suf : sn ? v[1] : box_join(nxt, v[1]);
+                const float g = cost(box_join(A, B), s1 - s0) - cost(A, c - s0) - cost(B, s1 - c);
+                if (g > gain) {
+                    gain = g;
+                    at = c;
+                }
+            }
+            const uint32_t key = __float_as_uint(gain), best = __reduce_max_sync(FULL, key);
+            if (best == 0u) break;
+            starts |= 1ull << __shfl_sync(FULL, at, __ffs(__ballot_sync(FULL, key == best)) - 1);
+        }
+        unsigned slot = 0;
+        const uint64_t own = cnt < 64 ? starts & ((1ull << cnt) - 1ull) : starts;
+        if (lane == 0) slot = atomicAdd(n_groups, (unsigned)__popcll(own));
+        slot = __shfl_sync(FULL, slot, 0);
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const int c = 2 * lane + r;
+            if (!((own >> c) & 1ull)) continue;
+            const uint64_t above = c < 63 ? starts >> (c + 1) : 0ull;
+            const int s1 = above ? c + __ffsll((long long)above) : cnt;
+            groups[slot + __popcll(own & ((1ull << c) - 1ull))] = make_int2((int)(tile * 64 + c), s1 - c);
+        }
+    }
+}
+
 __device__ __forceinline__ int lcp(const uint64_t *keys, int64_t n, int64_t i, int64_t j) {
     if (j < 0 || j >= n) return -1;
     return __clzll(keys[i] ^ keys[j]);
@@ -687,7 +808,8 @@ extern "C" rt_status rt_build_bvh(const float *mean, const float *scale, const f
     size_t off_keys = off_rank + align256(sizeof(int32_t) * (size_t)n);
     size_t off_par = off_keys + align256(sizeof(uint64_t) * (size_t)n);
     size_t off_bnd = off_par + align256(sizeof(int32_t) * (size_t)(n > 0 ? 2 * n - 1 : 0));
-    size_t off_wide = off_bnd + 256;
+    size_t off_grp = off_bnd + 256;
+    size_t off_wide = off_grp + align256(sizeof(int2) * (size_t)n);
     size_t total = off_wide + align256(sizeof(float4) * 8 * (size_t)ni);
     rt_status s = rt_alloc(&b->block, total, stream);
     if (s != RT_OK) {
@@ -703,8 +825,11 @@ extern "C" rt_status rt_build_bvh(const float *mean, const float *scale, const f
     b->keys = (uint64_t *)(base + off_keys);
     b->parent = (int32_t *)(base + off_par);
     b->bounds = (float *)(base + off_bnd);
+    b->groups = (int2 *)(base + off_grp);
+    b->n_groups = 0;
     b->wide = (float4 *)(base + off_wide);
     b->n_wide = 0;
+    b->levels = 0;
     b->links = nullptr;
     b->leaf_slot = b->wide_parent = nullptr;
     b->wide_arrivals = nullptr;
@@ -748,10 +873,10 @@ extern "C" rt_status rt_build_bvh(const float *mean, const float *scale, const f
     unsigned *wcnt = (unsigned *)(sb + s_cnt2);  // [0..63] level counts, [64] wide-node count (512 B region)
 
     rt_status result = RT_OK;
-    unsigned bad = 0;  // host copy of the input check (read with the bounds)
+    unsigned chk[2] = {0, 0};  // host copies of the input check and the group count (read with the bounds)
     do {
         if (cudaMemsetAsync(bounds_u, 0xff, 12, st) != cudaSuccess ||
-            cudaMemsetAsync(bounds_u + 3, 0, 20, st) != cudaSuccess) {
+            cudaMemsetAsync(bounds_u + 3, 0, 24, st) != cudaSuccess) {
             result = RT_ERR_CUDA;
             break;
         }
@@ -769,6 +894,7 @@ extern "C" rt_status rt_build_bvh(const float *mean, const float *scale, const f
         k_perm<<<grid_for(n, 256), 256, 0, st>>>(k0, v0, n, b->perm, b->rank, b->keys);
         k_prep<<<grid_for(n, 128), 128, 0, st>>>(mean, scale, quat, opacity, b->perm, n, prm, bounds_u,
                                                  b->gauss, leafbox);
+        k_tile_groups<<<grid_for((n + 63) / 64, 4), 128, 0, st>>>(b->gauss, leafbox, n, b->groups, bounds_u + 8);
         if (n == 1) {
             int32_t m1 = -1;
             if (cudaMemcpyAsync(b->parent, &m1, sizeof(int32_t), cudaMemcpyHostToDevice, st) != cudaSuccess)
@@ -795,9 +921,8 @@ extern "C" rt_status rt_build_bvh(const float *mean, const float *scale, const f
             for (int lvl = 0; lvl < 63; ++lvl)
                 k_collapse4<<<grid_c, 128, 0, st>>>(b->nodes, front[lvl & 1], wcnt + lvl, front[(lvl + 1) & 1],
                                                      wcnt + lvl + 1, wcnt + 64, b->wide);
-            unsigned nw = 0, left_over = 0;
-            if (cudaMemcpyAsync(&nw, wcnt + 64, sizeof(unsigned), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-                cudaMemcpyAsync(&left_over, wcnt + 63, sizeof(unsigned), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+            unsigned cnt[65] = {0};  // nodes of each level, then of the tree
+            if (cudaMemcpyAsync(cnt, wcnt, sizeof(cnt), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
                 cudaStreamSynchronize(st) != cudaSuccess) {
                 result = RT_ERR_CUDA;
                 break;
@@ -805,7 +930,8 @@ extern "C" rt_status rt_build_bvh(const float *mean, const float *scale, const f
             // a frontier left after the last level would mean an unfinished wide
             // tree (impossible for keys of <= 61 significant bits); then only
             // the binary tree is used
-            b->n_wide = (left_over || nw > (unsigned)ni) ? 0 : nw;
+            b->n_wide = (cnt[63] || cnt[64] > (unsigned)ni) ? 0 : cnt[64];
+            while (b->levels < 64 && cnt[b->levels]) ++b->levels;
         }
         if (rt_check_launch() != RT_OK) {
             result = RT_ERR_CUDA;
@@ -813,14 +939,15 @@ extern "C" rt_status rt_build_bvh(const float *mean, const float *scale, const f
         }
         if (cudaMemcpyAsync(b->lo, b->bounds, 3 * sizeof(float), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
             cudaMemcpyAsync(b->hi, b->bounds + 3, 3 * sizeof(float), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-            cudaMemcpyAsync(&bad, bounds_u + 7, sizeof(unsigned), cudaMemcpyDeviceToHost, st) != cudaSuccess) {
+            cudaMemcpyAsync(chk, bounds_u + 7, sizeof(chk), cudaMemcpyDeviceToHost, st) != cudaSuccess) {
             result = RT_ERR_CUDA;
             break;
         }
     } while (0);
     if (result == RT_OK && cudaStreamSynchronize(st) != cudaSuccess) result = RT_ERR_CUDA;
     rt_free(scratch, stream);
-    if (result == RT_OK && bad) result = RT_ERR_INVALID_ARG;
+    if (result == RT_OK && chk[0]) result = RT_ERR_INVALID_ARG;
+    b->n_groups = chk[1];
     if (result != RT_OK) {
         rt_free(b->block, stream);
         delete b;

@@ -15,7 +15,7 @@
 // for the same T.
 #include <string.h>
 
-#include "rt_trace_core.cuh"
+#include "rt_shaft.cuh"
 
 namespace {
 
@@ -160,16 +160,16 @@ __global__ void __launch_bounds__(128) k_pbr_shade_v(BvhDev b, ShadeDev S, const
 
 // Fused trace + reduction over all K rays of each Gaussian.  An item is a
 // tile of 32 Morton-adjacent Gaussians; the warp traces ray k of all 32
-// lanes together (STRAT 2/3: warp packet over the 4-wide tree, 3 when the
-// direction is shared; 4: one thread per ray) for k = 0..K-1.
+// lanes together (STRAT 2: warp packet over the 4-wide tree; 4: one thread per
+// ray) for k = 0..K-1.
 // MODE 0: PBR colour (Eq. 10); MODE 1: ambient occlusion (mean of T).
 template <int STRAT, int MODE>
 __global__ void __launch_bounds__(128, 8) k_trace_reduce(BvhDev b, RaySetDev rs, ShadeDev S, float *__restrict__ out,
                                                          int *status, unsigned long long *work) {
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
-    __shared__ int2 stk_all[(STRAT == 2 || STRAT == 3) ? 4 * RT_WIDE_STACK : 1];
-    int2 *stk = stk_all + ((STRAT == 2 || STRAT == 3) ? (threadIdx.x >> 5) * RT_WIDE_STACK : 0);
+    __shared__ int2 stk_all[STRAT == 2 ? 4 * RT_WIDE_STACK : 1];
+    int2 *stk = stk_all + (STRAT == 2 ? (threadIdx.x >> 5) * RT_WIDE_STACK : 0);
     extern __shared__ float env_s[];
     if (MODE == 0) load_env(S, env_s);
     const int64_t n_tiles = (b.n + 31) / 32;
@@ -198,7 +198,7 @@ __global__ void __launch_bounds__(128, 8) k_trace_reduce(BvhDev b, RaySetDev rs,
             const int32_t src = valid ? (int32_t)p : -1;
             float T;
             if (STRAT == 4) T = valid ? trace_ray_wide<false>(b, o, d, src, lg, wc, status, far_first(rs)) : 1.0f;
-            else T = trace_wide<false, STRAT == 3>(b, o, d, src, valid, lg, wc, status, stk);
+            else T = trace_wide<false>(b, o, d, src, valid, lg, wc, status, stk);
             if (!valid) continue;
             if (MODE == 0) {
                 // the per-Gaussian constants are rebuilt after each traversal
@@ -219,6 +219,39 @@ __global__ void __launch_bounds__(128, 8) k_trace_reduce(BvhDev b, RaySetDev rs,
         } else {
             out[g] = acc[0] / (float)rs.K;
         }
+    }
+}
+
+// Ambient occlusion of a direction set: an item is a shaft group, traced
+// along the K directions in turn, each lane summing its (up to two) rays.
+__global__ void __launch_bounds__(128, RT_SHAFT_MIN_BLOCKS) k_shaft_ao(BvhDev b, RaySetDev rs, int64_t n_groups,
+                                                                       float *__restrict__ ao, int *status,
+                                                                       unsigned long long *work) {
+    __shared__ ShaftSmem sm_all[4];
+    ShaftSmem &sm = sm_all[threadIdx.x >> 5];
+    const int lane = threadIdx.x & 31;
+    for (;;) {
+        unsigned long long item = 0;
+        if (lane == 0) item = atomicAdd(work, 1ull);
+        item = __shfl_sync(0xffffffffu, item, 0);
+        if ((int64_t)item >= n_groups) break;
+        const int2 gr = __ldg(b.groups + item);
+        float acc[2] = {0.0f, 0.0f};
+        for (int32_t k = 0; k < rs.K; ++k) {
+            shaft_group(b, rs.eps, make_float3(__ldg(rs.dirs + 3 * k), __ldg(rs.dirs + 3 * k + 1), __ldg(rs.dirs + 3 * k + 2)),
+                        gr.x, gr.y, status, sm);
+#pragma unroll
+            for (int r = 0; r < 2; ++r)
+                if (lane + 32 * r < gr.y) {
+                    const float T = sm.ro[lane + 32 * r].w;
+                    acc[r] += T < b.t_min ? 0.0f : T;
+                }
+            __syncwarp();
+        }
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+            if (lane + 32 * r < gr.y)
+                ao[__float_as_int(__ldg(b.gauss + 4 * (int64_t)(gr.x + lane + 32 * r) + 1).w)] = acc[r] / (float)rs.K;
     }
 }
 
@@ -254,8 +287,8 @@ rt_status shade_dev(const rt_bvh *bvh, const rt_rayspec *rays, const rt_pbr_inpu
     return RT_OK;
 }
 
-// strat: 2 warp packet (per-lane directions), 3 warp packet with a shared
-// direction (DIRS), 4 one thread per ray; all over the 4-wide tree.
+// strat: 2 warp packet (per-lane directions), 3 shaft packet (DIRS, MODE 1),
+// 4 one thread per ray; all over the 4-wide tree.
 template <int MODE>
 rt_status launch_reduce(const rt_bvh *bvh, const RaySetDev &rs, const ShadeDev &S, float *out, size_t smem,
                         int strat, cudaStream_t st) {
@@ -275,7 +308,11 @@ rt_status launch_reduce(const rt_bvh *bvh, const RaySetDev &rs, const ShadeDev &
         // handles it without touching one
         if (b.wide == nullptr && b.n >= 2) res = RT_ERR_UNSUPPORTED;
         else if (b.wide == nullptr) RT_REDUCE(4);
-        else if (strat == 3) RT_REDUCE(3);
+        else if (strat == 3) {  // ambient occlusion of a direction set
+            const int grid = grid_for((const void *)k_shaft_ao, 128, 0);
+            k_shaft_ao<<<grid, 128, 0, st>>>(b, rs, bvh->n_groups, out, rt_status_ptr(), work);
+            res = rt_check_launch();
+        }
         else if (strat == 2) RT_REDUCE(2);
         else RT_REDUCE(4);
 #undef RT_REDUCE
@@ -319,7 +356,7 @@ extern "C" rt_status rt_trace_ao(const rt_bvh *bvh, const rt_rayspec *rays, cons
     if (!ao) return RT_ERR_INVALID_ARG;
     ShadeDev S;
     memset(&S, 0, sizeof(S));
-    int strat = rays->kind == RT_RAYS_DIRS ? 3 : kHemiStrat;
+    int strat = rays->kind == RT_RAYS_DIRS && rt_shaft_pays(bvh) ? 3 : kHemiStrat;
     if (kernel == RT_KERNEL_WIDE) strat = rays->kind == RT_RAYS_DIRS ? 3 : 2;
     if (kernel == RT_KERNEL_RAY_WIDE) strat = 4;
     return launch_reduce<1>(bvh, rs, S, ao, 0, strat, (cudaStream_t)stream);

@@ -13,7 +13,7 @@
 // subsets are taken in chunks of 32 in the given order.
 #include <string.h>
 
-#include "rt_trace_core.cuh"
+#include "rt_shaft.cuh"
 
 // Resident blocks per SM the trace kernels are compiled for (register cap).
 #ifndef RT_TRACE_MIN_BLOCKS
@@ -27,8 +27,8 @@ __global__ void __launch_bounds__(128, RT_TRACE_MIN_BLOCKS) k_trace(BvhDev b, Ra
                                                TraceAux aux, unsigned long long *work) {
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
-    __shared__ int2 stk_all[(STRAT == 2 || STRAT == 3) ? 4 * RT_WIDE_STACK : 1];
-    int2 *stk = stk_all + ((STRAT == 2 || STRAT == 3) ? (threadIdx.x >> 5) * RT_WIDE_STACK : 0);
+    __shared__ int2 stk_all[STRAT == 2 ? 4 * RT_WIDE_STACK : 1];
+    int2 *stk = stk_all + (STRAT == 2 ? (threadIdx.x >> 5) * RT_WIDE_STACK : 0);
     WorkCounts wc = {0, 0, 0};
     unsigned long long rays_done = 0;
     if (STRAT == 5) {  // per-ray slots with lane refill (full implicit sets)
@@ -79,6 +79,20 @@ __global__ void __launch_bounds__(128, RT_TRACE_MIN_BLOCKS) k_trace(BvhDev b, Ra
         trace_item<STRAT, COUNT>(b, rs, job, T_out, aux, (int64_t)item, n_out, wc, rays_done, stk);
     }
     flush_counts<COUNT>(aux, wc, rays_done);
+}
+
+// Strategy 3 of a direction set: an item is a shaft group and a direction.
+__global__ void __launch_bounds__(128, RT_SHAFT_MIN_BLOCKS) k_trace_shaft(BvhDev b, RaySetDev rs, TraceJob job,
+                                                                          float *T_out, int *status,
+                                                                          unsigned long long *work) {
+    __shared__ ShaftSmem sm[4];
+    for (;;) {
+        unsigned long long item = 0;
+        if ((threadIdx.x & 31) == 0) item = atomicAdd(work, 1ull);
+        item = __shfl_sync(0xffffffffu, item, 0);
+        if ((int64_t)item >= job.n_items) break;
+        shaft_item(b, rs, job, T_out, (int64_t)item, status, sm[threadIdx.x >> 5]);
+    }
 }
 
 // Sort keys of an id list (per-ray traversal of long lists): rays of one
@@ -145,8 +159,8 @@ rt_status rt_trace_launch_job(const BvhDev &b, const RaySetDev &rs, const TraceJ
         k_trace<0, false><<<grid, threads, 0, st>>>(b, rs, job, T_out, aux, work);
     } else if (strat >= 2 && b.wide) {
         if (job.mode == MODE_FULL && rs.kind == RT_RAYS_DIRS) {
-            int grid = persistent_blocks((const void *)k_trace<3, false>, threads);
-            k_trace<3, false><<<grid, threads, 0, st>>>(b, rs, job, T_out, aux, work);
+            int grid = persistent_blocks((const void *)k_trace_shaft, threads);
+            k_trace_shaft<<<grid, threads, 0, st>>>(b, rs, job, T_out, aux.status, work);
         } else {
             int grid = persistent_blocks((const void *)k_trace<2, false>, threads);
             k_trace<2, false><<<grid, threads, 0, st>>>(b, rs, job, T_out, aux, work);
@@ -200,10 +214,12 @@ rt_status rt_trace_launch(const rt_bvh *bvh, const rt_rayspec *rays, float *T_ou
     // one warp per ray needs the 4-wide tree and keeps no hit log
     if (strat == 6 && (bvh->n_wide == 0 || o.hit_ids)) strat = bvh->n_wide ? 4 : 0;
     // AUTO:
-    // - a direction set: warp packets sharing the direction, except over at
-    //   most 2^19 Gaussians, where the per-ray walk (farthest child first)
-    //   is faster (object scenes: 100k 18 %, 300k 5 %, 500k 2.7 % with the
-    //   nearest child first; from 1M on the packets win);
+    // - a direction set: shaft packets where the groups are large enough
+    //   (rt_shaft_pays), else one thread per ray, farthest child first.  With
+    //   counters or a hit log, which shaft packets do not keep: one thread per
+    //   ray up to 2^19 Gaussians, plain packets beyond (object scenes: 100k
+    //   18 %, 300k 5 %, 500k 2.7 % in favour of the first; from 1M on the
+    //   packets win);
     // - env-map and hemisphere sets (directions differ across a tile): the
     //   per-ray walk with lane refill;
     // - explicit rays and id lists (scattered rays): one warp per ray up to
@@ -212,13 +228,18 @@ rt_status rt_trace_launch(const rt_bvh *bvh, const rt_rayspec *rays, float *T_ou
     //   walks), and one thread per ray over the 4-wide tree for longer lists
     //   (2^24 rays: 6 % faster than one warp per ray).
     if (o.kernel == RT_KERNEL_AUTO && job.mode == MODE_FULL)
-        strat = rays->kind == RT_RAYS_DIRS ? (bvh->n <= (int64_t(1) << 19) ? 4 : 2) : 5;
+        strat = rays->kind != RT_RAYS_DIRS ? 5
+                : o.counters || o.hit_ids  ? (bvh->n <= (int64_t(1) << 19) ? 4 : 2)
+                : rt_shaft_pays(bvh)       ? 2
+                                           : 4;
     if (o.kernel == RT_KERNEL_AUTO && job.mode != MODE_FULL) strat = count <= (int64_t(1) << 22) ? 6 : 4;
     // lane refill needs the 4-wide tree and a full implicit set, and keeps no hit log
     if (strat == 5 && (bvh->n_wide == 0 || job.mode != MODE_FULL || o.hit_ids)) strat = 4;
     if (strat == 2 && bvh->n_wide == 0) strat = 1;
     if (strat == 4 && bvh->n_wide == 0) strat = 0;
-    if (strat == 2 && job.mode == MODE_FULL && rays->kind == RT_RAYS_DIRS) strat = 3;  // shared direction
+    // a shared direction: shaft packets, which count no single ray's tests and
+    // keep no hit log (then the plain packet walk)
+    if (strat == 2 && job.mode == MODE_FULL && rays->kind == RT_RAYS_DIRS && !o.counters && !o.hit_ids) strat = 3;
 
     TraceAux aux;
     aux.counters = (unsigned long long *)o.counters;
@@ -279,7 +300,14 @@ rt_status rt_trace_launch(const rt_bvh *bvh, const rt_rayspec *rays, float *T_ou
         if (strat == 6) { if (count) RT_LAUNCH(6, true); else RT_LAUNCH(6, false); }
         else if (strat == 5) { if (count) RT_LAUNCH(5, true); else RT_LAUNCH(5, false); }
         else if (strat == 4) { if (count) RT_LAUNCH(4, true); else RT_LAUNCH(4, false); }
-        else if (strat == 3) { if (count) RT_LAUNCH(3, true); else RT_LAUNCH(3, false); }
+        else if (strat == 3) {
+            // its items are shaft groups instead of tiles
+            job.n_tiles = bvh->n_groups;
+            if (job.order_block > job.n_tiles) job.order_block = (int32_t)job.n_tiles;
+            job.n_items = job.n_tiles * rs.K;
+            int grid = persistent_blocks((const void *)k_trace_shaft, threads);
+            k_trace_shaft<<<grid, threads, 0, st>>>(b, rs, job, T_out, aux.status, work);
+        }
         else if (strat == 2) { if (count) RT_LAUNCH(2, true); else RT_LAUNCH(2, false); }
         else if (strat == 1) { if (count) RT_LAUNCH(1, true); else RT_LAUNCH(1, false); }
         else { if (count) RT_LAUNCH(0, true); else RT_LAUNCH(0, false); }

@@ -9,7 +9,9 @@ struct BvhDev {
     const float4 *nodes;
     const float4 *wide;  // null if the 4-wide tree is unavailable
     const int32_t *rank;
+    const int2 *groups;  // first sorted position and count of each shaft group
     int64_t n;
+    int32_t levels;      // levels of the 4-wide tree
     float k2;         // k_sigma^2
     float alpha_min;
     float t_min;
@@ -21,7 +23,9 @@ inline BvhDev bvh_dev(const rt_bvh *b) {
     d.nodes = b->nodes;
     d.wide = b->n_wide > 0 ? b->wide : nullptr;
     d.rank = b->rank;
+    d.groups = b->groups;
     d.n = b->n;
+    d.levels = b->levels;
     d.k2 = b->params.k_sigma * b->params.k_sigma;
     d.alpha_min = b->params.alpha_min;
     d.t_min = b->params.t_min;
@@ -173,25 +177,6 @@ __device__ __forceinline__ bool visit_order(float t0, float t1, float t2, float 
 // child first.
 __device__ __forceinline__ bool far_first(const RaySetDev &rs) { return rs.kind == RT_RAYS_DIRS; }
 
-// The slab test of two children at once with the planes already ordered
-// along the ray (near plane first on every axis: slab() without the per-axis
-// min/max): the plane distances of both along an axis come from one packed
-// FMA (fma.rn.f32x2 rounds each half as fmaf), so each packed instruction
-// does the work of two issued ones.  i* = (inv, inv), o* = (-oi, -oi).
-__device__ __forceinline__ void slab_sorted2(float2 nx, float2 fx, float2 ny, float2 fy, float2 nz, float2 fz,
-                                             float2 ix, float2 iy, float2 iz, float2 ox, float2 oy, float2 oz,
-                                             bool &ha, bool &hb) {
-    const float2 tnx = __ffma2_rn(nx, ix, ox), tfx = __ffma2_rn(fx, ix, ox);
-    const float2 tny = __ffma2_rn(ny, iy, oy), tfy = __ffma2_rn(fy, iy, oy);
-    const float2 tnz = __ffma2_rn(nz, iz, oz), tfz = __ffma2_rn(fz, iz, oz);
-    const float na = fmaxf(fmaxf(tnx.x, tny.x), fmaxf(tnz.x, 0.0f));
-    const float fa = fminf(fminf(tfx.x, tfy.x), tfz.x);
-    const float nb = fmaxf(fmaxf(tnx.y, tny.y), fmaxf(tnz.y, 0.0f));
-    const float fb = fminf(fminf(tfx.y, tfy.y), tfz.y);
-    ha = na <= fmaf(fabsf(fa), 1e-6f, fa);
-    hb = nb <= fmaf(fabsf(fb), 1e-6f, fb);
-}
-
 // Peak response of the Gaussian at sorted position p along the ray
 // (Eq. 13-14 with Sigma^-1).  In the whitened frame u = W (x - mu) the squared
 // Mahalanobis distance along the ray is |u_o + t u_d|^2, minimised at
@@ -217,12 +202,8 @@ __device__ __forceinline__ void two_diff2(float2 a, float2 b, float2 &hi, float2
     hi = s;
 }
 
-__device__ __forceinline__ bool gauss_eval(const BvhDev &b, int32_t p, float3 o, float3 d, float &alpha,
-                                           float3 &e) {
-    const float4 g0 = __ldg(b.gauss + 4 * p);
-    const float4 g1 = __ldg(b.gauss + 4 * p + 1);
-    const float4 g2 = __ldg(b.gauss + 4 * p + 2);
-    const float4 g3 = __ldg(b.gauss + 4 * p + 3);
+__device__ __forceinline__ bool gauss_eval(const BvhDev &b, float4 g0, float4 g1, float4 g2, float4 g3, float3 o,
+                                           float3 d, float &alpha, float3 &e) {
     float2 hxy, lxy;
     two_diff2(make_float2(o.x, o.y), make_float2(g0.x, g0.y), hxy, lxy);
     const float hx = hxy.x, hy = hxy.y;
@@ -243,6 +224,12 @@ __device__ __forceinline__ bool gauss_eval(const BvhDev &b, int32_t p, float3 o,
     if (!(m2 <= b.k2)) return false;
     alpha = g0.w * __expf(-0.5f * m2);
     return alpha >= b.alpha_min;
+}
+
+__device__ __forceinline__ bool gauss_eval(const BvhDev &b, int32_t p, float3 o, float3 d, float &alpha,
+                                           float3 &e) {
+    return gauss_eval(b, __ldg(b.gauss + 4 * p), __ldg(b.gauss + 4 * p + 1), __ldg(b.gauss + 4 * p + 2),
+                      __ldg(b.gauss + 4 * p + 3), o, d, alpha, e);
 }
 
 // gauss_eval and, when accepted, the transmittance update of Eq. 15.
@@ -444,10 +431,7 @@ __device__ __forceinline__ float trace_packet(const BvhDev &b, float3 o, float3 
 // tests four child boxes per lane (one float4 of each coordinate), evaluates
 // the leaf children each lane hit, and pushes all but one of the internal
 // children some lane still needs onto a warp stack in shared memory.
-// UNIFORM: every lane has the same direction (a direction set): each box is
-// then tested against its near and far planes, chosen once per packet from
-// the direction's signs, without per-box min/max.
-template <bool COUNT, bool UNIFORM>
+template <bool COUNT>
 __device__ __forceinline__ float trace_wide(const BvhDev &b, float3 o, float3 d, int32_t src, bool valid,
                                             LaneLog &lg, WorkCounts &wc, int *status, int2 *stk) {
     const unsigned FULL = 0xffffffffu;
@@ -466,9 +450,6 @@ __device__ __forceinline__ float trace_wide(const BvhDev &b, float3 o, float3 d,
     }
     const float3 inv = safe_inv(d);
     const float3 oi = make_float3(o.x * inv.x, o.y * inv.y, o.z * inv.z);
-    const int sx = inv.x < 0.0f, sy = inv.y < 0.0f, sz = inv.z < 0.0f;
-    const float2 ix2 = make_float2(inv.x, inv.x), iy2 = make_float2(inv.y, inv.y), iz2 = make_float2(inv.z, inv.z);
-    const float2 ox2 = make_float2(-oi.x, -oi.x), oy2 = make_float2(-oi.y, -oi.y), oz2 = make_float2(-oi.z, -oi.z);
     uint32_t alive = __ballot_sync(FULL, valid);
     int sp = 0;
     uint32_t node = 0, mask = alive;
@@ -479,29 +460,15 @@ __device__ __forceinline__ float trace_wide(const BvhDev &b, float3 o, float3 d,
         const uint32_t r0 = __float_as_uint(rf.x), r1 = __float_as_uint(rf.y), r2 = __float_as_uint(rf.z),
                        r3 = __float_as_uint(rf.w);
         bool h0 = false, h1 = false, h2 = false, h3 = false;
-        if (UNIFORM) {
-            // near/far planes by the shared direction's signs (sx = 1 if d.x < 0)
-            const float4 nx = __ldg(w + sx), fx = __ldg(w + 1 - sx), ny = __ldg(w + 2 + sy),
-                         fy = __ldg(w + 3 - sy), nz = __ldg(w + 4 + sz), fz = __ldg(w + 5 - sz);
-            if (mine) {
-                slab_sorted2(make_float2(nx.x, nx.y), make_float2(fx.x, fx.y), make_float2(ny.x, ny.y),
-                             make_float2(fy.x, fy.y), make_float2(nz.x, nz.y), make_float2(fz.x, fz.y), ix2, iy2, iz2,
-                             ox2, oy2, oz2, h0, h1);
-                slab_sorted2(make_float2(nx.z, nx.w), make_float2(fx.z, fx.w), make_float2(ny.z, ny.w),
-                             make_float2(fy.z, fy.w), make_float2(nz.z, nz.w), make_float2(fz.z, fz.w), ix2, iy2, iz2,
-                             ox2, oy2, oz2, h2, h3);
-            }
-        } else {
-            const float4 lx = __ldg(w), hx = __ldg(w + 1), ly = __ldg(w + 2), hy = __ldg(w + 3),
-                         lz = __ldg(w + 4), hz = __ldg(w + 5);
-            if (mine) {
-                bool h[4];
-                slab4(lx, hx, ly, hy, lz, hz, oi, inv, h);
-                h0 = h[0];
-                h1 = h[1];
-                h2 = h[2];
-                h3 = h[3];
-            }
+        const float4 lx = __ldg(w), hx = __ldg(w + 1), ly = __ldg(w + 2), hy = __ldg(w + 3), lz = __ldg(w + 4),
+                     hz = __ldg(w + 5);
+        if (mine) {
+            bool h[4];
+            slab4(lx, hx, ly, hy, lz, hz, oi, inv, h);
+            h0 = h[0];
+            h1 = h[1];
+            h2 = h[2];
+            h3 = h[3];
         }
         if (COUNT && mine) wc.box += (r0 != RT_EMPTY) + (r1 != RT_EMPTY) + (r2 != RT_EMPTY) + (r3 != RT_EMPTY);
         // leaf children this lane hit, one Gaussian test each
@@ -711,9 +678,8 @@ __device__ __forceinline__ bool ray_of(const BvhDev &b, const RaySetDev &rs, con
 
 // One work item (32 rays) of a trace job: build each lane's ray, traverse,
 // write T (and the hit log).  Shared by the single-scene and batched kernels.
-// STRAT: 0 per-ray binary, 1 packet binary, 2 packet 4-wide, 3 packet 4-wide
-// for a direction set (all lanes share the direction), 4 per-ray 4-wide
-// (stk: this warp's RT_WIDE_STACK shared-memory entries, strategies 2-3).
+// STRAT: 0 per-ray binary, 1 packet binary, 2 packet 4-wide, 4 per-ray 4-wide
+// (stk: this warp's RT_WIDE_STACK shared-memory entries, strategy 2).
 template <int STRAT, bool COUNT>
 __device__ __forceinline__ void trace_item(const BvhDev &b, const RaySetDev &rs, const TraceJob &job,
                                            float *T_out, const TraceAux &aux, int64_t item, int64_t n_out,
@@ -772,10 +738,8 @@ __device__ __forceinline__ void trace_item(const BvhDev &b, const RaySetDev &rs,
     float T;
     if (STRAT == 4) {
         T = valid ? trace_ray_wide<COUNT>(b, o, d, src, lg, wc, aux.status, far_first(rs)) : 1.0f;
-    } else if (STRAT == 3) {
-        T = trace_wide<COUNT, true>(b, o, d, src, valid, lg, wc, aux.status, stk);
     } else if (STRAT == 2) {
-        T = trace_wide<COUNT, false>(b, o, d, src, valid, lg, wc, aux.status, stk);
+        T = trace_wide<COUNT>(b, o, d, src, valid, lg, wc, aux.status, stk);
     } else if (STRAT == 1) {
         T = trace_packet<COUNT>(b, o, d, src, valid, lg, wc, aux.status);
     } else {
