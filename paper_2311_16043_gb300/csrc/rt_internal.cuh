@@ -214,8 +214,7 @@ __device__ __forceinline__ HemiFrame hemi_frame(const float *nrm) {
 }
 
 // Local direction h (z along the normal) in the frame: (h.x t1 + h.y t2) + h.z n.
-__device__ __forceinline__ float3 hemi_rotate(const HemiFrame &f, const float *h) {
-    const float hx = __ldg(h), hy = __ldg(h + 1), hz = __ldg(h + 2);
+__device__ __forceinline__ float3 hemi_rotate(const HemiFrame &f, float hx, float hy, float hz) {
     return make_float3(__fadd_rn(__fadd_rn(__fmul_rn(hx, f.t1.x), __fmul_rn(hy, f.t2.x)), __fmul_rn(hz, f.n.x)),
                        __fadd_rn(__fadd_rn(__fmul_rn(hx, f.t1.y), __fmul_rn(hy, f.t2.y)), __fmul_rn(hz, f.n.y)),
                        __fadd_rn(__fadd_rn(__fmul_rn(hx, f.t1.z), __fmul_rn(hy, f.t2.z)), __fmul_rn(hz, f.n.z)));
@@ -228,7 +227,8 @@ __device__ __forceinline__ void implicit_ray(const RaySetDev &rs, int64_t r, int
     if (rs.kind == RT_RAYS_DIRS) {
         d = make_float3(rs.dirs[3 * k], rs.dirs[3 * k + 1], rs.dirs[3 * k + 2]);
     } else if (rs.kind == RT_RAYS_HEMI) {
-        d = hemi_rotate(hemi_frame(rs.normals + 3 * g), rs.dirs + 3 * k);
+        d = hemi_rotate(hemi_frame(rs.normals + 3 * g), __ldg(rs.dirs + 3 * k), __ldg(rs.dirs + 3 * k + 1),
+                        __ldg(rs.dirs + 3 * k + 2));
     } else {
         d = env_direction(rs, r);
     }
