@@ -126,8 +126,7 @@ rt_status rt_bvh_destroy(rt_bvh *bvh, rt_stream_t stream);
  * moves during optimisation; traversal stays exact for any input (boxes
  * always contain the supports), it only loses efficiency as the Morton order
  * goes stale.  The scene bounds reported by rt_bvh_info stay those of the
- * build.  Asynchronous on `stream` (the first call also derives the 4-wide
- * tree's parent links once).  Refitting with the build's inputs reproduces
+ * build.  Asynchronous on `stream`.  Refitting with the build's inputs reproduces
  * the built tree bit for bit.  Errors: RT_ERR_INVALID_ARG (inputs failing the
  * check of rt_build_bvh are reported through the status word, since the call
  * does not synchronise). */

@@ -22,8 +22,9 @@
 //   nd[4i+0] = (L.lo.x, L.hi.x, L.lo.y, L.hi.y)
 //   nd[4i+1] = (L.lo.z, L.hi.z, R.lo.x, R.hi.x)
 //   nd[4i+2] = (R.lo.y, R.hi.y, R.lo.z, R.hi.z)
-//   nd[4i+3] = (left ref, right ref, 0, 0) as int bits; bit 31 = leaf,
-//              low bits = sorted position of the leaf's Gaussian.
+//   nd[4i+3] = (left ref, right ref, first, last) as int bits; bit 31 of a
+//              ref = leaf, low bits = sorted position of the leaf's Gaussian;
+//              first..last = the node's sorted positions.
 // ---------------------------------------------------------------------------
 
 #define RT_LEAF_BIT 0x80000000u
@@ -31,7 +32,8 @@
 #define RT_STACK 64  // >= tree depth: keys are 64-bit and unique
 #define RT_WIDE_STACK 256  // >= 3 pushes x 64 levels of the 4-wide tree
 
-// 4-wide node record, 128 B = 8 x float4, node j (root = 0):
+// 4-wide node record, 128 B = 8 x float4, node j (root = 0; j is the index of
+// the binary node it starts from, indices between are unused):
 //   w[8j+0..5] = lo.x[4], hi.x[4], lo.y[4], hi.y[4], lo.z[4], hi.z[4]
 //   w[8j+6]    = child refs (int bits): bit 31 = leaf (sorted position),
 //                RT_EMPTY = no child, else a wide node index
@@ -54,15 +56,8 @@ struct rt_bvh {
     int2 *groups;            // [n_groups] first sorted position and count of each shaft group
     int64_t n_groups;        // (host copy)
     float4 *wide;            // [8 * (n-1)] 4-wide nodes (collapsed binary tree)
-    int64_t n_wide;          // number of 4-wide nodes (host copy)
-    int32_t levels;          // levels of the 4-wide tree (host copy)
-    // refit links, made by the first rt_bvh_refit: 4*w + slot of each leaf
-    // (sorted position) and of each wide node in its wide parent (root: -1),
-    // and per-wide-node arrival counters
-    void *links;
-    int32_t *leaf_slot;      // [n]
-    int32_t *wide_parent;    // [n_wide]
-    uint32_t *wide_arrivals; // [n_wide]
+    int64_t n_wide;          // indices of 4-wide nodes: n-1, or 0 for n < 2
+    int32_t levels;          // levels of the binary tree, a bound on the 4-wide one's (host copy)
 };
 
 struct rt_envmap {

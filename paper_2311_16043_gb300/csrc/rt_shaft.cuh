@@ -48,7 +48,7 @@
 constexpr int kShaftRays = 64;      // rays of a group at most
 constexpr int kShaftCands = 64;     // Gaussians of a batch
 constexpr int kShaftNodes = 16;     // nodes of a step
-constexpr int kShaftStack = 256;    // nodes; a walk of single nodes adds 3 per level at most (193 for 64 levels)
+constexpr int kShaftStack = 320;    // nodes; a walk of single nodes adds 3 per level at most (193 for 64 levels)
 constexpr int kShaftPairs = 256;
 
 struct __align__(16) ShaftSmem {
@@ -58,7 +58,6 @@ struct __align__(16) ShaftSmem {
     float z[kShaftRays];                      //   and along d
     uint2 mask[kShaftRays];                   // by slot: Gaussians of the batch to evaluate
     float4 fr[5];                             // the shaft's frame (see shaft_cand)
-    uint32_t ids[kShaftCands];                // the batch's Gaussians (sorted positions)
     uint32_t stack[kShaftStack];
     uint32_t leaf[kShaftCands + 4 * kShaftNodes];  // fewer than a batch left over + one step's
     uint32_t pair[kShaftPairs];               // ray << 6 | Gaussian, then the pair's factor
@@ -338,8 +337,6 @@ __device__ __forceinline__ void shaft_group(const BvhDev &b, float eps, float3 d
             if (i < m)
                 cp_async16(sm.stage + 4 * i + ((lane ^ (i >> 1)) & 3), b.gauss + 4 * (int64_t)sm.leaf[nleaf + i] + (lane & 3));
         }
-        if (lane < m) sm.ids[lane] = sm.leaf[nleaf + lane];
-        if (lane + 32 < m) sm.ids[lane + 32] = sm.leaf[nleaf + lane + 32];
         cp_async_done();
         __syncwarp();
         ShaftCand g;
@@ -402,8 +399,8 @@ __device__ __forceinline__ void shaft_group(const BvhDev &b, float eps, float3 d
                     const float4 rb[4] = {rec(qb, 0), rec(qb, 1), rec(qb, 2), rec(qb, 3)};
                     float fa, fb;
                     gauss_factor2(b, ra, rb, oa, ob, d, fa, fb);
-                    if (sm.ids[qa] == (uint32_t)first + (pa >> 6)) fa = 1.0f;  // the ray's own Gaussian
-                    if (sm.ids[qb] == (uint32_t)first + (pb >> 6)) fb = 1.0f;
+                    if (sm.leaf[nleaf + qa] == (uint32_t)first + (pa >> 6)) fa = 1.0f;  // the ray's own Gaussian
+                    if (sm.leaf[nleaf + qb] == (uint32_t)first + (pb >> 6)) fb = 1.0f;
                     sm.pair[i] = __float_as_uint(fa);
                     if (i + 32 < total) sm.pair[i + 32] = __float_as_uint(fb);
                 }

@@ -11,7 +11,7 @@ struct BvhDev {
     const int32_t *rank;
     const int2 *groups;  // first sorted position and count of each shaft group
     int64_t n;
-    int32_t levels;      // levels of the 4-wide tree
+    int32_t levels;      // at least the levels of the 4-wide tree
     float k2;         // k_sigma^2
     float alpha_min;
     float t_min;
