@@ -60,10 +60,8 @@ __device__ __forceinline__ void grad_add(const GradOut &G, float *dst, int64_t i
 // reciprocal because m^2 itself is stationary in t).
 __device__ __forceinline__ void peak_accurate(const BvhDev &b, int32_t p, float3 o, float3 d, float &alpha,
                                               float3 &e) {
-    const float4 g0 = __ldg(b.gauss + 4 * p);
-    const float4 g1 = __ldg(b.gauss + 4 * p + 1);
-    const float4 g2 = __ldg(b.gauss + 4 * p + 2);
-    const float4 g3 = __ldg(b.gauss + 4 * p + 3);
+    const float4x2 r0 = ldg_pair(b.gauss + 4 * (int64_t)p), r1 = ldg_pair(b.gauss + 4 * (int64_t)p + 2);
+    const float4 g0 = r0.a, g1 = r0.b, g2 = r1.a, g3 = r1.b;
     float hx, lx, hy, ly, hz, lz;
     two_diff(o.x, g0.x, hx, lx);
     two_diff(o.y, g0.y, hy, ly);
@@ -187,10 +185,8 @@ __global__ void __launch_bounds__(128) k_backward(BvhDev b, RaySetDev rs, int64_
                 int sp = 0;
                 uint32_t node = 0;
                 for (;;) {
-                    const float4 n0 = __ldg(b.nodes + 4 * node);
-                    const float4 n1 = __ldg(b.nodes + 4 * node + 1);
-                    const float4 n2 = __ldg(b.nodes + 4 * node + 2);
-                    const float4 n3 = __ldg(b.nodes + 4 * node + 3);
+                    const float4x2 q0 = ldg_pair(b.nodes + 4 * (int64_t)node), q1 = ldg_pair(b.nodes + 4 * (int64_t)node + 2);
+        const float4 n0 = q0.a, n1 = q0.b, n2 = q1.a, n3 = q1.b;
                     bool hl = slab(n0.x, n0.y, n0.z, n0.w, n1.x, n1.y, oi, inv);
                     bool hr = slab(n1.z, n1.w, n2.x, n2.y, n2.z, n2.w, oi, inv);
                     const uint32_t ch[2] = {__float_as_uint(n3.x), __float_as_uint(n3.y)};

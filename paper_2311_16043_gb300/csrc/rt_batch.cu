@@ -153,8 +153,8 @@ __device__ __forceinline__ void batch_refill(const BatchJobDev *__restrict__ job
         const BvhDev &b = jobs[jl].b;
         const bool far = far_first(jobs[jl].rs);
         const float4 *w = b.wide + 8 * (int64_t)node;
-        const float4 lx = __ldg(w), hx = __ldg(w + 1), ly = __ldg(w + 2), hy = __ldg(w + 3), lz = __ldg(w + 4),
-                     hz = __ldg(w + 5), rf = __ldg(w + 6);
+        const float4x2 nx = ldg_pair(w), ny = ldg_pair(w + 2), nz = ldg_pair(w + 4), nr = ldg_pair(w + 6);
+        const float4 lx = nx.a, hx = nx.b, ly = ny.a, hy = ny.b, lz = nz.a, hz = nz.b, rf = nr.a;
         const uint32_t r[4] = {__float_as_uint(rf.x), __float_as_uint(rf.y), __float_as_uint(rf.z),
                                __float_as_uint(rf.w)};
         float tn[4];

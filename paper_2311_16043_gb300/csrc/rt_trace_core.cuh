@@ -228,8 +228,8 @@ __device__ __forceinline__ bool gauss_eval(const BvhDev &b, float4 g0, float4 g1
 
 __device__ __forceinline__ bool gauss_eval(const BvhDev &b, int32_t p, float3 o, float3 d, float &alpha,
                                            float3 &e) {
-    return gauss_eval(b, __ldg(b.gauss + 4 * p), __ldg(b.gauss + 4 * p + 1), __ldg(b.gauss + 4 * p + 2),
-                      __ldg(b.gauss + 4 * p + 3), o, d, alpha, e);
+    const float4x2 r = ldg_pair(b.gauss + 4 * (int64_t)p), s = ldg_pair(b.gauss + 4 * (int64_t)p + 2);
+    return gauss_eval(b, r.a, r.b, s.a, s.b, o, d, alpha, e);
 }
 
 // gauss_eval and, when accepted, the transmittance update of Eq. 15.
@@ -272,10 +272,8 @@ __device__ __forceinline__ float trace_ray(const BvhDev &b, float3 o, float3 d, 
     int sp = 0;
     uint32_t node = 0;
     for (;;) {
-        const float4 n0 = __ldg(b.nodes + 4 * node);
-        const float4 n1 = __ldg(b.nodes + 4 * node + 1);
-        const float4 n2 = __ldg(b.nodes + 4 * node + 2);
-        const float4 n3 = __ldg(b.nodes + 4 * node + 3);
+        const float4x2 q0 = ldg_pair(b.nodes + 4 * (int64_t)node), q1 = ldg_pair(b.nodes + 4 * (int64_t)node + 2);
+        const float4 n0 = q0.a, n1 = q0.b, n2 = q1.a, n3 = q1.b;
         bool hl = slab(n0.x, n0.y, n0.z, n0.w, n1.x, n1.y, oi, inv);
         bool hr = slab(n1.z, n1.w, n2.x, n2.y, n2.z, n2.w, oi, inv);
         if (COUNT) wc.box += 2;
@@ -353,10 +351,8 @@ __device__ __forceinline__ float trace_packet(const BvhDev &b, float3 o, float3 
     uint32_t node = 0, mask = alive;
     while (mask) {
         const bool mine = (mask >> lane) & 1u;
-        const float4 n0 = __ldg(b.nodes + 4 * node);
-        const float4 n1 = __ldg(b.nodes + 4 * node + 1);
-        const float4 n2 = __ldg(b.nodes + 4 * node + 2);
-        const float4 n3 = __ldg(b.nodes + 4 * node + 3);
+        const float4x2 q0 = ldg_pair(b.nodes + 4 * (int64_t)node), q1 = ldg_pair(b.nodes + 4 * (int64_t)node + 2);
+        const float4 n0 = q0.a, n1 = q0.b, n2 = q1.a, n3 = q1.b;
         bool hl = false, hr = false;
         if (mine) {
             hl = slab(n0.x, n0.y, n0.z, n0.w, n1.x, n1.y, oi, inv);
@@ -456,12 +452,12 @@ __device__ __forceinline__ float trace_wide(const BvhDev &b, float3 o, float3 d,
     while (mask) {
         const bool mine = (mask >> lane) & 1u;
         const float4 *w = b.wide + 8 * (int64_t)node;
+        const float4x2 px = ldg_pair(w), py = ldg_pair(w + 2), pz = ldg_pair(w + 4);
         const float4 rf = __ldg(w + 6);
         const uint32_t r0 = __float_as_uint(rf.x), r1 = __float_as_uint(rf.y), r2 = __float_as_uint(rf.z),
                        r3 = __float_as_uint(rf.w);
         bool h0 = false, h1 = false, h2 = false, h3 = false;
-        const float4 lx = __ldg(w), hx = __ldg(w + 1), ly = __ldg(w + 2), hy = __ldg(w + 3), lz = __ldg(w + 4),
-                     hz = __ldg(w + 5);
+        const float4 lx = px.a, hx = px.b, ly = py.a, hy = py.b, lz = pz.a, hz = pz.b;
         if (mine) {
             bool h[4];
             slab4(lx, hx, ly, hy, lz, hz, oi, inv, h);
@@ -551,8 +547,8 @@ __device__ __forceinline__ void trace_ray_wide_run(const BvhDev &b, float3 o, fl
     uint32_t node = 0;
     for (;;) {
         const float4 *w = b.wide + 8 * (int64_t)node;
-        const float4 lx = __ldg(w), hx = __ldg(w + 1), ly = __ldg(w + 2), hy = __ldg(w + 3), lz = __ldg(w + 4),
-                     hz = __ldg(w + 5), rf = __ldg(w + 6);
+        const float4x2 nx = ldg_pair(w), ny = ldg_pair(w + 2), nz = ldg_pair(w + 4), nr = ldg_pair(w + 6);
+        const float4 lx = nx.a, hx = nx.b, ly = ny.a, hy = ny.b, lz = nz.a, hz = nz.b, rf = nr.a;
         const uint32_t r[4] = {__float_as_uint(rf.x), __float_as_uint(rf.y), __float_as_uint(rf.z),
                                __float_as_uint(rf.w)};
         float tn[4];
@@ -836,8 +832,8 @@ __device__ __forceinline__ void trace_refill(const BvhDev &b, const RaySetDev &r
         if (!has) continue;
         // one visit of trace_ray_wide's loop
         const float4 *w = b.wide + 8 * (int64_t)node;
-        const float4 lx = __ldg(w), hx = __ldg(w + 1), ly = __ldg(w + 2), hy = __ldg(w + 3), lz = __ldg(w + 4),
-                     hz = __ldg(w + 5), rf = __ldg(w + 6);
+        const float4x2 nx = ldg_pair(w), ny = ldg_pair(w + 2), nz = ldg_pair(w + 4), nr = ldg_pair(w + 6);
+        const float4 lx = nx.a, hx = nx.b, ly = ny.a, hy = ny.b, lz = nz.a, hz = nz.b, rf = nr.a;
         const uint32_t r[4] = {__float_as_uint(rf.x), __float_as_uint(rf.y), __float_as_uint(rf.z),
                                __float_as_uint(rf.w)};
         float tn[4];
@@ -928,8 +924,8 @@ __device__ __forceinline__ float trace_warp_ray(const BvhDev &b, float3 o, float
         uint32_t r[4] = {0u, 0u, 0u, 0u}, pm = 0u;
         if (active) {
             const float4 *w = b.wide + 8 * (int64_t)node;
-            const float4 lx = __ldg(w), hx = __ldg(w + 1), ly = __ldg(w + 2), hy = __ldg(w + 3),
-                         lz = __ldg(w + 4), hz = __ldg(w + 5), rf = __ldg(w + 6);
+            const float4x2 nx = ldg_pair(w), ny = ldg_pair(w + 2), nz = ldg_pair(w + 4), nr = ldg_pair(w + 6);
+        const float4 lx = nx.a, hx = nx.b, ly = ny.a, hy = ny.b, lz = nz.a, hz = nz.b, rf = nr.a;
             r[0] = __float_as_uint(rf.x);
             r[1] = __float_as_uint(rf.y);
             r[2] = __float_as_uint(rf.z);
