@@ -261,9 +261,11 @@ typedef enum {
     RT_KERNEL_RAY_REFILL = 5, /* as RAY_WIDE, idle lanes refilled with new rays
                               as theirs finish (full implicit sets; otherwise
                               RAY_WIDE)                                       */
-    RT_KERNEL_WARP_RAY = 6   /* one warp per ray over the 4-wide tree: the lanes
-                              expand up to 32 of the ray's nodes at once (few
-                              or latency-bound rays; no hit log)             */
+    RT_KERNEL_WARP_RAY = 6   /* a group of lanes per ray over the 4-wide tree: they
+                              expand as many of the ray's nodes at once (full
+                              sets and up to 8192 rays: 32 lanes; lists up to
+                              2^16: 16, up to 2^18: 8, beyond: 4; scattered
+                              rays; no hit log)                              */
 } rt_kernel;
 
 typedef struct {
@@ -528,9 +530,9 @@ rt_status rt_surrogate_train(rt_surrogate *s, const rt_bvh *bvh, const rt_rayspe
 /* Visibility of an implicit ray set over `bvh` (DIRS or ENV, optionally a
  * ray_ids subset) from the surrogate: T_out[i] = p / (p + w (1 - p)), the
  * network's estimate (= p for w = 1).  If band > 0, rays with
- * |p - 0.5| < band are traced on `bvh` instead (the fallback: one warp per
- * ray, RT_KERNEL_WARP_RAY) and T_out holds the traced value, bit-equal to
- * rt_trace_visibility with that kernel; n_fallback (device int64[1], may be
+ * |p - 0.5| < band are traced on `bvh` instead (the fallback:
+ * RT_KERNEL_WARP_RAY) and T_out holds the traced value, bit-equal to
+ * rt_trace_visibility of the same ray set with that kernel; n_fallback (device int64[1], may be
  * NULL) receives their
  * number.  The scene bounds used to normalise origins are the surrogate's.
  * Errors: RT_ERR_INVALID_ARG. */

@@ -36,35 +36,6 @@ __global__ void __launch_bounds__(128, RT_TRACE_MIN_BLOCKS) k_trace(BvhDev b, Ra
         flush_counts<COUNT>(aux, wc, rays_done);
         return;
     }
-    if (STRAT == 6) {  // one warp per ray: an item is one ray
-        __shared__ uint32_t wstk_all[STRAT == 6 ? 4 * kWarpStack : 1];
-        uint32_t *wstk = wstk_all + (threadIdx.x >> 5) * kWarpStack;
-        for (;;) {
-            unsigned long long item = 0;
-            if (lane == 0) item = atomicAdd(work, 1ull);
-            item = __shfl_sync(FULL, item, 0);
-            int64_t n_out = job.mode == MODE_FULL ? job.n_items * 32 : job.n_out;  // slots
-            if (job.dyn_count) {
-                const int64_t c = (int64_t)*job.dyn_count;
-                n_out = c < n_out ? c : n_out;
-            }
-            if ((int64_t)item >= n_out) break;
-            float3 o, d;
-            int32_t src;
-            int64_t out_idx;
-            if (!ray_of(b, rs, job, (int64_t)item, o, d, src, out_idx, aux.status)) {
-                if (lane == 0 && out_idx >= 0) T_out[out_idx] = __int_as_float(0x7fc00000);
-                continue;
-            }
-            const float T = trace_warp_ray<COUNT>(b, o, d, src, wstk, wc, aux.status);
-            if (lane == 0) {
-                T_out[out_idx] = T;
-                rays_done++;
-            }
-        }
-        flush_counts<COUNT>(aux, wc, rays_done);
-        return;
-    }
     for (;;) {
         unsigned long long item = 0;
         if (lane == 0) item = atomicAdd(work, 1ull);
@@ -78,6 +49,19 @@ __global__ void __launch_bounds__(128, RT_TRACE_MIN_BLOCKS) k_trace(BvhDev b, Ra
         }
         trace_item<STRAT, COUNT>(b, rs, job, T_out, aux, (int64_t)item, n_out, wc, rays_done, stk);
     }
+    flush_counts<COUNT>(aux, wc, rays_done);
+}
+
+// Strategy 6: a group of lanes per ray.
+template <int LANES, bool COUNT>
+__global__ void __launch_bounds__(128, RT_TRACE_MIN_BLOCKS) k_trace_lanes(BvhDev b, RaySetDev rs, TraceJob job,
+                                                                          float *T_out, TraceAux aux,
+                                                                          unsigned long long *work) {
+    __shared__ uint32_t stk[128 * kLaneStack];
+    WorkCounts wc = {0, 0, 0};
+    unsigned long long rays_done = 0;
+    trace_lane_group<LANES, COUNT>(b, rs, job, T_out, aux, work, stk + threadIdx.x / LANES * (LANES * kLaneStack), wc,
+                                   rays_done);
     flush_counts<COUNT>(aux, wc, rays_done);
 }
 
@@ -134,6 +118,30 @@ int persistent_blocks(const void *kernel, int threads) {
     return per_sm * rt_num_sms();
 }
 
+// Lanes per ray for a list of m rays (a fallback list: the most it can be).
+// 300k object scene, shadow rays in no order, us with 32 / 16 / 8 / 4
+// lanes: 2,000 rays 53 / 70 / 105 / 167; 20,000 147 / 141 / 168 / 231; 100,000
+// 555 / 439 / 416 / 439; 600,000 3,102 / 2,329 / 2,031 / 1,889; 1M rays of the
+// 2M scene 10,230 / 8,868 / 8,778 / 8,900.
+// A full set keeps 32, so that a ray of it and of a short id list get the same
+// T bit for bit.
+int lanes_for(bool full, int64_t m) { return full || m <= 8192 ? 32 : m <= 65536 ? 16 : m <= 262144 ? 8 : 4; }
+
+template <bool COUNT>
+void launch_lanes(int lanes, const BvhDev &b, const RaySetDev &rs, const TraceJob &job, float *T_out,
+                  const TraceAux &aux, cudaStream_t st, unsigned long long *work) {
+#define RT_LANES(L)                                                                                      \
+    k_trace_lanes<L, COUNT><<<persistent_blocks((const void *)k_trace_lanes<L, COUNT>, 128), 128, 0, st>>>( \
+        b, rs, job, T_out, aux, work)
+    switch (lanes) {
+        case 32: RT_LANES(32); break;
+        case 16: RT_LANES(16); break;
+        case 8: RT_LANES(8); break;
+        default: RT_LANES(4);
+    }
+#undef RT_LANES
+}
+
 }  // namespace
 
 // Launch the single-scene kernel on an explicit job (used by the autotuner).
@@ -146,8 +154,7 @@ rt_status rt_trace_launch_job(const BvhDev &b, const RaySetDev &rs, const TraceJ
     if (cudaMemsetAsync(work, 0, sizeof(unsigned long long), st) != cudaSuccess) return RT_ERR_CUDA;
     const int threads = 128;
     if (strat == 6 && b.wide) {
-        int grid = persistent_blocks((const void *)k_trace<6, false>, threads);
-        k_trace<6, false><<<grid, threads, 0, st>>>(b, rs, job, T_out, aux, work);
+        launch_lanes<false>(lanes_for(job.mode == MODE_FULL, job.n_out), b, rs, job, T_out, aux, st, work);
     } else if (strat == 5 && b.wide && job.mode == MODE_FULL) {
         int grid = persistent_blocks((const void *)k_trace<5, false>, threads);
         k_trace<5, false><<<grid, threads, 0, st>>>(b, rs, job, T_out, aux, work);
@@ -211,8 +218,6 @@ rt_status rt_trace_launch(const rt_bvh *bvh, const rt_rayspec *rays, float *T_ou
     int strat = o.kernel == RT_KERNEL_WARP_RAY ? 6 : o.kernel == RT_KERNEL_RAY_REFILL ? 5
               : o.kernel == RT_KERNEL_RAY_WIDE ? 4 : o.kernel == RT_KERNEL_WIDE ? 2
               : o.kernel == RT_KERNEL_PACKET ? 1 : 0;
-    // one warp per ray needs the 4-wide tree and keeps no hit log
-    if (strat == 6 && (bvh->n_wide == 0 || o.hit_ids)) strat = bvh->n_wide ? 4 : 0;
     // AUTO:
     // - a direction set: shaft packets where the groups are large enough
     //   (rt_shaft_pays), else one thread per ray, farthest child first.  With
@@ -222,21 +227,22 @@ rt_status rt_trace_launch(const rt_bvh *bvh, const rt_rayspec *rays, float *T_ou
     //   packets win);
     // - env-map and hemisphere sets (directions differ across a tile): the
     //   per-ray walk with lane refill;
-    // - explicit rays and id lists (scattered rays): one warp per ray up to
-    //   2^22 rays, its lanes sharing one ray's nodes (2M object scene,
-    //   scattered ids: 2^16 rays 3.7x and 2^20 rays 1.25x the per-ray
-    //   walks), and one thread per ray over the 4-wide tree for longer lists
-    //   (2^24 rays: 6 % faster than one warp per ray).
+    // - explicit rays and id lists (scattered rays): a group of lanes per ray
+    //   up to 2^22 rays (lanes_for; one thread per ray takes 560 us for 2,000
+    //   rays of the 300k scene, 2.4 ms for 600,000), and one thread per ray
+    //   over the 4-wide tree for longer lists, which are sorted.
     if (o.kernel == RT_KERNEL_AUTO && job.mode == MODE_FULL)
         strat = rays->kind != RT_RAYS_DIRS ? 5
                 : o.counters || o.hit_ids  ? (bvh->n <= (int64_t(1) << 19) ? 4 : 2)
                 : rt_shaft_pays(bvh)       ? 2
                                            : 4;
     if (o.kernel == RT_KERNEL_AUTO && job.mode != MODE_FULL) strat = count <= (int64_t(1) << 22) ? 6 : 4;
+    // lanes per ray keep no hit log
+    if (strat == 6 && o.hit_ids) strat = 4;
     // lane refill needs the 4-wide tree and a full implicit set, and keeps no hit log
     if (strat == 5 && (bvh->n_wide == 0 || job.mode != MODE_FULL || o.hit_ids)) strat = 4;
     if (strat == 2 && bvh->n_wide == 0) strat = 1;
-    if (strat == 4 && bvh->n_wide == 0) strat = 0;
+    if ((strat == 4 || strat == 6) && bvh->n_wide == 0) strat = 0;  // fewer than two Gaussians
     // a shared direction: shaft packets, which count no single ray's tests and
     // keep no hit log (then the plain packet walk)
     if (strat == 2 && job.mode == MODE_FULL && rays->kind == RT_RAYS_DIRS && !o.counters && !o.hit_ids) strat = 3;
@@ -297,7 +303,11 @@ rt_status rt_trace_launch(const rt_bvh *bvh, const rt_rayspec *rays, float *T_ou
         int grid = persistent_blocks((const void *)k_trace<S, C>, threads);                 \
         k_trace<S, C><<<grid, threads, 0, st>>>(b, rs, job, T_out, aux, work);              \
     } while (0)
-        if (strat == 6) { if (count) RT_LAUNCH(6, true); else RT_LAUNCH(6, false); }
+        if (strat == 6) {
+            const int lanes = lanes_for(job.mode == MODE_FULL, job.n_out);
+            if (count) launch_lanes<true>(lanes, b, rs, job, T_out, aux, st, work);
+            else launch_lanes<false>(lanes, b, rs, job, T_out, aux, st, work);
+        }
         else if (strat == 5) { if (count) RT_LAUNCH(5, true); else RT_LAUNCH(5, false); }
         else if (strat == 4) { if (count) RT_LAUNCH(4, true); else RT_LAUNCH(4, false); }
         else if (strat == 3) {
@@ -347,12 +357,10 @@ rt_status rt_trace_launch_list(const rt_bvh *bvh, const rt_rayspec *rays, const 
     cudaStream_t st = (cudaStream_t)stream;
     if (cudaMemsetAsync(work, 0, sizeof(unsigned long long), st) != cudaSuccess) return RT_ERR_CUDA;
     const int threads = 128;
-    // the listed rays are few and scattered: one warp per ray over the 4-wide
-    // tree (its lanes expand the ray's nodes in parallel), which cuts the
-    // latency of the longest traversal
+    // the listed rays are few and scattered: a group of lanes per ray over the
+    // 4-wide tree, which cuts the latency of the longest traversal
     if (bvh->n_wide > 0) {
-        int grid = persistent_blocks((const void *)k_trace<6, false>, threads);
-        k_trace<6, false><<<grid, threads, 0, st>>>(bvh_dev(bvh), rs, job, T_out, aux, work);
+        launch_lanes<false>(lanes_for(!rays->ray_ids, max_count), bvh_dev(bvh), rs, job, T_out, aux, st, work);
     } else {
         int grid = persistent_blocks((const void *)k_trace<0, false>, threads);
         k_trace<0, false><<<grid, threads, 0, st>>>(bvh_dev(bvh), rs, job, T_out, aux, work);

@@ -872,66 +872,76 @@ __device__ __forceinline__ void trace_refill(const BvhDev &b, const RaySetDev &r
     }
 }
 
-// Strategy 6: one warp per ray over the 4-wide tree, for few or latency-bound
-// rays (fallback lists, small sets).  The lanes take up to 32 entries off the
-// top of a shared stack, visit those nodes in parallel, multiply the factors
-// of their leaf hits into lane-local partial products and push the hit
-// internal children (warp prefix sum); T is the product of the partials,
-// formed by a warp butterfly after every step for the early exit.  A step
-// takes k = min(32, size, (cap - size)/3) entries, so the stack never exceeds
-// cap (RT_ERR_STACK_OVERFLOW if no entry can be taken).  Same accepted set as
-// the per-ray traversals; the product is formed in another order.
-constexpr int kWarpStack = 2048;
-
-__device__ __forceinline__ float warp_product(float v) {
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v *= __shfl_xor_sync(0xffffffffu, v, off);
-    return v;
-}
-
-template <bool COUNT>
-__device__ __forceinline__ float trace_warp_ray(const BvhDev &b, float3 o, float3 d, int32_t src, uint32_t *wstk,
-                                                WorkCounts &wc, int *status) {
+// Strategy 6: LANES (4, 8, 16 or 32) lanes per ray over the 4-wide tree, for
+// scattered rays (fallback lists, explicit rays).  The lanes take up to that many
+// entries off the top of the ray's stack in shared memory, visit those nodes
+// in parallel, multiply the factors of their leaf hits into lane-local partial
+// products and push the hit internal children; T is the product of the
+// partials, formed by a butterfly after every step for the early exit.  A
+// step takes as many entries as keep 3 places free per level of the tree, and
+// one where that is not possible: one at a time the walk is depth first and
+// grows the stack by 3 a level at most (RT_ERR_STACK_OVERFLOW for a tree too
+// deep even for that).  Same accepted
+// set as the per-ray traversals; the product is formed in another order.  A
+// group of lanes fetches its next ray as soon as it is done.  `work` counts
+// rays (slots of a full implicit set).  A ray's walk has few nodes at a time:
+// with all 32 lanes on it most idle, with few lanes a single ray takes longer
+// (lanes_for, rt_trace.cu).
+constexpr int kLaneStack = 64;  // entries per lane: >= 3 x 64 levels for 4 lanes
+template <int LANES, bool COUNT>
+__device__ __forceinline__ void trace_lane_group(const BvhDev &b, const RaySetDev &rs, const TraceJob &job,
+                                                 float *T_out, const TraceAux &aux, unsigned long long *work,
+                                                 uint32_t *stk, WorkCounts &wc, unsigned long long &rays_done) {
     const unsigned FULL = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
-    float Tl = 1.0f;
-    if (b.n <= 0) return 1.0f;
-    if (b.n == 1) {
-        if (lane == 0 && src != 0) {
-            if (COUNT) wc.gauss++;
-            if (gauss_hit(b, 0, o, d, Tl) && COUNT) wc.hits++;
-        }
-        const float T = __shfl_sync(FULL, Tl, 0);
-        return T < b.t_min ? 0.0f : T;
+    const int lane = threadIdx.x & 31, sub = lane & (LANES - 1);
+    const unsigned group = (LANES == 32 ? FULL : ((1u << LANES) - 1u) << (lane - sub));
+    int64_t n_out = job.mode == MODE_FULL ? job.n_items * 32 : job.n_out;  // slots
+    if (job.dyn_count) {
+        const int64_t c = (int64_t)*job.dyn_count;
+        n_out = c < n_out ? c : n_out;
     }
-    const float3 inv = safe_inv(d);
-    const float3 oi = make_float3(o.x * inv.x, o.y * inv.y, o.z * inv.z);
-    if (lane == 0) wstk[0] = 0u;
-    int size = 1;
-    __syncwarp();
+    const int room = kLaneStack * LANES - 4 - 3 * b.levels;
+    bool has = false, more = true;
+    float3 o = make_float3(0.f, 0.f, 0.f), d = make_float3(0.f, 0.f, 1.f), inv = d, oi = o;
+    int32_t src = -1;
+    int64_t out_idx = 0;
+    float Tl = 1.0f;
+    int size = 0;
     for (;;) {
-        int k = min(32, min(size, (kWarpStack - size) / 3));
-        if (k <= 0) {
-            if (size > 0) rt_set_error(status, RT_ERR_STACK_OVERFLOW);
-            break;
+        if (!has && more) {
+            unsigned long long item = 0;
+            if (sub == 0) item = atomicAdd(work, 1ull);
+            item = __shfl_sync(group, item, 0, LANES);
+            if ((int64_t)item >= n_out) {
+                more = false;
+            } else if (!ray_of(b, rs, job, (int64_t)item, o, d, src, out_idx, aux.status)) {
+                if (sub == 0 && out_idx >= 0) T_out[out_idx] = __int_as_float(0x7fc00000);
+            } else {
+                has = true;
+                inv = safe_inv(d);
+                oi = make_float3(o.x * inv.x, o.y * inv.y, o.z * inv.z);
+                Tl = 1.0f;
+                size = 1;
+                if (sub == 0) stk[0] = 0u;
+            }
         }
-        const bool active = lane < k;
-        const uint32_t node = active ? wstk[size - 1 - lane] : 0u;
+        if (!__any_sync(FULL, has || more)) break;
+        __syncwarp();
+        // one step: entries off the top, their nodes' children
+        const int k = has ? min(min(LANES, size), max(1, (room - size) / 3)) : 0;
+        const uint32_t node = sub < k ? stk[size - 1 - sub] : 0u;
         size -= k;
         __syncwarp();
-        // internal children to push: a mask over c (a register array indexed by
-        // a running count would live in local memory)
-        uint32_t r[4] = {0u, 0u, 0u, 0u}, pm = 0u;
-        if (active) {
+        uint32_t r[4] = {0u, 0u, 0u, 0u}, pm = 0u;  // internal children to push: a mask over c
+        if (sub < k) {
             const float4 *w = b.wide + 8 * (int64_t)node;
             const float4x2 nx = ldg_pair(w), ny = ldg_pair(w + 2), nz = ldg_pair(w + 4), nr = ldg_pair(w + 6);
-        const float4 lx = nx.a, hx = nx.b, ly = ny.a, hy = ny.b, lz = nz.a, hz = nz.b, rf = nr.a;
-            r[0] = __float_as_uint(rf.x);
-            r[1] = __float_as_uint(rf.y);
-            r[2] = __float_as_uint(rf.z);
-            r[3] = __float_as_uint(rf.w);
+            r[0] = __float_as_uint(nr.a.x);
+            r[1] = __float_as_uint(nr.a.y);
+            r[2] = __float_as_uint(nr.a.z);
+            r[3] = __float_as_uint(nr.a.w);
             bool h[4];
-            slab4(lx, hx, ly, hy, lz, hz, oi, inv, h);
+            slab4(nx.a, nx.b, ny.a, ny.b, nz.a, nz.b, oi, inv, h);
             if (COUNT) wc.box += (r[0] != RT_EMPTY) + (r[1] != RT_EMPTY) + (r[2] != RT_EMPTY) + (r[3] != RT_EMPTY);
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
@@ -947,23 +957,33 @@ __device__ __forceinline__ float trace_warp_ray(const BvhDev &b, float3 o, float
                 }
             }
         }
-        // warp prefix sum of the pushes, then write them above the stack top
+        __syncwarp();
+        // prefix sum of the pushes over the group, then write them above the top
         const int n_push = __popc(pm);
         int pre = n_push;
+        float T = Tl;
 #pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const int v = __shfl_up_sync(FULL, pre, off);
-            if (lane >= off) pre += v;
+        for (int off = 1; off < LANES; off <<= 1) {
+            const int v = __shfl_up_sync(FULL, pre, off, LANES);
+            if (sub >= off) pre += v;
+            T *= __shfl_xor_sync(FULL, T, off);
         }
-        const int total = __shfl_sync(FULL, pre, 31);
+        const int total = __shfl_sync(FULL, pre, LANES - 1, LANES);
         int at = size + pre - n_push;
 #pragma unroll
         for (int c = 0; c < 4; ++c)
-            if ((pm >> c) & 1u) wstk[at++] = r[c];
+            if ((pm >> c) & 1u) stk[at++] = r[c];
         size += total;
+        const bool full = size > kLaneStack * LANES - 4;  // no place for another node's children
+        if (has && (full || T < b.t_min || size == 0)) {
+            if (full) rt_set_error(aux.status, RT_ERR_STACK_OVERFLOW);
+            if (sub == 0) {
+                T_out[out_idx] = T < b.t_min ? 0.0f : T;
+                rays_done++;
+            }
+            has = false;
+            size = 0;
+        }
         __syncwarp();
-        if (warp_product(Tl) < b.t_min || size == 0) break;
     }
-    const float T = warp_product(Tl);
-    return T < b.t_min ? 0.0f : T;
 }
