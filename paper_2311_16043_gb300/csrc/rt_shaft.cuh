@@ -341,13 +341,11 @@ __device__ __forceinline__ void shaft_group(const BvhDev &b, float eps, float3 d
         __syncwarp();
         ShaftCand g;
         {
-            // lanes past the batch repeat its first Gaussian and never pass
+            // lanes past the batch repeat its first Gaussian (their votes are dropped)
             const int ia = lane < m ? lane : 0, ib = lane + 32 < m ? lane + 32 : 0;
             const float4 ra[4] = {rec(ia, 0), rec(ia, 1), rec(ia, 2), rec(ia, 3)};
             const float4 rb[4] = {rec(ib, 0), rec(ib, 1), rec(ib, 2), rec(ib, 3)};
             shaft_cand(sm, ra, rb, g);
-            if (lane >= m) g.thr.x = -inf;
-            if (lane + 32 >= m) g.thr.y = -inf;
         }
 #pragma unroll 2
         for (int t = 0; t < live; ++t) {
@@ -366,6 +364,9 @@ __device__ __forceinline__ void shaft_group(const BvhDev &b, float eps, float3 d
             uint32_t ray = 0u;
             if (s0 + lane < live) {
                 mk = sm.mask[s0 + lane];
+                // a NaN test passes: not in the lanes past the batch
+                mk.x &= m >= 32 ? FULL : (1u << m) - 1u;
+                mk.y &= m >= 64 ? FULL : m > 32 ? (1u << (m - 32)) - 1u : 0u;
                 ray = sm.live[s0 + lane];
             }
             while (__any_sync(FULL, (mk.x | mk.y) != 0u)) {

@@ -103,3 +103,14 @@ def test_order_block_and_refit():
     a = rt.rt_trace_visibility_dirs(bvh, _dev(dirs), opts=rt.trace_opts(kernel=1)).cpu().numpy().astype(np.float64)
     b = rt.rt_trace_visibility_dirs(bvh, _dev(dirs), opts=rt.trace_opts(kernel=3)).cpu().numpy().astype(np.float64)
     assert ((np.abs(b - a) <= RTOL * a) | ((np.minimum(a, b) == 0) & (np.maximum(a, b) <= 1.001e-4))).all()
+
+
+@pytest.mark.parametrize("n", [40, 90, 700])
+def test_overflowing_inverse_scales(n):
+    """Inverse scales whose squares overflow make every plane test of their
+    Gaussian NaN: it is a candidate of all rays, accepted by none, and the lanes
+    past a batch that starts with it add nothing."""
+    sc = _cut(scenes.uniform_scene(700, 8), n)
+    sc["scale"] = sc["scale"].copy()
+    sc["scale"][::3] = 1e-20
+    _check(sc, scenes.fibonacci_sphere(11))
