@@ -430,8 +430,9 @@ rt_status rt_trace_ao(const rt_bvh *bvh, const rt_rayspec *rays, const rt_trace_
  * not NULL, writes d_ray_o[R*3].  T[R] are the traced values.  With
  * hit_ids/hit_count from the forward (capacity hit_cap) the accepted hits are
  * replayed; rays whose count exceeds hit_cap, or all rays if hit_ids is NULL,
- * are re-traversed.  The mean, scale, quat, opacity arrays must be the ones
- * the BVH was built from.  Accumulation uses float32 atomics (summation order
+ * are re-traversed (a full direction set in shaft packets where these pay,
+ * which is faster than a replay).  The mean, scale, quat, opacity arrays must
+ * be the ones the BVH was built from.  Accumulation uses float32 atomics (summation order
  * is not deterministic) unless the tree's params.deterministic is set: then
  * 64-bit fixed-point sums (device scratch of 88 bytes per Gaussian) are added
  * to the outputs once, bit-reproducibly. */
@@ -442,6 +443,10 @@ rt_status rt_trace_visibility_backward(const rt_bvh *bvh, const rt_rayspec *rays
                                        int32_t hit_cap, float *d_mean, float *d_scale,
                                        float *d_quat, float *d_opacity, float *d_ray_o,
                                        rt_stream_t stream);
+
+/* 1 if the adjoint of this ray set is faster with the forward's hit log, 0 if
+ * it takes shaft packets (no log is needed then); 0 for NULL arguments. */
+int32_t rt_backward_wants_log(const rt_bvh *bvh, const rt_rayspec *rays);
 
 
 /* ------------------------------------------------------------------------ */

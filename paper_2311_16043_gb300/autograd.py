@@ -3,9 +3,9 @@ every Gaussian in a direction set, differentiable with respect to mean,
 scale, quaternion and opacity through the hand-written adjoint
 (``rt_trace_visibility_backward``).
 
-The forward builds the LBVH, traces, and keeps a per-ray hit log when it fits
-the memory budget; otherwise (or for rays that overflow the log) the backward
-re-traverses.  Log-scale parameterisations compose in torch
+The forward builds the LBVH, traces, and keeps a per-ray hit log where the
+backward is faster with one and it fits the memory budget; otherwise (or for
+rays that overflow the log) the backward re-traverses.  Log-scale parameterisations compose in torch
 (``scale = log_scale.exp()``), which supplies the s * d/ds factor.
 """
 from __future__ import annotations
@@ -23,7 +23,7 @@ class Visibility(torch.autograd.Function):
         bvh = rt.rt_build_bvh(mean_c, scale_c, quat_c, opac_c, prm)
         rs = rt.rayspec(rt.RT_RAYS_DIRS, dirs=dirs_c)
         R = rt.rt_rayspec_count(bvh, rs)
-        cap = hit_cap if R * hit_cap * 4 <= log_budget_bytes else 0
+        cap = hit_cap if R * hit_cap * 4 <= log_budget_bytes and rt.rt_backward_wants_log(bvh, rs) else 0
         hit_ids = torch.empty((R, cap), dtype=torch.int32, device=mean.device) if cap else None
         hit_count = torch.empty(R, dtype=torch.int32, device=mean.device) if cap else None
         opts = rt.trace_opts(hit_ids=hit_ids, hit_count=hit_count)

@@ -235,7 +235,7 @@ __global__ void __launch_bounds__(128, RT_BATCH_MIN_BLOCKS) k_trace_batch(const 
 __global__ void __launch_bounds__(128, RT_SHAFT_MIN_BLOCKS) k_shaft_batch(const BatchJobDev *__restrict__ jobs, int n_jobs,
                                                                           int64_t total_items, int *status,
                                                                           unsigned long long *work) {
-    __shared__ ShaftSmem sm[4];
+    __shared__ ShaftSmem<false> sm[4];
     for (;;) {
         unsigned long long item = 0;
         if ((threadIdx.x & 31) == 0) item = atomicAdd(work, 1ull);

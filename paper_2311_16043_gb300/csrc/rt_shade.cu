@@ -353,8 +353,8 @@ __global__ void __launch_bounds__(128, 8) k_trace_reduce(BvhDev b, RaySetDev rs,
 __global__ void __launch_bounds__(128, RT_SHAFT_MIN_BLOCKS) k_shaft_ao(BvhDev b, RaySetDev rs, int64_t n_groups,
                                                                        float *__restrict__ ao, int *status,
                                                                        unsigned long long *work) {
-    __shared__ ShaftSmem sm_all[4];
-    ShaftSmem &sm = sm_all[threadIdx.x >> 5];
+    __shared__ ShaftSmem<false> sm_all[4];
+    ShaftSmem<false> &sm = sm_all[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
     for (;;) {
         unsigned long long item = 0;
@@ -364,7 +364,7 @@ __global__ void __launch_bounds__(128, RT_SHAFT_MIN_BLOCKS) k_shaft_ao(BvhDev b,
         const int2 gr = __ldg(b.groups + item);
         float acc[2] = {0.0f, 0.0f};
         for (int32_t k = 0; k < rs.K; ++k) {
-            shaft_group(b, rs.eps, make_float3(__ldg(rs.dirs + 3 * k), __ldg(rs.dirs + 3 * k + 1), __ldg(rs.dirs + 3 * k + 2)),
+            shaft_group<false>(b, rs.eps, make_float3(__ldg(rs.dirs + 3 * k), __ldg(rs.dirs + 3 * k + 1), __ldg(rs.dirs + 3 * k + 2)),
                         gr.x, gr.y, status, sm);
 #pragma unroll
             for (int r = 0; r < 2; ++r)

@@ -43,25 +43,32 @@
 //   - 6 resident blocks (80 registers) instead of 5 (96): 6 %.
 #pragma once
 
+#include <type_traits>
+
 #include "rt_trace_core.cuh"
 
 constexpr int kShaftRays = 64;      // rays of a group at most
 constexpr int kShaftCands = 64;     // Gaussians of a batch
 constexpr int kShaftNodes = 16;     // nodes of a step
 constexpr int kShaftStack = 320;    // nodes; a walk of single nodes adds 3 per level at most (193 for 64 levels)
-constexpr int kShaftPairs = 256;
+template <bool GRAD>
+constexpr int kShaftPairs = GRAD ? 160 : 256;
 
+// The adjoint (GRAD) keeps a record per pair, (dL/dm^2, u) with u = S^-1 R^T e.
+template <bool GRAD>
 struct __align__(16) ShaftSmem {
     float4 stage[4 * kShaftCands];            // the batch's records, or a step's nodes
-    float4 ro[kShaftRays];                    // by ray: origin, T
+    float4 ro[kShaftRays];                    // by ray: origin, T (GRAD: by slot: origin, dL/dT T)
+    typename std::conditional<GRAD, float4, uint32_t>::type pair[kShaftPairs<GRAD>];  // ray << 6 | Gaussian,
+                                              //   then the pair's factor (GRAD: record)
     float2 xy[kShaftRays];                    // by slot of a live ray: its place across d
     float z[kShaftRays];                      //   and along d
     uint2 mask[kShaftRays];                   // by slot: Gaussians of the batch to evaluate
     float4 fr[5];                             // the shaft's frame (see shaft_cand)
     uint32_t stack[kShaftStack];
     uint32_t leaf[kShaftCands + 4 * kShaftNodes];  // fewer than a batch left over + one step's
-    uint32_t pair[kShaftPairs];               // ray << 6 | Gaussian, then the pair's factor
     uint8_t live[kShaftRays];                 // by slot: ray
+    uint8_t from[GRAD ? kShaftRays : 1];      // GRAD: by slot: its first pair
 };
 
 __device__ __forceinline__ void cp_async16(void *dst, const void *src) {
@@ -128,7 +135,8 @@ struct ShaftCand {
 // carries |s| ulps, and gauss_eval's own error is within the same terms.
 // frame: fr[0] = (c, |d|^2), fr[1] = (d, |d|), fr[2] = (d / |d|^2, group
 // radius), fr[3] = (e1, k_sigma^2 log2(e)/2), fr[4] = (e2, log2(alpha_min)).
-__device__ __forceinline__ void shaft_cand(const ShaftSmem &sm, const float4 (&a)[4], const float4 (&b)[4],
+template <bool GRAD>
+__device__ __forceinline__ void shaft_cand(const ShaftSmem<GRAD> &sm, const float4 (&a)[4], const float4 (&b)[4],
                                            ShaftCand &g) {
     const float4 F0 = sm.fr[0], F1 = sm.fr[1], F2 = sm.fr[2], F3 = sm.fr[3], F4 = sm.fr[4];
     const f2x3 w0 = pack3(a[1], b[1]), w1 = pack3(a[2], b[2]), w2 = pack3(a[3], b[3]);
@@ -177,65 +185,95 @@ __device__ __forceinline__ void shaft_cand(const ShaftSmem &sm, const float4 (&a
     lim(nn.y, px.y, py.y, s.y, iu.y, b[0].w, hb.y, g.thr.y, g.h.y);
 }
 
-// gauss_eval of two pairs at once, each operation rounded as there: the
-// factor 1 - alpha of an accepted pair, else 1.
-__device__ __forceinline__ void gauss_factor2(const BvhDev &b, const float4 (&ga)[4], const float4 (&gb)[4], float4 oa,
-                                              float4 ob, float3 d, float &fa, float &fb) {
-    auto dot = [](f2x3 x, f2x3 y) { return __ffma2_rn(x.x, y.x, __ffma2_rn(x.y, y.y, __fmul2_rn(x.z, y.z))); };
-    const f2x3 mu = pack3(ga[0], gb[0]), w0 = pack3(ga[1], gb[1]), w1 = pack3(ga[2], gb[2]), w2 = pack3(ga[3], gb[3]);
-    const f2x3 o = pack3(oa, ob);
-    f2x3 hi, lo, D;
-    two_diff2(o.x, mu.x, hi.x, lo.x);
-    two_diff2(o.y, mu.y, hi.y, lo.y);
-    two_diff2(o.z, mu.z, hi.z, lo.z);
-    D.x = dup(d.x);
-    D.y = dup(d.y);
-    D.z = dup(d.z);
-    f2x3 ud, uo, u, e;
-    ud.x = dot(w0, D);
-    ud.y = dot(w1, D);
-    ud.z = dot(w2, D);
-    uo.x = dot(w0, hi);
-    uo.y = dot(w1, hi);
-    uo.z = dot(w2, hi);
-    const float2 num = dot(uo, ud), den = dot(ud, ud);
-    const float2 t = make_float2(__fdividef(-num.x, den.x), __fdividef(-num.y, den.y));
-    e.x = __fadd2_rn(__ffma2_rn(t, D.x, hi.x), lo.x);
-    e.y = __fadd2_rn(__ffma2_rn(t, D.y, hi.y), lo.y);
-    e.z = __fadd2_rn(__ffma2_rn(t, D.z, hi.z), lo.z);
-    u.x = dot(w0, e);
-    u.y = dot(w1, e);
-    u.z = dot(w2, e);
-    const float2 m2 = dot(u, u);
-    const float aa = ga[0].w * __expf(-0.5f * m2.x), ab = gb[0].w * __expf(-0.5f * m2.y);
-    fa = t.x > 0.0f && m2.x <= b.k2 && aa >= b.alpha_min ? 1.0f - aa : 1.0f;
-    fb = t.y > 0.0f && m2.y <= b.k2 && ab >= b.alpha_min ? 1.0f - ab : 1.0f;
-}
+// gauss_eval of two pairs at once, each operation rounded as there.
+struct PairEval {
+    f2x3 w0, w1, w2, hi, lo, D;
+    float2 num, den, alpha;  // t* = -num / den
+    bool acc[2];
+    __device__ __forceinline__ float2 dot(f2x3 x, f2x3 y) const {
+        return __ffma2_rn(x.x, y.x, __ffma2_rn(x.y, y.y, __fmul2_rn(x.z, y.z)));
+    }
+    __device__ __forceinline__ f2x3 peak(float2 t) const {  // x(t) - mu
+        f2x3 e;
+        e.x = __fadd2_rn(__ffma2_rn(t, D.x, hi.x), lo.x);
+        e.y = __fadd2_rn(__ffma2_rn(t, D.y, hi.y), lo.y);
+        e.z = __fadd2_rn(__ffma2_rn(t, D.z, hi.z), lo.z);
+        return e;
+    }
+    __device__ __forceinline__ f2x3 whiten(f2x3 e) const {
+        f2x3 u;
+        u.x = dot(w0, e);
+        u.y = dot(w1, e);
+        u.z = dot(w2, e);
+        return u;
+    }
+    __device__ __forceinline__ PairEval(const BvhDev &b, const float4 (&ga)[4], const float4 (&gb)[4], float4 oa,
+                                        float4 ob, float3 d) {
+        const f2x3 mu = pack3(ga[0], gb[0]), o = pack3(oa, ob);
+        w0 = pack3(ga[1], gb[1]);
+        w1 = pack3(ga[2], gb[2]);
+        w2 = pack3(ga[3], gb[3]);
+        two_diff2(o.x, mu.x, hi.x, lo.x);
+        two_diff2(o.y, mu.y, hi.y, lo.y);
+        two_diff2(o.z, mu.z, hi.z, lo.z);
+        D.x = dup(d.x);
+        D.y = dup(d.y);
+        D.z = dup(d.z);
+        const f2x3 ud = whiten(D), uo = whiten(hi);
+        num = dot(uo, ud);
+        den = dot(ud, ud);
+        const float2 t = make_float2(__fdividef(-num.x, den.x), __fdividef(-num.y, den.y));
+        const f2x3 u = whiten(peak(t));
+        const float2 m2 = dot(u, u);
+        alpha = make_float2(ga[0].w * __expf(-0.5f * m2.x), gb[0].w * __expf(-0.5f * m2.y));
+        acc[0] = t.x > 0.0f && m2.x <= b.k2 && alpha.x >= b.alpha_min;
+        acc[1] = t.y > 0.0f && m2.y <= b.k2 && alpha.y >= b.alpha_min;
+    }
+};
 
 // T of the `count` (1..64) rays of sorted positions first, first + 1, ...
 // along d (the same in every lane): in sm.ro[i].w, not snapped.
+// GRAD: `gr` has the rays' dL/dT and T and takes their hits' gradients (rays
+// without a gradient never join the group; none leaves it).
+template <bool GRAD, class Grad = int>
 __device__ __forceinline__ void shaft_group(const BvhDev &b, float eps, float3 d, int64_t first, int count,
-                                            int *status, ShaftSmem &sm) {
+                                            int *status, ShaftSmem<GRAD> &sm, Grad *gr = nullptr) {
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
     const float inf = __int_as_float(0x7f800000);
     const float3 inv = safe_inv(d);
+    int live = count;
+    if constexpr (GRAD) live = 0;
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
         const int i = lane + 32 * r;
-        if (i >= count) continue;
+        int slot = i;
+        float w = 1.0f;
+        bool in = i < count;
+        if constexpr (GRAD) {
+            w = gr->load(b, first, i, in);
+            const unsigned v = __ballot_sync(FULL, in);
+            slot = live + __popc(v & lt);
+            live += __popc(v);
+        }
+        if (!in) continue;
         const float4 mu = __ldg(b.gauss + 4 * (first + i));
-        sm.ro[i] = make_float4(__fadd_rn(mu.x, __fmul_rn(eps, d.x)), __fadd_rn(mu.y, __fmul_rn(eps, d.y)),
-                               __fadd_rn(mu.z, __fmul_rn(eps, d.z)), 1.0f);
-        sm.live[i] = (uint8_t)i;
+        sm.ro[slot] = make_float4(__fadd_rn(mu.x, __fmul_rn(eps, d.x)), __fadd_rn(mu.y, __fmul_rn(eps, d.y)),
+                                  __fadd_rn(mu.z, __fmul_rn(eps, d.z)), w);
+        sm.live[slot] = (uint8_t)i;
+    }
+    if constexpr (GRAD) {
+        gr->live = live;
+        if (live == 0) return;
+        __syncwarp();
     }
     // the box of n live rays' origins: centre c, half extents hh (outwards)
     float3 c, hh, cn, cf;
     auto bounds = [&](int n) {
         float3 lo = make_float3(inf, inf, inf), hi = make_float3(-inf, -inf, -inf);
         for (int s = lane; s < n; s += 32) {
-            const float4 o = sm.ro[sm.live[s]];
+            const float4 o = sm.ro[GRAD ? s : sm.live[s]];
             lo = make_float3(fminf(lo.x, o.x), fminf(lo.y, o.y), fminf(lo.z, o.z));
             hi = make_float3(fmaxf(hi.x, o.x), fmaxf(hi.y, o.y), fmaxf(hi.z, o.z));
         }
@@ -248,7 +286,7 @@ __device__ __forceinline__ void shaft_group(const BvhDev &b, float eps, float3 d
         cn = make_float3(fmaf(c.x, inv.x, w.x), fmaf(c.y, inv.y, w.y), fmaf(c.z, inv.z, w.z));
         cf = make_float3(fmaf(c.x, inv.x, -w.x), fmaf(c.y, inv.y, -w.y), fmaf(c.z, inv.z, -w.z));
     };
-    bounds(count);
+    bounds(live);
     {
         // plane frame (e1, e2) across d (Duff et al. 2017)
         const float dd = dot3(d, d), il = rsqrtf(dd);
@@ -259,7 +297,7 @@ __device__ __forceinline__ void shaft_group(const BvhDev &b, float eps, float3 d
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
             const int i = lane + 32 * r;
-            if (i >= count) continue;
+            if (i >= live) continue;
             const float4 o = sm.ro[i];
             const float3 v = make_float3(o.x - c.x, o.y - c.y, o.z - c.z);
             sm.xy[i] = make_float2(dot3(e1, v), dot3(e2, v));
@@ -284,7 +322,8 @@ __device__ __forceinline__ void shaft_group(const BvhDev &b, float eps, float3 d
     // step 2: 16-byte row r of staged record i lies at chunk r ^ ((i >> 1) & 3)
     auto rec = [&](int i, int r) { return sm.stage[4 * i + (r ^ ((i >> 1) & 3))]; };
     const int room = kShaftStack - 4 - 3 * b.levels;  // beyond it, nodes are walked one at a time
-    int live = count, bound = count, size = 1, nleaf = 0;
+    int bound = live, size = 1, nleaf = 0;
+    (void)bound;
     __syncwarp();
     for (;;) {
         while (nleaf < kShaftCands && size > 0) {
@@ -347,112 +386,126 @@ __device__ __forceinline__ void shaft_group(const BvhDev &b, float eps, float3 d
             const float4 rb[4] = {rec(ib, 0), rec(ib, 1), rec(ib, 2), rec(ib, 3)};
             shaft_cand(sm, ra, rb, g);
         }
+        uint2 ca = make_uint2(0u, 0u), cb = ca;  // GRAD: the slots that voted for this lane's Gaussians
 #pragma unroll 2
         for (int t = 0; t < live; ++t) {
             const float2 v = sm.xy[t], X = dup(v.x), Y = dup(v.y);
             const float2 v1 = __ffma2_rn(g.r11, X, __ffma2_rn(g.r12, Y, g.c1)), v2 = __ffma2_rn(g.r22, Y, g.c2);
             const float2 q = __ffma2_rn(v1, v1, __fmul2_rn(v2, v2));
             const float2 z = __ffma2_rn(g.qx, X, __ffma2_rn(g.qy, Y, dup(sm.z[t])));
-            const uint32_t ma = __ballot_sync(FULL, !(q.x >= g.thr.x) && !(z.x >= g.h.x)),
-                           mb = __ballot_sync(FULL, !(q.y >= g.thr.y) && !(z.y >= g.h.y));
+            const bool pa = !(q.x >= g.thr.x) && !(z.x >= g.h.x), pb = !(q.y >= g.thr.y) && !(z.y >= g.h.y);
+            const uint32_t ma = __ballot_sync(FULL, pa), mb = __ballot_sync(FULL, pb);
             if (lane == 0) sm.mask[t] = make_uint2(ma, mb);
+            if constexpr (GRAD) {
+                const uint32_t bit = 1u << (t & 31), b0 = t < 32 ? bit : 0u, b1 = t < 32 ? 0u : bit;
+                ca.x |= pa ? b0 : 0u;
+                ca.y |= pa ? b1 : 0u;
+                cb.x |= pb ? b0 : 0u;
+                cb.y |= pb ? b1 : 0u;
+            }
         }
         __syncwarp();
-        // step 3, the live rays of 32 slots at a time
-        for (int s0 = 0; s0 < live; s0 += 32) {
-            uint2 mk = make_uint2(0u, 0u);
-            uint32_t ray = 0u;
-            if (s0 + lane < live) {
-                mk = sm.mask[s0 + lane];
-                // a NaN test passes: not in the lanes past the batch
-                mk.x &= m >= 32 ? FULL : (1u << m) - 1u;
-                mk.y &= m >= 64 ? FULL : m > 32 ? (1u << (m - 32)) - 1u : 0u;
-                ray = sm.live[s0 + lane];
-            }
-            while (__any_sync(FULL, (mk.x | mk.y) != 0u)) {
-                int na = __popc(mk.x), nb = __popc(mk.y);
-                if (__reduce_add_sync(FULL, na + nb) > kShaftPairs) {  // a part of each ray's
-                    na = min(na, kShaftPairs / 64);
-                    nb = min(nb, kShaftPairs / 64);
-                }
-                int end = na + nb;
-#pragma unroll
-                for (int off = 1; off < 32; off <<= 1) {
-                    const int v = __shfl_up_sync(FULL, end, off);
-                    if (lane >= off) end += v;
-                }
-                const int total = __shfl_sync(FULL, end, 31), from = end - na - nb;
-                int at = from;
-                for (; na > 0; --na) {
-                    sm.pair[at++] = ray << 6 | (uint32_t)(__ffs(mk.x) - 1);
-                    mk.x &= mk.x - 1u;
-                }
-                for (; nb > 0; --nb) {
-                    sm.pair[at++] = ray << 6 | (uint32_t)(__ffs(mk.y) + 31);
-                    mk.y &= mk.y - 1u;
-                }
-                __syncwarp();
-                for (int i = lane; i < total; i += 64) {
-                    const uint32_t pa = sm.pair[i], pb = i + 32 < total ? sm.pair[i + 32] : pa;
-                    const int qa = pa & 63u, qb = pb & 63u;
-                    const float4 oa = sm.ro[pa >> 6], ob = sm.ro[pb >> 6];
-                    const float4 ra[4] = {rec(qa, 0), rec(qa, 1), rec(qa, 2), rec(qa, 3)};
-                    const float4 rb[4] = {rec(qb, 0), rec(qb, 1), rec(qb, 2), rec(qb, 3)};
-                    float fa, fb;
-                    gauss_factor2(b, ra, rb, oa, ob, d, fa, fb);
-                    if (sm.leaf[nleaf + qa] == (uint32_t)first + (pa >> 6)) fa = 1.0f;  // the ray's own Gaussian
-                    if (sm.leaf[nleaf + qb] == (uint32_t)first + (pb >> 6)) fb = 1.0f;
-                    sm.pair[i] = __float_as_uint(fa);
-                    if (i + 32 < total) sm.pair[i + 32] = __float_as_uint(fb);
-                }
-                __syncwarp();
+        if constexpr (GRAD) {
+            if (lane >= m) ca = make_uint2(0u, 0u);
+            if (lane + 32 >= m) cb = make_uint2(0u, 0u);
+            gr->batch(b, d, first, live, m, sm.leaf + nleaf, ca, cb, sm);
+        } else {
+            // step 3, the live rays of 32 slots at a time
+            for (int s0 = 0; s0 < live; s0 += 32) {
+                uint2 mk = make_uint2(0u, 0u);
+                uint32_t ray = 0u;
                 if (s0 + lane < live) {
-                    float T = sm.ro[ray].w;
-                    for (int i = from; i < end; ++i) T *= __uint_as_float(sm.pair[i]);
-                    sm.ro[ray].w = T;
-                    if (T < b.t_min) mk = make_uint2(0u, 0u);
+                    mk = sm.mask[s0 + lane];
+                    // a NaN test passes: not in the lanes past the batch
+                    mk.x &= m >= 32 ? FULL : (1u << m) - 1u;
+                    mk.y &= m >= 64 ? FULL : m > 32 ? (1u << (m - 32)) - 1u : 0u;
+                    ray = sm.live[s0 + lane];
                 }
-                __syncwarp();
+                while (__any_sync(FULL, (mk.x | mk.y) != 0u)) {
+                    int na = __popc(mk.x), nb = __popc(mk.y);
+                    if (__reduce_add_sync(FULL, na + nb) > kShaftPairs<GRAD>) {  // a part of each ray's
+                        na = min(na, kShaftPairs<GRAD> / 64);
+                        nb = min(nb, kShaftPairs<GRAD> / 64);
+                    }
+                    int end = na + nb;
+#pragma unroll
+                    for (int off = 1; off < 32; off <<= 1) {
+                        const int v = __shfl_up_sync(FULL, end, off);
+                        if (lane >= off) end += v;
+                    }
+                    const int total = __shfl_sync(FULL, end, 31), from = end - na - nb;
+                    int at = from;
+                    for (; na > 0; --na) {
+                        sm.pair[at++] = ray << 6 | (uint32_t)(__ffs(mk.x) - 1);
+                        mk.x &= mk.x - 1u;
+                    }
+                    for (; nb > 0; --nb) {
+                        sm.pair[at++] = ray << 6 | (uint32_t)(__ffs(mk.y) + 31);
+                        mk.y &= mk.y - 1u;
+                    }
+                    __syncwarp();
+                    for (int i = lane; i < total; i += 64) {
+                        const uint32_t pa = sm.pair[i], pb = i + 32 < total ? sm.pair[i + 32] : pa;
+                        const int qa = pa & 63u, qb = pb & 63u;
+                        const float4 oa = sm.ro[pa >> 6], ob = sm.ro[pb >> 6];
+                        const float4 ra[4] = {rec(qa, 0), rec(qa, 1), rec(qa, 2), rec(qa, 3)};
+                        const float4 rb[4] = {rec(qb, 0), rec(qb, 1), rec(qb, 2), rec(qb, 3)};
+                        const PairEval e(b, ra, rb, oa, ob, d);
+                        float fa = e.acc[0] ? 1.0f - e.alpha.x : 1.0f, fb = e.acc[1] ? 1.0f - e.alpha.y : 1.0f;
+                        if (sm.leaf[nleaf + qa] == (uint32_t)first + (pa >> 6)) fa = 1.0f;  // the ray's own Gaussian
+                        if (sm.leaf[nleaf + qb] == (uint32_t)first + (pb >> 6)) fb = 1.0f;
+                        sm.pair[i] = __float_as_uint(fa);
+                        if (i + 32 < total) sm.pair[i + 32] = __float_as_uint(fb);
+                    }
+                    __syncwarp();
+                    if (s0 + lane < live) {
+                        float T = sm.ro[ray].w;
+                        for (int i = from; i < end; ++i) T *= __uint_as_float(sm.pair[i]);
+                        sm.ro[ray].w = T;
+                        if (T < b.t_min) mk = make_uint2(0u, 0u);
+                    }
+                    __syncwarp();
+                }
             }
-        }
-        // the rays still live, closed up
-        bool ok[2];
-        float2 vxy[2];
-        float vz[2];
-        uint8_t id[2];
+            // the rays still live, closed up
+            bool ok[2];
+            float2 vxy[2];
+            float vz[2];
+            uint8_t id[2];
 #pragma unroll
-        for (int r = 0; r < 2; ++r) {
-            const int s = lane + 32 * r;
-            ok[r] = s < live;
-            if (ok[r]) {
-                id[r] = sm.live[s];
-                ok[r] = !(sm.ro[id[r]].w < b.t_min);
+            for (int r = 0; r < 2; ++r) {
+                const int s = lane + 32 * r;
+                ok[r] = s < live;
+                if (ok[r]) {
+                    id[r] = sm.live[s];
+                    ok[r] = !(sm.ro[id[r]].w < b.t_min);
+                }
             }
-        }
-        const unsigned k0 = __ballot_sync(FULL, ok[0]), k1 = __ballot_sync(FULL, ok[1]);
-        const int now = __popc(k0) + __popc(k1);
-        if (now == 0) break;
-        if (now < live) {
+            const unsigned k0 = __ballot_sync(FULL, ok[0]), k1 = __ballot_sync(FULL, ok[1]);
+            const int now = __popc(k0) + __popc(k1);
+            if (now == 0) break;
+            if (now < live) {
 #pragma unroll
-            for (int r = 0; r < 2; ++r)
-                if (ok[r]) {
-                    vxy[r] = sm.xy[lane + 32 * r];
-                    vz[r] = sm.z[lane + 32 * r];
-                }
-            __syncwarp();
-#pragma unroll
-            for (int r = 0; r < 2; ++r)
-                if (ok[r]) {
-                    const int s = r == 0 ? __popc(k0 & lt) : __popc(k0) + __popc(k1 & lt);
-                    sm.xy[s] = vxy[r];
-                    sm.z[s] = vz[r];
-                    sm.live[s] = id[r];
-                }
-            live = now;
-            if (4 * live <= 3 * bound) {  // the shaft of the rays left
-                bound = live;
+                for (int r = 0; r < 2; ++r)
+                    if (ok[r]) {
+                        vxy[r] = sm.xy[lane + 32 * r];
+                        vz[r] = sm.z[lane + 32 * r];
+                    }
                 __syncwarp();
-                bounds(live);
+#pragma unroll
+                for (int r = 0; r < 2; ++r)
+                    if (ok[r]) {
+                        const int s = r == 0 ? __popc(k0 & lt) : __popc(k0) + __popc(k1 & lt);
+                        sm.xy[s] = vxy[r];
+                        sm.z[s] = vz[r];
+                        sm.live[s] = id[r];
+                    }
+                live = now;
+                if (4 * live <= 3 * bound) {  // the shaft of the rays left
+                    bound = live;
+                    __syncwarp();
+                    bounds(live);
+                }
             }
         }
         __syncwarp();
@@ -463,12 +516,12 @@ __device__ __forceinline__ void shaft_group(const BvhDev &b, float eps, float3 d
 // One item of a direction set: group and direction, T written in the caller's
 // order.
 __device__ __forceinline__ void shaft_item(const BvhDev &b, const RaySetDev &rs, const TraceJob &job, float *T_out,
-                                           int64_t item, int *status, ShaftSmem &sm) {
+                                           int64_t item, int *status, ShaftSmem<false> &sm) {
     int64_t gi;
     int32_t k;
     full_item(job, rs.K, item, gi, k);
     const int2 gr = __ldg(b.groups + gi);
-    shaft_group(b, rs.eps, make_float3(__ldg(rs.dirs + 3 * k), __ldg(rs.dirs + 3 * k + 1), __ldg(rs.dirs + 3 * k + 2)),
+    shaft_group<false>(b, rs.eps, make_float3(__ldg(rs.dirs + 3 * k), __ldg(rs.dirs + 3 * k + 1), __ldg(rs.dirs + 3 * k + 2)),
                 gr.x, gr.y, status, sm);
     for (int i = threadIdx.x & 31; i < gr.y; i += 32) {
         const int64_t g = __float_as_int(__ldg(b.gauss + 4 * (int64_t)(gr.x + i) + 1).w);

@@ -69,7 +69,7 @@ __global__ void __launch_bounds__(128, RT_TRACE_MIN_BLOCKS) k_trace_lanes(BvhDev
 __global__ void __launch_bounds__(128, RT_SHAFT_MIN_BLOCKS) k_trace_shaft(BvhDev b, RaySetDev rs, TraceJob job,
                                                                           float *T_out, int *status,
                                                                           unsigned long long *work) {
-    __shared__ ShaftSmem sm[4];
+    __shared__ ShaftSmem<false> sm[4];
     for (;;) {
         unsigned long long item = 0;
         if ((threadIdx.x & 31) == 0) item = atomicAdd(work, 1ull);

@@ -103,6 +103,7 @@ _SIGS = {
     "rt_trace_visibility_dirs": (_I32, [_P, _P, _I32, _P, _P, _P]),
     "rt_visibility_dirs_host": (_I32, [_P, _P, _P, _P, _I64, _P, _I32, _P, _P, _P, _P]),
     "rt_memory_trim": (_I32, [_I64]),
+    "rt_backward_wants_log": (_I32, [_P, _P]),
     "rt_trace_visibility_backward": (_I32, [_P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _I32,
                                             _P, _P, _P, _P, _P, _P]),
     "rt_mlp_cfg_default": (None, [_P]),
@@ -563,6 +564,11 @@ def rt_materialize_rays(bvh: Bvh, rs: rt_rayspec, ray_ids, stream=None):
     _check(lib().rt_materialize_rays(bvh.handle, C.byref(rs), _ptr(ray_ids, torch.int64, "ray_ids"), m,
                                      _ptr(o), _ptr(d), _ptr(s), _stream(stream)), "rt_materialize_rays")
     return o, d, s
+
+
+def rt_backward_wants_log(bvh: Bvh, rs: rt_rayspec) -> bool:
+    """Whether the adjoint of this ray set is faster with the forward's hit log."""
+    return bool(lib().rt_backward_wants_log(bvh.handle, C.byref(rs)))
 
 
 def rt_trace_visibility_backward(bvh: Bvh, rs: rt_rayspec, mean, scale, quat, opacity, T, dL_dT,
