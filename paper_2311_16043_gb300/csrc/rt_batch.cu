@@ -93,99 +93,31 @@ struct BatchJobDev {
 // as in trace_refill, each lane carrying its own job.
 __device__ __forceinline__ void batch_refill(const BatchJobDev *__restrict__ jobs, int first, int n_jobs,
                                              int64_t total_slots, int *status, unsigned long long *work) {
-    const unsigned FULL = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
-    const unsigned lt_mask = (1u << lane) - 1u;
-    bool has = false, exhausted = false;
-    int jl = first;
-    float3 o = make_float3(0.f, 0.f, 0.f), d = make_float3(0.f, 0.f, 1.f), inv = d, oi = o;
-    int32_t src = -1;
-    int64_t out_idx = 0;
-    float T = 1.0f;
-    uint32_t node = 0;
-    int sp = 0;
-    uint32_t stack[RT_WIDE_STACK];
-    for (;;) {
-        const unsigned idle = __ballot_sync(FULL, !has);
-        const int n_idle = __popc(idle);
-        if (!exhausted && (n_idle >= kRefillMin || n_idle == 32)) {
-            unsigned long long base = 0;
-            if (lane == 0) base = atomicAdd(work, (unsigned long long)n_idle);
-            base = __shfl_sync(FULL, base, 0);
-            if (base + (unsigned long long)n_idle >= (unsigned long long)total_slots) exhausted = true;
-            if (!has) {
-                const int64_t slot = (int64_t)(base + (unsigned long long)__popc(idle & lt_mask));
-                if (slot < total_slots) {
-                    int lo = first, hi = n_jobs - 1;  // last refill job with slot_begin <= slot
-                    while (lo < hi) {
-                        const int mid = (lo + hi + 1) >> 1;
-                        if (jobs[mid].slot_begin <= slot) lo = mid;
-                        else hi = mid - 1;
-                    }
-                    jl = lo;
-                    const BatchJobDev &J = jobs[jl];
-                    const int64_t local = slot - J.slot_begin;
-                    int64_t tile;
-                    int32_t k;
-                    full_item(J.job, J.rs.K, local >> 5, tile, k);
-                    const int64_t p = tile * 32 + (local & 31);
-                    if (p < J.b.n) {
-                        const float4 mu = __ldg(J.b.gauss + 4 * p);
-                        const int64_t g = __float_as_int(__ldg(J.b.gauss + 4 * p + 1).w);
-                        out_idx = g * J.rs.K + k;
-                        implicit_ray(J.rs, out_idx, k, g, mu, o, d);
-                        inv = safe_inv(d);
-                        oi = make_float3(o.x * inv.x, o.y * inv.y, o.z * inv.z);
-                        src = (int32_t)p;
-                        T = 1.0f;
-                        node = 0;
-                        sp = 0;
-                        has = true;
-                    }
-                }
+    struct {
+        const BatchJobDev *__restrict__ jobs;
+        int first, n_jobs;
+        int64_t total;
+        int jl;
+        int64_t out_idx;
+        __device__ __forceinline__ unsigned long long slots() const { return (unsigned long long)total; }
+        __device__ __forceinline__ bool fetch(unsigned long long slot, float3 &o, float3 &d, int32_t &src) {
+            int lo = first, hi = n_jobs - 1;  // last refill job with slot_begin <= slot
+            while (lo < hi) {
+                const int mid = (lo + hi + 1) >> 1;
+                if (jobs[mid].slot_begin <= (int64_t)slot) lo = mid;
+                else hi = mid - 1;
             }
+            jl = lo;
+            const BatchJobDev &J = jobs[lo];
+            return slot_ray(J.b, J.rs, J.job, (int64_t)slot - J.slot_begin, o, d, src, out_idx);
         }
-        if (__ballot_sync(FULL, has) == 0) {
-            if (exhausted) break;
-            continue;
-        }
-        if (!has) continue;
-        const BvhDev &b = jobs[jl].b;
-        const bool far = far_first(jobs[jl].rs);
-        const float4 *w = b.wide + 8 * (int64_t)node;
-        const float4x2 nx = ldg_pair(w), ny = ldg_pair(w + 2), nz = ldg_pair(w + 4), nr = ldg_pair(w + 6);
-        const float4 lx = nx.a, hx = nx.b, ly = ny.a, hy = ny.b, lz = nz.a, hz = nz.b, rf = nr.a;
-        const uint32_t r[4] = {__float_as_uint(rf.x), __float_as_uint(rf.y), __float_as_uint(rf.z),
-                               __float_as_uint(rf.w)};
-        float tn[4];
-        slab4_near(lx, hx, ly, hy, lz, hz, oi, inv, tn);
-        const float inf = __int_as_float(0x7f800000);
-        float ti[4];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            ti[c] = inf;
-            if (!(tn[c] < inf)) continue;
-            if (r[c] & RT_LEAF_BIT) {
-                const int32_t p = (int32_t)(r[c] & ~RT_LEAF_BIT);
-                if (p != src) gauss_hit(b, p, o, d, T);
-            } else {
-                ti[c] = tn[c];
-            }
-        }
-        int next = -1;
-        const bool overflow = !visit_order(ti[0], ti[1], ti[2], ti[3], r[0], r[1], r[2], r[3], far, stack, sp, next);
-        if (overflow) rt_set_error(status, RT_ERR_STACK_OVERFLOW);
-        bool done = overflow || T < b.t_min;
-        if (!done) {
-            if (next >= 0) node = (uint32_t)next;
-            else if (sp > 0) node = stack[--sp];
-            else done = true;
-        }
-        if (done) {
-            jobs[jl].T_out[out_idx] = T < b.t_min ? 0.0f : T;
-            has = false;
-        }
-    }
+        __device__ __forceinline__ const BvhDev &tree() const { return jobs[jl].b; }
+        __device__ __forceinline__ bool far() const { return far_first(jobs[jl].rs); }
+        __device__ __forceinline__ void store(float T) const { jobs[jl].T_out[out_idx] = T; }
+    } from = {jobs, first, n_jobs, total_slots, first, 0};
+    WorkCounts wc = {0, 0, 0};
+    unsigned long long rays_done = 0;
+    refill_walk<false>(from, status, work, wc, rays_done);
 }
 
 // Jobs [0, n_item_jobs) are consumed as 32-ray items (work[0]); jobs

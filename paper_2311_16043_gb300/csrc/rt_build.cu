@@ -742,6 +742,49 @@ __device__ __forceinline__ void wide_children(const float4 *__restrict__ nodes, 
     r.area = (r.ref & RT_LEAF_BIT) ? -2.0f : box_area(r.b);
 }
 
+// One axis of a 64-byte node: base, step and the bytes of the children's
+// planes.  The children's extent takes bytes 1 to 251; the step is at least
+// 2^-19 of the coordinates, so that a plane's own rounding is below 0.04
+// steps, and planes are moved outwards by 0.1 steps before they are rounded.
+// A child with a NaN box gets an inside-out one, an axis beyond 1e23 a NaN
+// base (every child passes).
+__device__ __forceinline__ void quantize_axis(const float (&lo)[4], const float (&hi)[4], float &base, float &step,
+                                              uint32_t &ql, uint32_t &qh) {
+    const float l = fminf(fminf(lo[0], lo[1]), fminf(lo[2], lo[3])), h = fmaxf(fmaxf(hi[0], hi[1]), fmaxf(hi[2], hi[3]));
+    ql = 0xffffffffu;
+    qh = 0u;
+    base = 0.0f;
+    step = 1.0f;
+    if (!(l == l)) return;  // no child has a box
+    const float big = fmaxf(fabsf(l), fabsf(h)), s = fmaxf(fmaxf((h - l) * (1.0f / 248.0f), big * 1.9073486e-6f), 1e-30f);
+    if (!(big < 1e23f)) {
+        base = __int_as_float(0x7fc00000);
+        return;
+    }
+    step = 32768.0f * s;
+    base = (l - 2.0f * s) - step;
+    const float zero = base + step, is = 1.0f / s;
+    ql = qh = 0u;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        const bool box = lo[c] == lo[c];
+        const float a = floorf(fmaf(lo[c] - zero, is, -0.1f)), b = ceilf(fmaf(hi[c] - zero, is, 0.1f));
+        ql |= (box ? (uint32_t)fminf(fmaxf(a, 0.0f), 255.0f) : 255u) << (8 * c);
+        qh |= (box ? (uint32_t)fminf(fmaxf(b, 0.0f), 255.0f) : 0u) << (8 * c);
+    }
+}
+__device__ __forceinline__ void store_qnode(float4 *q, const float (&lo)[3][4], const float (&hi)[3][4], float4 refs) {
+    float base[3], step[3];
+    uint32_t ql[3], qh[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) quantize_axis(lo[a], hi[a], base[a], step[a], ql[a], qh[a]);
+    auto f = [](uint32_t u) { return __uint_as_float(u); };
+    q[0] = make_float4(base[0], base[1], base[2], step[0]);
+    q[1] = make_float4(step[1], step[2], f(ql[0]), f(qh[0]));
+    q[2] = make_float4(f(ql[1]), f(qh[1]), f(ql[2]), f(qh[2]));
+    q[3] = refs;
+}
+
 // The 4-wide tree.  The children of a wide node that starts from binary node
 // e are found by greedy expansion (the internal child of largest surface area
 // is replaced by its two children, twice), which depends on e's descendants
@@ -750,7 +793,8 @@ __device__ __forceinline__ void wide_children(const float4 *__restrict__ nodes, 
 // it starts from.  The nodes no other refers to (about half) are never read.
 // Top-down, level by level, took 63 launches (276 us at 300k Gaussians, 181 us
 // at 4k; 105 and 40 us with one block for the top and a thread per subtree).
-__global__ void __launch_bounds__(128) k_wide(const float4 *__restrict__ nodes, int64_t ni, float4 *wide) {
+__global__ void __launch_bounds__(128) k_wide(const float4 *__restrict__ nodes, int64_t ni, float4 *wide,
+                                              float4 *qwide) {
     for (int64_t e = blockIdx.x * 128ll + threadIdx.x; e < ni; e += (int64_t)gridDim.x * 128) {
         // 2 children, then the larger's two behind the other, then the largest
         // of three replaced by the last and its two children appended
@@ -782,39 +826,75 @@ __global__ void __launch_bounds__(128) k_wide(const float4 *__restrict__ nodes, 
         float4 *w = wide + 8 * e;
 #pragma unroll
         for (int k = 0; k < 6; ++k) w[k] = make_float4(s0.b[k], s1.b[k], s2.b[k], s3.b[k]);
-        w[6] = make_float4(__uint_as_float(s0.ref), __uint_as_float(s1.ref), __uint_as_float(s2.ref),
-                           __uint_as_float(s3.ref));
+        const float4 refs = make_float4(__uint_as_float(s0.ref), __uint_as_float(s1.ref), __uint_as_float(s2.ref),
+                                        __uint_as_float(s3.ref));
+        w[6] = refs;
         w[7] = make_float4(0.f, 0.f, 0.f, 0.f);
+        float lo[3][4], hi[3][4];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            lo[a][0] = s0.b[2 * a], lo[a][1] = s1.b[2 * a], lo[a][2] = s2.b[2 * a], lo[a][3] = s3.b[2 * a];
+            hi[a][0] = s0.b[2 * a + 1], hi[a][1] = s1.b[2 * a + 1], hi[a][2] = s2.b[2 * a + 1];
+            hi[a][3] = s3.b[2 * a + 1];
+        }
+        store_qnode(qwide + 4 * e, lo, hi, refs);
     }
 }
 
 // Refit of the 4-wide tree with its slots kept, after the binary tree's: the
 // box of a child is the leaf's, or the union of the binary node's two.
+// A thread per child, the four of a node side by side; lane a < 3 of them then
+// quantizes axis a of the 64-byte node.
 __global__ void __launch_bounds__(256) k_refit_wide(const float *__restrict__ leafbox, const float4 *__restrict__ nodes,
-                                                    int64_t ni, float *wide) {
-    for (int64_t j = blockIdx.x * 256ll + threadIdx.x; j < 4 * ni; j += (int64_t)gridDim.x * 256) {
-        float *w = wide + 32 * (j >> 2) + (j & 3);
-        const uint32_t r = __float_as_uint(w[24]);
-        if (r == RT_EMPTY) continue;
-        float lo[3], hi[3];
-        if (r & RT_LEAF_BIT) {
-            const float *b = leafbox + 6 * (int64_t)(r & ~RT_LEAF_BIT);
+                                                    int64_t ni, float *wide, float *qwide) {
+    const int64_t total = (4 * ni + 31) / 32 * 32;  // whole warps
+    for (int64_t j = blockIdx.x * 256ll + threadIdx.x; j < total; j += (int64_t)gridDim.x * 256) {
+        const bool in = j < 4 * ni;
+        float *w = wide + 32 * (in ? j >> 2 : 0) + (j & 3);
+        const uint32_t r = in ? __float_as_uint(w[24]) : RT_EMPTY;
+        const float none = __int_as_float(0x7fc00000);
+        float lo[3] = {none, none, none}, hi[3] = {none, none, none};
+        if (r != RT_EMPTY) {
+            if (r & RT_LEAF_BIT) {
+                const float *b = leafbox + 6 * (int64_t)(r & ~RT_LEAF_BIT);
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    lo[c] = b[c];
+                    hi[c] = b[3 + c];
+                }
+            } else {
+                const float4 x = nodes[4 * (int64_t)r], y = nodes[4 * (int64_t)r + 1], z = nodes[4 * (int64_t)r + 2];
+                lo[0] = fminf(x.x, y.z); hi[0] = fmaxf(x.y, y.w);
+                lo[1] = fminf(x.z, z.x); hi[1] = fmaxf(x.w, z.y);
+                lo[2] = fminf(y.x, z.z); hi[2] = fmaxf(y.y, z.w);
+            }
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                lo[c] = b[c];
-                hi[c] = b[3 + c];
+                w[8 * c] = lo[c];
+                w[8 * c + 4] = hi[c];
             }
-        } else {
-            const float4 x = nodes[4 * (int64_t)r], y = nodes[4 * (int64_t)r + 1], z = nodes[4 * (int64_t)r + 2];
-            lo[0] = fminf(x.x, y.z); hi[0] = fmaxf(x.y, y.w);
-            lo[1] = fminf(x.z, z.x); hi[1] = fmaxf(x.w, z.y);
-            lo[2] = fminf(y.x, z.z); hi[2] = fmaxf(y.y, z.w);
         }
+        const int axis = (int)(j & 3);
+        float l4[4], h4[4];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            w[8 * c] = lo[c];
-            w[8 * c + 4] = hi[c];
-        }
+        for (int k = 0; k < 4; ++k)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const float l = __shfl_sync(0xffffffffu, lo[c], k, 4), h = __shfl_sync(0xffffffffu, hi[c], k, 4);
+                if (c == axis || c == 0) {
+                    l4[k] = l;
+                    h4[k] = h;
+                }
+            }
+        if (!in || axis == 3) continue;
+        float base, step;
+        uint32_t ql, qh;
+        quantize_axis(l4, h4, base, step, ql, qh);
+        float *q = qwide + 16 * (j >> 2);
+        q[axis] = base;
+        q[3 + axis] = step;
+        q[6 + 2 * axis] = __uint_as_float(ql);
+        q[7 + 2 * axis] = __uint_as_float(qh);
     }
 }
 
@@ -944,7 +1024,8 @@ extern "C" rt_status rt_build_bvh(const float *mean, const float *scale, const f
     size_t off_bnd = off_par + align256(sizeof(int32_t) * (size_t)(n > 0 ? 2 * n - 1 : 0));
     size_t off_grp = off_bnd + 256;
     size_t off_wide = off_grp + align256(sizeof(int2) * (size_t)n);
-    size_t total = off_wide + align256(sizeof(float4) * 8 * (size_t)ni);
+    size_t off_qwide = off_wide + align256(sizeof(float4) * 8 * (size_t)ni);
+    size_t total = off_qwide + align256(sizeof(float4) * 4 * (size_t)ni);
     rt_status s = rt_alloc(&b->block, total, stream);
     if (s != RT_OK) {
         delete b;
@@ -962,6 +1043,7 @@ extern "C" rt_status rt_build_bvh(const float *mean, const float *scale, const f
     b->groups = (int2 *)(base + off_grp);
     b->n_groups = 0;
     b->wide = (float4 *)(base + off_wide);
+    b->qwide = (float4 *)(base + off_qwide);
     b->n_wide = 0;
     b->levels = 0;
     for (int c = 0; c < 3; ++c) b->lo[c] = b->hi[c] = 0.f;
@@ -1013,7 +1095,7 @@ extern "C" rt_status rt_build_bvh(const float *mean, const float *scale, const f
             if (cudaMemsetAsync(b->parent, 0xff, sizeof(int32_t), st) != cudaSuccess) result = RT_ERR_CUDA;  // -1
         } else {
             k_refit<<<refit_grid(n), kRefitLeaves, 0, st>>>(leafbox, b->parent, n, b->nodes, arrivals, scn + SCN_LEVELS);
-            k_wide<<<grid_for(ni, 128), 128, 0, st>>>(b->nodes, ni, b->wide);
+            k_wide<<<grid_for(ni, 128), 128, 0, st>>>(b->nodes, ni, b->wide, b->qwide);
             b->n_wide = ni;
         }
         if (rt_check_launch() != RT_OK) result = RT_ERR_CUDA;
@@ -1072,7 +1154,8 @@ extern "C" rt_status rt_bvh_refit(rt_bvh *b, const float *mean, const float *sca
             k_refit<<<refit_grid(n), kRefitLeaves, 0, st>>>(leafbox, b->parent, n, b->nodes, arrivals, scn + SCN_LEVELS);
         }
         if (b->n_wide > 0)
-            k_refit_wide<<<grid_for(4 * ni, 256), 256, 0, st>>>(leafbox, b->nodes, ni, (float *)b->wide);
+            k_refit_wide<<<grid_for(4 * ni, 256), 256, 0, st>>>(leafbox, b->nodes, ni, (float *)b->wide,
+                                                                       (float *)b->qwide);
         result = rt_check_launch();
     } while (0);
     rt_free(scratch, stream);

@@ -39,6 +39,15 @@
 //                RT_EMPTY = no child, else a wide node index
 //   w[8j+7]    = unused
 // Empty children and empty leaf boxes are NaN boxes, which no ray hits.
+//
+// The same node in 64 bytes for the walks of single rays, node j:
+//   q[4j]   = base.x, base.y, base.z, step.x
+//   q[4j+1] = step.y, step.z, lo.x[4], hi.x[4] (a byte per child)
+//   q[4j+2] = lo.y[4], hi.y[4], lo.z[4], hi.z[4]
+//   q[4j+3] = child refs
+// A plane of byte k lies at base + step (1 + k / 2^15), rounded outwards (see
+// quantize_axis): 1 + k / 2^15 is the float with k in the second byte of its
+// mantissa, so decoding is one byte permutation.
 
 struct rt_bvh {
     int64_t n;
@@ -56,6 +65,7 @@ struct rt_bvh {
     int2 *groups;            // [n_groups] first sorted position and count of each shaft group
     int64_t n_groups;        // (host copy)
     float4 *wide;            // [8 * (n-1)] 4-wide nodes (collapsed binary tree)
+    float4 *qwide;           // [4 * (n-1)] the same nodes in 64 bytes (below)
     int64_t n_wide;          // indices of 4-wide nodes: n-1, or 0 for n < 2
     int32_t levels;          // levels of the binary tree, a bound on the 4-wide one's (host copy)
 };

@@ -8,6 +8,7 @@ struct BvhDev {
     const float4 *gauss;
     const float4 *nodes;
     const float4 *wide;  // null if the 4-wide tree is unavailable
+    const float4 *qwide;
     const int32_t *rank;
     const int2 *groups;  // first sorted position and count of each shaft group
     int64_t n;
@@ -22,6 +23,7 @@ inline BvhDev bvh_dev(const rt_bvh *b) {
     d.gauss = b->gauss;
     d.nodes = b->nodes;
     d.wide = b->n_wide > 0 ? b->wide : nullptr;
+    d.qwide = b->qwide;
     d.rank = b->rank;
     d.groups = b->groups;
     d.n = b->n;
@@ -124,6 +126,62 @@ __device__ __forceinline__ void slab4_near(float4 lx, float4 hx, float4 ly, floa
         const float fb = fminf(fminf(fmaxf(tx0.y, tx1.y), fmaxf(ty0.y, ty1.y)), fmaxf(tz0.y, tz1.y));
         tn[2 * pr] = na <= fmaf(fabsf(fa), 1e-6f, fa) ? na : inf;
         tn[2 * pr + 1] = nb <= fmaf(fabsf(fb), 1e-6f, fb) ? nb : inf;
+    }
+}
+
+// Per-ray terms of qnode_near.  Only the sign and the order of the distances
+// along the ray matter, so d is scaled by its largest component; a small
+// component counts as 1e-12 of it (off by the boxes' margin, 1e-6 of the scene,
+// after 1e6 scenes) so that step * inv stays finite for nodes of up to 1e23.
+// False for a ray with a component that is not finite, which meets no Gaussian.
+__device__ __forceinline__ bool qnode_ray(float3 o, float3 d, float3 &inv, float3 &oi) {
+    const float m = fmaxf(fmaxf(fabsf(d.x), fabsf(d.y)), fmaxf(fabsf(d.z), 1e-30f)), tiny = fmaxf(1e-12f * m, 1e-37f);
+    auto rcp = [&](float x) { return m / (fabsf(x) < tiny ? copysignf(tiny, x) : x); };
+    inv = make_float3(rcp(d.x), rcp(d.y), rcp(d.z));
+    oi = make_float3(o.x * inv.x, o.y * inv.y, o.z * inv.z);
+    const float inf = __int_as_float(0x7f800000);
+    return fabsf(o.x) < inf && fabsf(o.y) < inf && fabsf(o.z) < inf && fabsf(d.x) < inf && fabsf(d.y) < inf &&
+           fabsf(d.z) < inf;
+}
+
+// The four children of a 64-byte node against a ray: child refs, and each
+// box's entry distance (in units of qnode_ray), +inf where the ray misses the
+// box or there is no child.  A plane's distance is (1 + k / 2^15) a + c with
+// a = step inv and c = base inv - o inv; the two roundings of up to 2^-24 of
+// 2^15 steps are 0.004 steps, within the 0.1 that quantize_axis adds.  An axis
+// of NaN base does not count.
+// Two 32-byte loads instead of four: the walks of single rays are bound by the
+// L1 data pipe, a wavefront per lane and load.
+__device__ __forceinline__ void qnode_near(const float4 *__restrict__ q, float3 inv, float3 oi, float (&tn)[4],
+                                           uint32_t (&r)[4]) {
+    const float4x2 n0 = ldg_pair(q), n1 = ldg_pair(q + 2);
+    const float ax = n0.a.w * inv.x, ay = n0.b.x * inv.y, az = n0.b.y * inv.z;
+    const float cx = fmaf(n0.a.x, inv.x, -oi.x), cy = fmaf(n0.a.y, inv.y, -oi.y), cz = fmaf(n0.a.z, inv.z, -oi.z);
+    const bool sx = inv.x < 0.0f, sy = inv.y < 0.0f, sz = inv.z < 0.0f;
+    const uint32_t lx = __float_as_uint(n0.b.z), hx = __float_as_uint(n0.b.w), ly = __float_as_uint(n1.a.x),
+                   hy = __float_as_uint(n1.a.y), lz = __float_as_uint(n1.a.z), hz = __float_as_uint(n1.a.w);
+    const uint32_t nx = sx ? hx : lx, fx = sx ? lx : hx, ny = sy ? hy : ly, fy = sy ? ly : hy, nz = sz ? hz : lz,
+                   fz = sz ? lz : hz;
+    r[0] = __float_as_uint(n1.b.x);
+    r[1] = __float_as_uint(n1.b.y);
+    r[2] = __float_as_uint(n1.b.z);
+    r[3] = __float_as_uint(n1.b.w);
+    const float inf = __int_as_float(0x7f800000);
+#pragma unroll
+    for (int pr = 0; pr < 2; ++pr) {
+        auto two = [&](uint32_t w) {
+            return make_float2(__uint_as_float(__byte_perm(w, 0x3f800000u, pr ? 0x7624u : 0x7604u)),
+                               __uint_as_float(__byte_perm(w, 0x3f800000u, pr ? 0x7634u : 0x7614u)));
+        };
+        auto dist = [&](uint32_t w, float a, float c) {
+            return __ffma2_rn(two(w), make_float2(a, a), make_float2(c, c));
+        };
+        const float2 nx2 = dist(nx, ax, cx), fx2 = dist(fx, ax, cx), ny2 = dist(ny, ay, cy), fy2 = dist(fy, ay, cy),
+                     nz2 = dist(nz, az, cz), fz2 = dist(fz, az, cz);
+        const float na = fmaxf(fmaxf(nx2.x, ny2.x), fmaxf(nz2.x, 0.0f)), fa = fminf(fminf(fx2.x, fy2.x), fz2.x);
+        const float nb = fmaxf(fmaxf(nx2.y, ny2.y), fmaxf(nz2.y, 0.0f)), fb = fminf(fminf(fx2.y, fy2.y), fz2.y);
+        tn[2 * pr] = !(na > fmaf(fabsf(fa), 1e-6f, fa)) && r[2 * pr] != RT_EMPTY ? na : inf;
+        tn[2 * pr + 1] = !(nb > fmaf(fabsf(fb), 1e-6f, fb)) && r[2 * pr + 1] != RT_EMPTY ? nb : inf;
     }
 }
 
@@ -769,31 +827,35 @@ __device__ __forceinline__ void flush_counts(const TraceAux &aux, const WorkCoun
 // item order); whenever at least kRefillMin lanes of the warp are idle, lane
 // 0 takes that many slots with one atomic and the idle lanes start them, so a
 // warp no longer waits for its longest ray.  Each step of a lane is one node
-// visit of trace_ray_wide's loop, and a ray's visits and factors come in the
-// same order as there: the same T.  Slots past a ragged last tile are
-// skipped.  `work` counts slots.
+// visit.  Slots past a ragged last tile are skipped.  `work` counts slots.
+// Nodes are the 64-byte ones: with the 128-byte nodes the L1 data pipe was 91 %
+// busy (a wavefront per lane and 32-byte load, 76 nodes and 71 Gaussians a ray);
+// hemisphere set of the 300k object scene x 64 44.9 -> 35.9 ms, 200k
+// environment set x 64 28.7 -> 23.2, 600k shadow rays (strategy 6) 2.02 -> 1.65.
+// The quantized boxes cost 1.5 % more nodes and Gaussians, the nodes 64 bytes a
+// Gaussian and 4 us of the build at 4k, 13 at 300k.
 #ifndef RT_REFILL_MIN
 #define RT_REFILL_MIN 8
 #endif
 constexpr int kRefillMin = RT_REFILL_MIN;
 
-template <bool COUNT>
-__device__ __forceinline__ void trace_refill(const BvhDev &b, const RaySetDev &rs, const TraceJob &job, float *T_out,
-                                             const TraceAux &aux, unsigned long long *work, WorkCounts &wc,
-                                             unsigned long long &rays_done) {
+// `Src` is what the rays come from: slots(), fetch(slot, o, d, src) (false past
+// a ragged last tile; remembers where the slot's T goes), tree(), far() and
+// store(T).
+template <bool COUNT, class Src>
+__device__ __forceinline__ void refill_walk(Src &from, int *status, unsigned long long *work, WorkCounts &wc,
+                                            unsigned long long &rays_done) {
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const unsigned lt_mask = (1u << lane) - 1u;
-    const unsigned long long total = (unsigned long long)job.n_items * 32ull;
+    const unsigned long long total = from.slots();
     bool has = false, exhausted = false;
     float3 o = make_float3(0.f, 0.f, 0.f), d = make_float3(0.f, 0.f, 1.f), inv = d, oi = o;
     int32_t src = -1;
-    int64_t out_idx = 0;
     float T = 1.0f;
     uint32_t node = 0;
     int sp = 0;
     uint32_t stack[RT_WIDE_STACK];
-    const bool far = far_first(rs);
     for (;;) {
         const unsigned idle = __ballot_sync(FULL, !has);
         const int n_idle = __popc(idle);
@@ -804,23 +866,14 @@ __device__ __forceinline__ void trace_refill(const BvhDev &b, const RaySetDev &r
             if (base + (unsigned long long)n_idle >= total) exhausted = true;
             if (!has) {
                 const unsigned long long slot = base + (unsigned long long)__popc(idle & lt_mask);
-                if (slot < total) {
-                    int64_t tile;
-                    int32_t k;
-                    full_item(job, rs.K, (int64_t)(slot >> 5), tile, k);
-                    const int64_t p = tile * 32 + (int64_t)(slot & 31ull);
-                    if (p < b.n) {
-                        const float4 mu = __ldg(b.gauss + 4 * p);
-                        const int64_t g = __float_as_int(__ldg(b.gauss + 4 * p + 1).w);
-                        out_idx = g * rs.K + k;
-                        implicit_ray(rs, out_idx, k, g, mu, o, d);
-                        inv = safe_inv(d);
-                        oi = make_float3(o.x * inv.x, o.y * inv.y, o.z * inv.z);
-                        src = (int32_t)p;
-                        T = 1.0f;
-                        node = 0;
-                        sp = 0;
-                        has = true;
+                if (slot < total && from.fetch(slot, o, d, src)) {
+                    has = qnode_ray(o, d, inv, oi);
+                    T = 1.0f;
+                    node = 0;
+                    sp = 0;
+                    if (!has) {
+                        from.store(1.0f);
+                        rays_done++;
                     }
                 }
             }
@@ -830,14 +883,10 @@ __device__ __forceinline__ void trace_refill(const BvhDev &b, const RaySetDev &r
             continue;
         }
         if (!has) continue;
-        // one visit of trace_ray_wide's loop
-        const float4 *w = b.wide + 8 * (int64_t)node;
-        const float4x2 nx = ldg_pair(w), ny = ldg_pair(w + 2), nz = ldg_pair(w + 4), nr = ldg_pair(w + 6);
-        const float4 lx = nx.a, hx = nx.b, ly = ny.a, hy = ny.b, lz = nz.a, hz = nz.b, rf = nr.a;
-        const uint32_t r[4] = {__float_as_uint(rf.x), __float_as_uint(rf.y), __float_as_uint(rf.z),
-                               __float_as_uint(rf.w)};
+        const BvhDev &b = from.tree();
         float tn[4];
-        slab4_near(lx, hx, ly, hy, lz, hz, oi, inv, tn);
+        uint32_t r[4];
+        qnode_near(b.qwide + 4 * (int64_t)node, inv, oi, tn, r);
         if (COUNT) wc.box += (r[0] != RT_EMPTY) + (r[1] != RT_EMPTY) + (r[2] != RT_EMPTY) + (r[3] != RT_EMPTY);
         const float inf = __int_as_float(0x7f800000);
         float ti[4];
@@ -856,8 +905,9 @@ __device__ __forceinline__ void trace_refill(const BvhDev &b, const RaySetDev &r
             }
         }
         int next = -1;
-        const bool overflow = !visit_order(ti[0], ti[1], ti[2], ti[3], r[0], r[1], r[2], r[3], far, stack, sp, next);
-        if (overflow) rt_set_error(aux.status, RT_ERR_STACK_OVERFLOW);
+        const bool overflow =
+            !visit_order(ti[0], ti[1], ti[2], ti[3], r[0], r[1], r[2], r[3], from.far(), stack, sp, next);
+        if (overflow) rt_set_error(status, RT_ERR_STACK_OVERFLOW);
         bool done = overflow || T < b.t_min;
         if (!done) {
             if (next >= 0) node = (uint32_t)next;
@@ -865,11 +915,48 @@ __device__ __forceinline__ void trace_refill(const BvhDev &b, const RaySetDev &r
             else done = true;
         }
         if (done) {
-            T_out[out_idx] = T < b.t_min ? 0.0f : T;
+            from.store(T < b.t_min ? 0.0f : T);
             rays_done++;
             has = false;
         }
     }
+}
+
+// The ray of slot `slot` of a full implicit set: false past a ragged last tile.
+__device__ __forceinline__ bool slot_ray(const BvhDev &b, const RaySetDev &rs, const TraceJob &job, int64_t slot,
+                                         float3 &o, float3 &d, int32_t &src, int64_t &out_idx) {
+    int64_t tile;
+    int32_t k;
+    full_item(job, rs.K, slot >> 5, tile, k);
+    const int64_t p = tile * 32 + (slot & 31);
+    if (p >= b.n) return false;
+    const float4 mu = __ldg(b.gauss + 4 * p);
+    const int64_t g = __float_as_int(__ldg(b.gauss + 4 * p + 1).w);
+    out_idx = g * rs.K + k;
+    implicit_ray(rs, out_idx, k, g, mu, o, d);
+    src = (int32_t)p;
+    return true;
+}
+
+template <bool COUNT>
+__device__ __forceinline__ void trace_refill(const BvhDev &b, const RaySetDev &rs, const TraceJob &job, float *T_out,
+                                             const TraceAux &aux, unsigned long long *work, WorkCounts &wc,
+                                             unsigned long long &rays_done) {
+    struct {
+        const BvhDev &b;
+        const RaySetDev &rs;
+        const TraceJob &job;
+        float *T_out;
+        int64_t out_idx;
+        __device__ __forceinline__ unsigned long long slots() const { return (unsigned long long)job.n_items * 32ull; }
+        __device__ __forceinline__ bool fetch(unsigned long long slot, float3 &o, float3 &d, int32_t &src) {
+            return slot_ray(b, rs, job, (int64_t)slot, o, d, src, out_idx);
+        }
+        __device__ __forceinline__ const BvhDev &tree() const { return b; }
+        __device__ __forceinline__ bool far() const { return far_first(rs); }
+        __device__ __forceinline__ void store(float T) const { T_out[out_idx] = T; }
+    } from = {b, rs, job, T_out, 0};
+    refill_walk<COUNT>(from, aux.status, work, wc, rays_done);
 }
 
 // Strategy 6: LANES (4, 8, 16 or 32) lanes per ray over the 4-wide tree, for
@@ -917,12 +1004,16 @@ __device__ __forceinline__ void trace_lane_group(const BvhDev &b, const RaySetDe
             } else if (!ray_of(b, rs, job, (int64_t)item, o, d, src, out_idx, aux.status)) {
                 if (sub == 0 && out_idx >= 0) T_out[out_idx] = __int_as_float(0x7fc00000);
             } else {
-                has = true;
-                inv = safe_inv(d);
-                oi = make_float3(o.x * inv.x, o.y * inv.y, o.z * inv.z);
+                has = qnode_ray(o, d, inv, oi);
                 Tl = 1.0f;
                 size = 1;
-                if (sub == 0) stk[0] = 0u;
+                if (sub == 0) {
+                    stk[0] = 0u;
+                    if (!has) {
+                        T_out[out_idx] = 1.0f;
+                        rays_done++;
+                    }
+                }
             }
         }
         if (!__any_sync(FULL, has || more)) break;
@@ -934,18 +1025,12 @@ __device__ __forceinline__ void trace_lane_group(const BvhDev &b, const RaySetDe
         __syncwarp();
         uint32_t r[4] = {0u, 0u, 0u, 0u}, pm = 0u;  // internal children to push: a mask over c
         if (sub < k) {
-            const float4 *w = b.wide + 8 * (int64_t)node;
-            const float4x2 nx = ldg_pair(w), ny = ldg_pair(w + 2), nz = ldg_pair(w + 4), nr = ldg_pair(w + 6);
-            r[0] = __float_as_uint(nr.a.x);
-            r[1] = __float_as_uint(nr.a.y);
-            r[2] = __float_as_uint(nr.a.z);
-            r[3] = __float_as_uint(nr.a.w);
-            bool h[4];
-            slab4(nx.a, nx.b, ny.a, ny.b, nz.a, nz.b, oi, inv, h);
+            float tn[4];
+            qnode_near(b.qwide + 4 * (int64_t)node, inv, oi, tn, r);
             if (COUNT) wc.box += (r[0] != RT_EMPTY) + (r[1] != RT_EMPTY) + (r[2] != RT_EMPTY) + (r[3] != RT_EMPTY);
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
-                if (!h[c]) continue;
+                if (!(tn[c] < __int_as_float(0x7f800000))) continue;
                 if (r[c] & RT_LEAF_BIT) {
                     const int32_t p = (int32_t)(r[c] & ~RT_LEAF_BIT);
                     if (p != src) {
