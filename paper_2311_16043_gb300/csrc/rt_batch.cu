@@ -12,10 +12,10 @@
 // Batch: the work items of all jobs form virtual queues, job after job in
 // decreasing estimated cost (rays x log2 n), consumed through device counters
 // by persistent grids; each warp finds its job by binary search over the jobs'
-// first item and runs that job's strategy.  Shaft jobs (direction sets) have
-// a kernel of their own, since its shared memory would cost the other
-// strategies residency (20 instead of 32 warps); the two are parallel
-// branches of one captured CUDA graph with the counters' reset.
+// first item and runs that job's strategy.  Shaft jobs (direction sets), lane
+// refill jobs (env-map and hemisphere sets) and the others have a kernel each
+// (20, 36 and 32 warps a multiprocessor fit), parallel branches of one captured
+// CUDA graph after the counters' reset.
 #include <math.h>
 #include <string.h>
 
@@ -44,17 +44,18 @@ std::map<TuneKey, std::pair<int, int>> g_tune_cache;
 constexpr int kTuneBlocks = 4;
 constexpr float kTuneMargin = 0.97f;
 
-// The strategy used without tuning: for a direction set over more than 2^15
-// Gaussians shaft packets where they pay (rt_shaft_pays), else one thread per
-// ray on the 4-wide tree (far-first; small jobs keep the strategy they always
-// reported here, tuning finds the faster one); one thread per ray on the
+// The strategy used without tuning: for a direction set over more than 20,000
+// Gaussians shaft packets where they pay (rt_shaft_pays; uniform 30k x 32
+// directions 1.2 ms against 4.4), else one thread per ray on the 4-wide tree
+// (far-first; jobs of up to 20,000 keep the strategy they always reported
+// here, tuning finds the faster one: uniform 4k 0.13 ms against 0.30); one thread per ray on the
 // 4-wide tree with lane refill for env-map and hemisphere rays (their
 // directions differ within a tile); binary variants when there is no 4-wide
 // tree.
 int default_kernel(const rt_bvh *bvh, int32_t kind) {
     if (kind == RT_RAYS_DIRS) {
         if (bvh->n_wide == 0) return RT_KERNEL_PACKET;
-        return bvh->n > (int64_t(1) << 15) && rt_shaft_pays(bvh) ? RT_KERNEL_WIDE : RT_KERNEL_RAY_WIDE;
+        return bvh->n > 20000 && rt_shaft_pays(bvh) ? RT_KERNEL_WIDE : RT_KERNEL_RAY_WIDE;
     }
     return bvh->n_wide > 0 ? RT_KERNEL_RAY_REFILL : RT_KERNEL_RAY;
 }
@@ -120,15 +121,12 @@ __device__ __forceinline__ void batch_refill(const BatchJobDev *__restrict__ job
     refill_walk<false>(from, status, work, wc, rays_done);
 }
 
-// Jobs [0, n_item_jobs) are consumed as 32-ray items (work[0]); jobs
-// [n_item_jobs, n_jobs) as per-ray slots with lane refill (work[1]), after a
-// warp finds the item queue empty.
+// The jobs [0, n_item_jobs) that are consumed as 32-ray items.
 #ifndef RT_BATCH_MIN_BLOCKS
 #define RT_BATCH_MIN_BLOCKS 8
 #endif
-__global__ void __launch_bounds__(128, RT_BATCH_MIN_BLOCKS) k_trace_batch(const BatchJobDev *__restrict__ jobs, int n_item_jobs, int n_jobs,
-                                                     int64_t total_items, int64_t total_slots, int *status,
-                                                     unsigned long long *work) {
+__global__ void __launch_bounds__(128, RT_BATCH_MIN_BLOCKS) k_trace_batch(const BatchJobDev *__restrict__ jobs, int n_item_jobs,
+                                                     int64_t total_items, int *status, unsigned long long *work) {
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     __shared__ int2 stk_all[4 * RT_WIDE_STACK];
@@ -159,7 +157,12 @@ __global__ void __launch_bounds__(128, RT_BATCH_MIN_BLOCKS) k_trace_batch(const 
         else if (J.strat == 1) trace_item<1, false>(J.b, J.rs, J.job, J.T_out, aux, local, J.job.n_out, wc, rays_done, stk);
         else trace_item<0, false>(J.b, J.rs, J.job, J.T_out, aux, local, J.job.n_out, wc, rays_done, stk);
     }
-    if (total_slots > 0) batch_refill(jobs, n_item_jobs, n_jobs, total_slots, status, work + 1);
+}
+
+__global__ void __launch_bounds__(128, RT_REFILL_MIN_BLOCKS) k_refill_batch(const BatchJobDev *__restrict__ jobs, int n_jobs,
+                                                                            int64_t total_slots, int *status,
+                                                                            unsigned long long *work) {
+    batch_refill(jobs, 0, n_jobs, total_slots, status, work);
 }
 
 // The shaft jobs [0, n_jobs) of a batch, their (group, direction) items one
@@ -403,39 +406,42 @@ extern "C" rt_status rt_batch_create(const rt_batch_job *jobs, int32_t n_jobs, i
         delete bt;
         return RT_ERR_CUDA;
     }
-    // capture: reset the queue counters, then one persistent launch for the
-    // shaft jobs and one for the others on branches of their own, so that the
-    // second fills the multiprocessors as the first one's blocks leave
-    cudaStream_t cap = nullptr, side = nullptr;
-    cudaEvent_t fork = nullptr, join = nullptr;
-    bool ok = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking) == cudaSuccess &&
-              cudaStreamCreateWithFlags(&side, cudaStreamNonBlocking) == cudaSuccess &&
-              cudaEventCreateWithFlags(&fork, cudaEventDisableTiming) == cudaSuccess &&
-              cudaEventCreateWithFlags(&join, cudaEventDisableTiming) == cudaSuccess;
+    // capture: reset the queue counters, then one persistent launch for each
+    // kind of job on a branch of its own, so that each fills the
+    // multiprocessors as the blocks of the one before leave
+    const int n_refill_jobs = n_jobs - n_shaft_jobs - n_item_jobs;
+    cudaStream_t cap[3] = {nullptr, nullptr, nullptr};
+    cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};  // fork, the joins
+    bool ok = true;
+    for (int q = 0; q < 3; ++q)
+        ok = ok && cudaStreamCreateWithFlags(&cap[q], cudaStreamNonBlocking) == cudaSuccess &&
+             cudaEventCreateWithFlags(&ev[q], cudaEventDisableTiming) == cudaSuccess;
     int *status = rt_status_ptr();
-    if (ok && (ok = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal) == cudaSuccess)) {
-        const int n_other = n_jobs - n_shaft_jobs;
-        cudaMemsetAsync(work, 0, 24, cap);
-        if (n_other > 0) {
-            cudaEventRecord(fork, cap);
-            cudaStreamWaitEvent(side, fork, 0);
-        }
+    if (ok && (ok = cudaStreamBeginCapture(cap[0], cudaStreamCaptureModeThreadLocal) == cudaSuccess)) {
+        cudaMemsetAsync(work, 0, 24, cap[0]);
+        cudaEventRecord(ev[0], cap[0]);
         if (n_shaft_jobs > 0)
-            k_shaft_batch<<<persistent_grid((const void *)k_shaft_batch), 128, 0, cap>>>(dtab, n_shaft_jobs, shafts,
-                                                                                         status, work + 2);
-        if (n_other > 0) {
-            k_trace_batch<<<persistent_grid((const void *)k_trace_batch), 128, 0, side>>>(
-                dtab + n_shaft_jobs, n_item_jobs, n_other, items, slots, status, work);
-            cudaEventRecord(join, side);
-            cudaStreamWaitEvent(cap, join, 0);
+            k_shaft_batch<<<persistent_grid((const void *)k_shaft_batch), 128, 0, cap[0]>>>(dtab, n_shaft_jobs, shafts,
+                                                                                            status, work + 2);
+        for (int q = 1; q < 3; ++q) {
+            if ((q == 1 ? n_item_jobs : n_refill_jobs) == 0) continue;
+            cudaStreamWaitEvent(cap[q], ev[0], 0);
+            if (q == 1)
+                k_trace_batch<<<persistent_grid((const void *)k_trace_batch), 128, 0, cap[q]>>>(
+                    dtab + n_shaft_jobs, n_item_jobs, items, status, work);
+            else
+                k_refill_batch<<<persistent_grid((const void *)k_refill_batch), 128, 0, cap[q]>>>(
+                    dtab + n_shaft_jobs + n_item_jobs, n_refill_jobs, slots, status, work + 1);
+            cudaEventRecord(ev[q], cap[q]);
+            cudaStreamWaitEvent(cap[0], ev[q], 0);
         }
-        ok = cudaStreamEndCapture(cap, &bt->graph) == cudaSuccess;
+        ok = cudaStreamEndCapture(cap[0], &bt->graph) == cudaSuccess;
     }
     if (ok) ok = cudaGraphInstantiate(&bt->exec, bt->graph, 0) == cudaSuccess;
-    if (fork) cudaEventDestroy(fork);
-    if (join) cudaEventDestroy(join);
-    if (side) cudaStreamDestroy(side);
-    if (cap) cudaStreamDestroy(cap);
+    for (int q = 0; q < 3; ++q) {
+        if (ev[q]) cudaEventDestroy(ev[q]);
+        if (cap[q]) cudaStreamDestroy(cap[q]);
+    }
     if (!ok) {
         cudaGetLastError();
         if (bt->exec) cudaGraphExecDestroy(bt->exec);

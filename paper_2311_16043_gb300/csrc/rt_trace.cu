@@ -23,15 +23,15 @@
 namespace {
 
 template <int STRAT, bool COUNT>
-__global__ void __launch_bounds__(128, RT_TRACE_MIN_BLOCKS) k_trace(BvhDev b, RaySetDev rs, TraceJob job, float *T_out,
-                                               TraceAux aux, unsigned long long *work) {
+__global__ void __launch_bounds__(128, STRAT == 5 ? RT_REFILL_MIN_BLOCKS : RT_TRACE_MIN_BLOCKS)
+    k_trace(BvhDev b, RaySetDev rs, TraceJob job, float *T_out, TraceAux aux, unsigned long long *work) {
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     __shared__ int2 stk_all[STRAT == 2 ? 4 * RT_WIDE_STACK : 1];
     int2 *stk = stk_all + (STRAT == 2 ? (threadIdx.x >> 5) * RT_WIDE_STACK : 0);
     WorkCounts wc = {0, 0, 0};
     unsigned long long rays_done = 0;
-    if (STRAT == 5) {  // per-ray slots with lane refill (full implicit sets)
+    if constexpr (STRAT == 5) {  // per-ray slots with lane refill (full implicit sets)
         trace_refill<COUNT>(b, rs, job, T_out, aux, work, wc, rays_done);
         flush_counts<COUNT>(aux, wc, rays_done);
         return;

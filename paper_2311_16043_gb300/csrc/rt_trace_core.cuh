@@ -201,9 +201,10 @@ __device__ __forceinline__ void cswap_near(float &ta, uint32_t &qa, float &tb, u
 // them in the same order.  The order decides only how soon the walk stops
 // once T < T_min: the accepted set and the factors are the same.
 // Returns false (nothing pushed) if the stack would overflow.
+// put(i, ref) stores entry i of the stack.
+template <class Put>
 __device__ __forceinline__ bool visit_order(float t0, float t1, float t2, float t3, uint32_t r0, uint32_t r1,
-                                            uint32_t r2, uint32_t r3, bool far, uint32_t *stack, int &sp,
-                                            int &next) {
+                                            uint32_t r2, uint32_t r3, bool far, Put put, int &sp, int &next) {
     const float inf = __int_as_float(0x7f800000);
     if (far) {
         t0 = t0 < inf ? -t0 : inf;
@@ -219,9 +220,9 @@ __device__ __forceinline__ bool visit_order(float t0, float t1, float t2, float 
     next = t0 < inf ? (int)r0 : -1;
     const int n = (t1 < inf) + (t2 < inf) + (t3 < inf);
     if (sp + n > RT_WIDE_STACK) return false;
-    if (t3 < inf) stack[sp++] = r3;
-    if (t2 < inf) stack[sp++] = r2;
-    if (t1 < inf) stack[sp++] = r1;
+    if (t3 < inf) put(sp++, r3);
+    if (t2 < inf) put(sp++, r2);
+    if (t1 < inf) put(sp++, r1);
     return true;
 }
 
@@ -632,7 +633,8 @@ __device__ __forceinline__ void trace_ray_wide_run(const BvhDev &b, float3 o, fl
             }
         }
         int next = -1;
-        const bool overflow = !visit_order(ti[0], ti[1], ti[2], ti[3], r[0], r[1], r[2], r[3], far, stack, sp, next);
+        const bool overflow = !visit_order(ti[0], ti[1], ti[2], ti[3], r[0], r[1], r[2], r[3], far,
+                                           [&](int at, uint32_t ref) { stack[at] = ref; }, sp, next);
         if (overflow) {
             rt_set_error(status, RT_ERR_STACK_OVERFLOW);
             break;
@@ -826,18 +828,40 @@ __device__ __forceinline__ void flush_counts(const TraceAux &aux, const WorkCoun
 // 2009).  Rays are the slots item*32 + l of a full implicit set (in the job's
 // item order); whenever at least kRefillMin lanes of the warp are idle, lane
 // 0 takes that many slots with one atomic and the idle lanes start them, so a
-// warp no longer waits for its longest ray.  Each step of a lane is one node
-// visit.  Slots past a ragged last tile are skipped.  `work` counts slots.
-// Nodes are the 64-byte ones: with the 128-byte nodes the L1 data pipe was 91 %
-// busy (a wavefront per lane and 32-byte load, 76 nodes and 71 Gaussians a ray);
-// hemisphere set of the 300k object scene x 64 44.9 -> 35.9 ms, 200k
-// environment set x 64 28.7 -> 23.2, 600k shadow rays (strategy 6) 2.02 -> 1.65.
+// warp no longer waits for its longest ray.  Slots past a ragged last tile are
+// skipped.  `work` counts slots.
+// A step of a lane is one node visit, which puts the leaves met into a queue of
+// the lane's own (first in first out, so a ray's factors come in the order of
+// its walk whatever its neighbours do); the Gaussians are evaluated, one per
+// lane, once kLeafMin lanes have one waiting: in the visit itself each of the
+// four children had a branch with 6 of 32 lanes busy.
+// Bound: the L1 data pipe (0.8 of it; a wavefront per lane and 32-byte load, 78
+// nodes and 71 Gaussians a ray, hit rate 0.2), then issue (0.65).  Measured on
+// the way, ms for the 300k object scene's hemisphere set x 64, the 200k's
+// environment set x 64 and a uniform 200k's x 16:
+//   128-byte nodes                                44.9   28.7   17.7
+//   64-byte nodes (qnode_near)                    35.9   23.2   14.1
+//   leaf queue, 16 lanes waiting (8: 32.9)        31.0   20.2   12.5
+//   refill from 6 idle lanes instead of 8         30.7   20.2   12.3
+//   lower stack entries shared, 9 blocks for 8    29.3   19.3   11.8
 // The quantized boxes cost 1.5 % more nodes and Gaussians, the nodes 64 bytes a
 // Gaussian and 4 us of the build at 4k, 13 at 300k.
+#ifndef RT_REFILL_MIN_BLOCKS
+#define RT_REFILL_MIN_BLOCKS 9
+#endif
 #ifndef RT_REFILL_MIN
-#define RT_REFILL_MIN 8
+#define RT_REFILL_MIN 6
 #endif
 constexpr int kRefillMin = RT_REFILL_MIN;
+#ifndef RT_LEAF_MIN
+#define RT_LEAF_MIN 16
+#endif
+constexpr int kLeafMin = RT_LEAF_MIN;
+constexpr int kLeafQueue = 8;
+#ifndef RT_STACK_SHARED
+#define RT_STACK_SHARED 24
+#endif
+constexpr int kStackShared = RT_STACK_SHARED;
 
 // `Src` is what the rays come from: slots(), fetch(slot, o, d, src) (false past
 // a ragged last tile; remembers where the slot's T goes), tree(), far() and
@@ -853,9 +877,19 @@ __device__ __forceinline__ void refill_walk(Src &from, int *status, unsigned lon
     float3 o = make_float3(0.f, 0.f, 0.f), d = make_float3(0.f, 0.f, 1.f), inv = d, oi = o;
     int32_t src = -1;
     float T = 1.0f;
-    uint32_t node = 0;
+    int32_t node = -1;  // the next to visit, -1: none left
     int sp = 0;
-    uint32_t stack[RT_WIDE_STACK];
+    // by lane, in shared memory: leaves met, first in first out, and the lower
+    // entries of the stack
+    __shared__ int32_t shared[kLeafQueue + kStackShared][128];
+    int32_t *const queue = &shared[0][threadIdx.x], *const low = &shared[kLeafQueue][threadIdx.x];
+    uint32_t high[RT_WIDE_STACK - kStackShared];
+    auto put = [&](int at, uint32_t ref) {
+        if (at < kStackShared) low[at * 128] = (int32_t)ref;
+        else high[at - kStackShared] = ref;
+    };
+    auto get = [&](int at) { return at < kStackShared ? low[at * 128] : (int32_t)high[at - kStackShared]; };
+    int qh = 0, qn = 0;
     for (;;) {
         const unsigned idle = __ballot_sync(FULL, !has);
         const int n_idle = __popc(idle);
@@ -869,8 +903,9 @@ __device__ __forceinline__ void refill_walk(Src &from, int *status, unsigned lon
                 if (slot < total && from.fetch(slot, o, d, src)) {
                     has = qnode_ray(o, d, inv, oi);
                     T = 1.0f;
-                    node = 0;
+                    node = has ? 0 : -1;
                     sp = 0;
+                    qn = 0;
                     if (!has) {
                         from.store(1.0f);
                         rays_done++;
@@ -882,39 +917,48 @@ __device__ __forceinline__ void refill_walk(Src &from, int *status, unsigned lon
             if (exhausted) break;
             continue;
         }
-        if (!has) continue;
         const BvhDev &b = from.tree();
-        float tn[4];
-        uint32_t r[4];
-        qnode_near(b.qwide + 4 * (int64_t)node, inv, oi, tn, r);
-        if (COUNT) wc.box += (r[0] != RT_EMPTY) + (r[1] != RT_EMPTY) + (r[2] != RT_EMPTY) + (r[3] != RT_EMPTY);
-        const float inf = __int_as_float(0x7f800000);
-        float ti[4];
+        if (node >= 0 && qn <= kLeafQueue - 4) {
+            float tn[4];
+            uint32_t r[4];
+            qnode_near(b.qwide + 4 * (int64_t)node, inv, oi, tn, r);
+            if (COUNT) wc.box += (r[0] != RT_EMPTY) + (r[1] != RT_EMPTY) + (r[2] != RT_EMPTY) + (r[3] != RT_EMPTY);
+            const float inf = __int_as_float(0x7f800000);
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            ti[c] = inf;
-            if (!(tn[c] < inf)) continue;
-            if (r[c] & RT_LEAF_BIT) {
-                const int32_t p = (int32_t)(r[c] & ~RT_LEAF_BIT);
-                if (p != src) {
-                    if (COUNT) wc.gauss++;
-                    if (gauss_hit(b, p, o, d, T) && COUNT) wc.hits++;
+            for (int c = 0; c < 4; ++c) {
+                if (tn[c] < inf && (r[c] & RT_LEAF_BIT)) {
+                    const int32_t p = (int32_t)(r[c] & ~RT_LEAF_BIT);
+                    tn[c] = inf;
+                    if (p != src) {
+                        queue[((qh + qn) & (kLeafQueue - 1)) * 128] = p;
+                        ++qn;
+                    }
                 }
-            } else {
-                ti[c] = tn[c];
+            }
+            int next = -1;
+            if (!visit_order(tn[0], tn[1], tn[2], tn[3], r[0], r[1], r[2], r[3], from.far(), put, sp, next)) {
+                rt_set_error(status, RT_ERR_STACK_OVERFLOW);
+                sp = 0;
+                next = -1;
+            }
+            node = next >= 0 ? next : sp > 0 ? get(--sp) : -1;
+        }
+        for (;;) {
+            const unsigned pend = __ballot_sync(FULL, qn > 0), walk = __ballot_sync(FULL, node >= 0 && qn <= kLeafQueue - 4);
+            if (pend == 0 || (__popc(pend) < kLeafMin && walk != 0)) break;
+            if (qn > 0) {
+                const int32_t p = queue[qh * 128];
+                qh = (qh + 1) & (kLeafQueue - 1);
+                --qn;
+                if (COUNT) wc.gauss++;
+                if (gauss_hit(b, p, o, d, T) && COUNT) wc.hits++;
+                if (T < b.t_min) {
+                    node = -1;
+                    qn = 0;
+                }
             }
         }
-        int next = -1;
-        const bool overflow =
-            !visit_order(ti[0], ti[1], ti[2], ti[3], r[0], r[1], r[2], r[3], from.far(), stack, sp, next);
-        if (overflow) rt_set_error(status, RT_ERR_STACK_OVERFLOW);
-        bool done = overflow || T < b.t_min;
-        if (!done) {
-            if (next >= 0) node = (uint32_t)next;
-            else if (sp > 0) node = stack[--sp];
-            else done = true;
-        }
-        if (done) {
+        if (has && node < 0 && qn == 0) {
             from.store(T < b.t_min ? 0.0f : T);
             rays_done++;
             has = false;
