@@ -57,11 +57,12 @@ template <int LANES, bool COUNT>
 __global__ void __launch_bounds__(128, RT_TRACE_MIN_BLOCKS) k_trace_lanes(BvhDev b, RaySetDev rs, TraceJob job,
                                                                           float *T_out, TraceAux aux,
                                                                           unsigned long long *work) {
-    __shared__ uint32_t stk[128 * kLaneStack];
+    __shared__ uint32_t stk[128 * kLaneStack<LANES>];
+    __shared__ int32_t queue[kLeafQueue * 128];
     WorkCounts wc = {0, 0, 0};
     unsigned long long rays_done = 0;
-    trace_lane_group<LANES, COUNT>(b, rs, job, T_out, aux, work, stk + threadIdx.x / LANES * (LANES * kLaneStack), wc,
-                                   rays_done);
+    trace_lane_group<LANES, COUNT>(b, rs, job, T_out, aux, work, stk + threadIdx.x / LANES * (LANES * kLaneStack<LANES>),
+                                   queue + threadIdx.x, wc, rays_done);
     flush_counts<COUNT>(aux, wc, rays_done);
 }
 
@@ -120,12 +121,18 @@ int persistent_blocks(const void *kernel, int threads) {
 
 // Lanes per ray for a list of m rays (a fallback list: the most it can be).
 // 300k object scene, shadow rays in no order, us with 32 / 16 / 8 / 4
-// lanes: 2,000 rays 53 / 70 / 105 / 167; 20,000 147 / 141 / 168 / 231; 100,000
-// 555 / 439 / 416 / 439; 600,000 3,102 / 2,329 / 2,031 / 1,889; 1M rays of the
-// 2M scene 10,230 / 8,868 / 8,778 / 8,900.
+// lanes: 2,000 rays 50 / 69 / 101 / 176; 20,000 122 / 122 / 154 / 230; 100,000
+// 433 / 368 / 325 / 361; 250,000 1,019 / 836 / 683 / 667; 600,000 2,384 /
+// 1,929 / 1,491 / 1,322.  Beyond 2^20 Gaussians nodes and records exceed the L2
+// cache and more lanes hide its misses: 1M rays of the 2M scene 6,138 / 5,724 /
+// 5,302 / 6,443.  4 lanes' stack holds a walk of single nodes through 36 levels.
 // A full set keeps 32, so that a ray of it and of a short id list get the same
 // T bit for bit.
-int lanes_for(bool full, int64_t m) { return full || m <= 8192 ? 32 : m <= 65536 ? 16 : m <= 262144 ? 8 : 4; }
+int lanes_for(bool full, int64_t m, const BvhDev &b) {
+    if (full || m <= 8192) return 32;
+    if (m <= 65536) return 16;
+    return m <= 262144 || b.levels > 36 || b.n > (int64_t(1) << 20) ? 8 : 4;
+}
 
 template <bool COUNT>
 void launch_lanes(int lanes, const BvhDev &b, const RaySetDev &rs, const TraceJob &job, float *T_out,
@@ -154,7 +161,7 @@ rt_status rt_trace_launch_job(const BvhDev &b, const RaySetDev &rs, const TraceJ
     if (cudaMemsetAsync(work, 0, sizeof(unsigned long long), st) != cudaSuccess) return RT_ERR_CUDA;
     const int threads = 128;
     if (strat == 6 && b.wide) {
-        launch_lanes<false>(lanes_for(job.mode == MODE_FULL, job.n_out), b, rs, job, T_out, aux, st, work);
+        launch_lanes<false>(lanes_for(job.mode == MODE_FULL, job.n_out, b), b, rs, job, T_out, aux, st, work);
     } else if (strat == 5 && b.wide && job.mode == MODE_FULL) {
         int grid = persistent_blocks((const void *)k_trace<5, false>, threads);
         k_trace<5, false><<<grid, threads, 0, st>>>(b, rs, job, T_out, aux, work);
@@ -228,7 +235,7 @@ rt_status rt_trace_launch(const rt_bvh *bvh, const rt_rayspec *rays, float *T_ou
     // - env-map and hemisphere sets (directions differ across a tile): the
     //   per-ray walk with lane refill;
     // - explicit rays and id lists (scattered rays): a group of lanes per ray
-    //   up to 2^22 rays (lanes_for; one thread per ray takes 560 us for 2,000
+    //   up to 2^22 rays (lanes_for; one thread per ray takes 570 us for 2,000
     //   rays of the 300k scene, 2.4 ms for 600,000), and one thread per ray
     //   over the 4-wide tree for longer lists, which are sorted.
     if (o.kernel == RT_KERNEL_AUTO && job.mode == MODE_FULL)
@@ -304,7 +311,7 @@ rt_status rt_trace_launch(const rt_bvh *bvh, const rt_rayspec *rays, float *T_ou
         k_trace<S, C><<<grid, threads, 0, st>>>(b, rs, job, T_out, aux, work);              \
     } while (0)
         if (strat == 6) {
-            const int lanes = lanes_for(job.mode == MODE_FULL, job.n_out);
+            const int lanes = lanes_for(job.mode == MODE_FULL, job.n_out, b);
             if (count) launch_lanes<true>(lanes, b, rs, job, T_out, aux, st, work);
             else launch_lanes<false>(lanes, b, rs, job, T_out, aux, st, work);
         }
@@ -359,11 +366,12 @@ rt_status rt_trace_launch_list(const rt_bvh *bvh, const rt_rayspec *rays, const 
     const int threads = 128;
     // the listed rays are few and scattered: a group of lanes per ray over the
     // 4-wide tree, which cuts the latency of the longest traversal
+    const BvhDev b = bvh_dev(bvh);
     if (bvh->n_wide > 0) {
-        launch_lanes<false>(lanes_for(!rays->ray_ids, max_count), bvh_dev(bvh), rs, job, T_out, aux, st, work);
+        launch_lanes<false>(lanes_for(!rays->ray_ids, max_count, b), b, rs, job, T_out, aux, st, work);
     } else {
         int grid = persistent_blocks((const void *)k_trace<0, false>, threads);
-        k_trace<0, false><<<grid, threads, 0, st>>>(bvh_dev(bvh), rs, job, T_out, aux, work);
+        k_trace<0, false><<<grid, threads, 0, st>>>(b, rs, job, T_out, aux, work);
     }
     return rt_check_launch();
 }

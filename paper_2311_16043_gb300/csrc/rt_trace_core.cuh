@@ -686,6 +686,33 @@ __device__ __forceinline__ void full_item(const TraceJob &job, int32_t K, int64_
 }
 
 
+// The ray of slot `slot` of a full implicit set: false past a ragged last tile.
+__device__ __forceinline__ bool slot_ray(const BvhDev &b, const RaySetDev &rs, const TraceJob &job, int64_t slot,
+                                         float3 &o, float3 &d, int32_t &src, int64_t &out_idx) {
+    int64_t tile;
+    int32_t k;
+    full_item(job, rs.K, slot >> 5, tile, k);
+    const int64_t p = tile * 32 + (slot & 31);
+    if (p >= b.n) return false;
+    const float4 mu = __ldg(b.gauss + 4 * p);
+    const int64_t g = __float_as_int(__ldg(b.gauss + 4 * p + 1).w);
+    out_idx = g * rs.K + k;
+    implicit_ray(rs, out_idx, k, g, mu, o, d);
+    src = (int32_t)p;
+    return true;
+}
+
+// Slots of a job: rays of a full implicit set (those past a ragged last tile
+// included) or entries of a list.
+__device__ __forceinline__ int64_t job_slots(const TraceJob &job) {
+    int64_t n = job.mode == MODE_FULL ? job.n_items * 32 : job.n_out;
+    if (job.dyn_count) {
+        const int64_t c = (int64_t)*job.dyn_count;
+        n = c < n ? c : n;
+    }
+    return n;
+}
+
 // Ray r of a job in slot order: MODE_FULL slot r (item r/32, lane r%32;
 // false past a ragged last tile, out_idx = -1), MODE_EXPLICIT / MODE_IDS
 // entry r (an invalid id records RT_ERR_INVALID_ARG and returns false with
@@ -696,19 +723,7 @@ __device__ __forceinline__ bool ray_of(const BvhDev &b, const RaySetDev &rs, con
     out_idx = -1;
     o = make_float3(0.f, 0.f, 0.f);
     d = make_float3(0.f, 0.f, 1.f);
-    if (job.mode == MODE_FULL) {
-        int64_t tile;
-        int32_t k;
-        full_item(job, rs.K, r >> 5, tile, k);
-        const int64_t p = tile * 32 + (r & 31);
-        if (p >= b.n) return false;
-        const float4 mu = __ldg(b.gauss + 4 * p);
-        const int64_t g = __float_as_int(__ldg(b.gauss + 4 * p + 1).w);
-        out_idx = g * rs.K + k;
-        implicit_ray(rs, out_idx, k, g, mu, o, d);
-        src = (int32_t)p;
-        return true;
-    }
+    if (job.mode == MODE_FULL) return slot_ray(b, rs, job, r, o, d, src, out_idx);
     out_idx = job.out_index ? job.out_index[r] : r;
     if (job.mode == MODE_EXPLICIT) {
         o = make_float3(rs.ray_o[3 * r], rs.ray_o[3 * r + 1], rs.ray_o[3 * r + 2]);
@@ -966,22 +981,6 @@ __device__ __forceinline__ void refill_walk(Src &from, int *status, unsigned lon
     }
 }
 
-// The ray of slot `slot` of a full implicit set: false past a ragged last tile.
-__device__ __forceinline__ bool slot_ray(const BvhDev &b, const RaySetDev &rs, const TraceJob &job, int64_t slot,
-                                         float3 &o, float3 &d, int32_t &src, int64_t &out_idx) {
-    int64_t tile;
-    int32_t k;
-    full_item(job, rs.K, slot >> 5, tile, k);
-    const int64_t p = tile * 32 + (slot & 31);
-    if (p >= b.n) return false;
-    const float4 mu = __ldg(b.gauss + 4 * p);
-    const int64_t g = __float_as_int(__ldg(b.gauss + 4 * p + 1).w);
-    out_idx = g * rs.K + k;
-    implicit_ray(rs, out_idx, k, g, mu, o, d);
-    src = (int32_t)p;
-    return true;
-}
-
 template <bool COUNT>
 __device__ __forceinline__ void trace_refill(const BvhDev &b, const RaySetDev &rs, const TraceJob &job, float *T_out,
                                              const TraceAux &aux, unsigned long long *work, WorkCounts &wc,
@@ -1003,41 +1002,48 @@ __device__ __forceinline__ void trace_refill(const BvhDev &b, const RaySetDev &r
     refill_walk<COUNT>(from, aux.status, work, wc, rays_done);
 }
 
-// Strategy 6: LANES (4, 8, 16 or 32) lanes per ray over the 4-wide tree, for
-// scattered rays (fallback lists, explicit rays).  The lanes take up to that many
-// entries off the top of the ray's stack in shared memory, visit those nodes
-// in parallel, multiply the factors of their leaf hits into lane-local partial
-// products and push the hit internal children; T is the product of the
-// partials, formed by a butterfly after every step for the early exit.  A
-// step takes as many entries as keep 3 places free per level of the tree, and
-// one where that is not possible: one at a time the walk is depth first and
-// grows the stack by 3 a level at most (RT_ERR_STACK_OVERFLOW for a tree too
-// deep even for that).  Same accepted
-// set as the per-ray traversals; the product is formed in another order.  A
-// group of lanes fetches its next ray as soon as it is done.  `work` counts
-// rays (slots of a full implicit set).  A ray's walk has few nodes at a time:
-// with all 32 lanes on it most idle, with few lanes a single ray takes longer
-// (lanes_for, rt_trace.cu).
-constexpr int kLaneStack = 64;  // entries per lane: >= 3 x 64 levels for 4 lanes
+// Strategy 6: LANES (4, 8, 16 or 32) lanes per ray over the 64-byte nodes, for
+// scattered rays (fallback lists, explicit rays).  The lanes take up to that
+// many entries off the top of the ray's stack in shared memory, visit those
+// nodes in parallel and push the hit internal children; leaves met go to a
+// queue per lane and are evaluated as in refill_walk, into lane-local partial
+// products.  T is their product, formed by a butterfly after every step for
+// the early exit.  A step takes as many entries as keep 3 places free per level
+// of the tree, and one where that is not possible: one at a time the walk is
+// depth first and grows the stack by 3 a level at most (RT_ERR_STACK_OVERFLOW
+// for a tree too deep even for that).  Same accepted set as the per-ray
+// traversals; the product is formed in another order, which the ray and LANES
+// alone decide.  A group of lanes fetches its next ray as soon as it is done.
+// `work` counts slots.  A ray's walk has few nodes at a time: with all 32 lanes
+// on it most idle, with few lanes a single ray takes longer (lanes_for,
+// rt_trace.cu).
+// Bound: issue (0.53) and memory latency at 30 warps an SM, then the L1 data
+// pipe (0.50).  600k shadow rays of the 300k object scene: 32 lanes 3.00 ms, 4
+// lanes 2.02, 64-byte nodes 1.65, leaf queue (12 lanes waiting) 1.38, stacks of
+// 144 entries instead of 256 (more warps, and an L1 that holds something: hit
+// rate 0.02 before) 1.32; 1M rays of the 2M scene 7.9 -> 6.4 by the last alone.
+#ifndef RT_LANE_LEAF_MIN
+#define RT_LANE_LEAF_MIN 10
+#endif
+constexpr int kLaneLeafMin = RT_LANE_LEAF_MIN;
+template <int LANES>
+constexpr int kLaneStack = LANES == 4 ? 36 : LANES == 8 ? 28 : LANES == 16 ? 18 : 12;  // entries per lane
 template <int LANES, bool COUNT>
 __device__ __forceinline__ void trace_lane_group(const BvhDev &b, const RaySetDev &rs, const TraceJob &job,
                                                  float *T_out, const TraceAux &aux, unsigned long long *work,
-                                                 uint32_t *stk, WorkCounts &wc, unsigned long long &rays_done) {
+                                                 uint32_t *stk, int32_t *queue, WorkCounts &wc,
+                                                 unsigned long long &rays_done) {
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31, sub = lane & (LANES - 1);
     const unsigned group = (LANES == 32 ? FULL : ((1u << LANES) - 1u) << (lane - sub));
-    int64_t n_out = job.mode == MODE_FULL ? job.n_items * 32 : job.n_out;  // slots
-    if (job.dyn_count) {
-        const int64_t c = (int64_t)*job.dyn_count;
-        n_out = c < n_out ? c : n_out;
-    }
-    const int room = kLaneStack * LANES - 4 - 3 * b.levels;
+    const int64_t n_out = job_slots(job);
+    const int room = kLaneStack<LANES> * LANES - 4 - 3 * b.levels;
     bool has = false, more = true;
     float3 o = make_float3(0.f, 0.f, 0.f), d = make_float3(0.f, 0.f, 1.f), inv = d, oi = o;
     int32_t src = -1;
     int64_t out_idx = 0;
     float Tl = 1.0f;
-    int size = 0;
+    int size = 0, qh = 0, qn = 0;
     for (;;) {
         if (!has && more) {
             unsigned long long item = 0;
@@ -1050,7 +1056,7 @@ __device__ __forceinline__ void trace_lane_group(const BvhDev &b, const RaySetDe
             } else {
                 has = qnode_ray(o, d, inv, oi);
                 Tl = 1.0f;
-                size = 1;
+                size = has ? 1 : 0;
                 if (sub == 0) {
                     stk[0] = 0u;
                     if (!has) {
@@ -1063,7 +1069,9 @@ __device__ __forceinline__ void trace_lane_group(const BvhDev &b, const RaySetDe
         if (!__any_sync(FULL, has || more)) break;
         __syncwarp();
         // one step: entries off the top, their nodes' children
-        const int k = has ? min(min(LANES, size), max(1, (room - size) / 3)) : 0;
+        const unsigned held = __ballot_sync(FULL, qn > kLeafQueue - 4);
+        const bool step = size > 0 && (held & group) == 0u;
+        const int k = step ? min(min(LANES, size), max(1, (room - size) / 3)) : 0;
         const uint32_t node = sub < k ? stk[size - 1 - sub] : 0u;
         size -= k;
         __syncwarp();
@@ -1075,27 +1083,19 @@ __device__ __forceinline__ void trace_lane_group(const BvhDev &b, const RaySetDe
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
                 if (!(tn[c] < __int_as_float(0x7f800000))) continue;
-                if (r[c] & RT_LEAF_BIT) {
-                    const int32_t p = (int32_t)(r[c] & ~RT_LEAF_BIT);
-                    if (p != src) {
-                        if (COUNT) wc.gauss++;
-                        if (gauss_hit(b, p, o, d, Tl) && COUNT) wc.hits++;
-                    }
-                } else {
-                    pm |= 1u << c;
-                }
+                const int32_t p = (int32_t)(r[c] & ~RT_LEAF_BIT);
+                if (!(r[c] & RT_LEAF_BIT)) pm |= 1u << c;
+                else if (p != src) queue[((qh + qn++) & (kLeafQueue - 1)) * 128] = p;
             }
         }
         __syncwarp();
         // prefix sum of the pushes over the group, then write them above the top
         const int n_push = __popc(pm);
         int pre = n_push;
-        float T = Tl;
 #pragma unroll
         for (int off = 1; off < LANES; off <<= 1) {
             const int v = __shfl_up_sync(FULL, pre, off, LANES);
             if (sub >= off) pre += v;
-            T *= __shfl_xor_sync(FULL, T, off);
         }
         const int total = __shfl_sync(FULL, pre, LANES - 1, LANES);
         int at = size + pre - n_push;
@@ -1103,8 +1103,26 @@ __device__ __forceinline__ void trace_lane_group(const BvhDev &b, const RaySetDe
         for (int c = 0; c < 4; ++c)
             if ((pm >> c) & 1u) stk[at++] = r[c];
         size += total;
-        const bool full = size > kLaneStack * LANES - 4;  // no place for another node's children
-        if (has && (full || T < b.t_min || size == 0)) {
+        // Gaussians, one per lane, while enough lanes have one or no group can step
+        unsigned pend;
+        for (;;) {
+            pend = __ballot_sync(FULL, qn > 0);
+            const unsigned over = __ballot_sync(FULL, qn > kLeafQueue - 4);
+            const bool any_step = __any_sync(FULL, size > 0 && (over & group) == 0u) != 0;
+            if (pend == 0u || (__popc(pend) < kLaneLeafMin && any_step)) break;
+            if (qn > 0) {
+                const int32_t p = queue[qh * 128];
+                qh = (qh + 1) & (kLeafQueue - 1);
+                --qn;
+                if (COUNT) wc.gauss++;
+                if (gauss_hit(b, p, o, d, Tl) && COUNT) wc.hits++;
+            }
+        }
+        float T = Tl;
+#pragma unroll
+        for (int off = 1; off < LANES; off <<= 1) T *= __shfl_xor_sync(FULL, T, off);
+        const bool full = size > kLaneStack<LANES> * LANES - 4;  // no place for another node's children
+        if (has && (full || T < b.t_min || (size == 0 && (pend & group) == 0u))) {
             if (full) rt_set_error(aux.status, RT_ERR_STACK_OVERFLOW);
             if (sub == 0) {
                 T_out[out_idx] = T < b.t_min ? 0.0f : T;
@@ -1112,6 +1130,7 @@ __device__ __forceinline__ void trace_lane_group(const BvhDev &b, const RaySetDe
             }
             has = false;
             size = 0;
+            qn = 0;
         }
         __syncwarp();
     }
