@@ -5,9 +5,10 @@
 // direction sweep a narrow shaft.  One warp walks the tree for the whole
 // shaft; its lanes are split over what each step has most of:
 //   1. nodes: up to 16 nodes at a time come off a shared stack, two lanes
-//      per node test its boxes against the shaft: the ray from the centre of
-//      the origins' box against boxes grown by that box's half extents (the
-//      Minkowski sum, exact for parallel rays).  Leaves met go to a list.
+//      per 64-byte node test its boxes against the shaft: the ray from the
+//      centre of the origins' box against boxes grown by that box's half
+//      extents (the Minkowski sum, exact for parallel rays).  Leaves met go to
+//      a list.
 //   2. Gaussians: 64 leaves at a time, two per lane (packed FMAs).  A lane
 //      reduces its Gaussians to what is left of them along d: a whitened 2D
 //      offset v = (r11 x + r12 y + c1, r22 y + c2) of the ray through (x, y)
@@ -27,13 +28,15 @@
 // 182k warp instructions per 32 rays of the 2M-Gaussian object scene (307 per
 // node visit, of which a ray needs half); this takes ~28k, 0.7 of them in
 // steps 1 and 3.  Measured, trace only, against that walk (2M x 64
-// directions: 751 -> 127 ms, 1.0 G rays/s) and the per-ray walk (300k x 128:
-// 96 -> 28 ms, 1.36 G rays/s).  Bound: instruction issue (0.7 of the slots;
+// directions: 751 -> 125 ms, 1.0 G rays/s) and the per-ray walk (300k x 128:
+// 96 -> 26.5 ms, 1.45 G rays/s).  Bound: instruction issue (0.7 of the slots;
 // the rest fixed-latency dependences), with shared memory at 0.65 of its
 // wavefronts; DRAM 0.1 %.  Choices measured on the way (300k / 2M scenes):
-//   - records and nodes staged by 4 and 8 lanes each with 16-byte async
-//     copies: with a 16-byte load per lane and row the kernel was bound by L1
-//     tag lookups (91 %);
+//   - records staged by 4 lanes each with 16-byte async copies: with a 16-byte
+//     load per lane and row the kernel was bound by L1 tag lookups (91 %);
+//   - 64-byte nodes in two 32-byte loads a lane instead of 128-byte ones staged
+//     like the records: 4 to 6 % (300k x 32 7.07 -> 6.68 ms, 50k x 32 875 -> 825
+//     us); one lane per node, 32 a step: 50k 946 us;
 //   - pairs evaluated from a list: with each ray walking its own mask, 9 of
 //     32 lanes were busy; writing the list from the voting lanes instead of
 //     the rays' masks was 10 % slower;
@@ -50,6 +53,7 @@
 constexpr int kShaftRays = 64;      // rays of a group at most
 constexpr int kShaftCands = 64;     // Gaussians of a batch
 constexpr int kShaftNodes = 16;     // nodes of a step
+constexpr int kShaftLeaves = 128;   // leaves met: fewer than a batch left over and a step's
 constexpr int kShaftStack = 320;    // nodes; a walk of single nodes adds 3 per level at most (193 for 64 levels)
 template <bool GRAD>
 constexpr int kShaftPairs = GRAD ? 160 : 256;
@@ -57,7 +61,7 @@ constexpr int kShaftPairs = GRAD ? 160 : 256;
 // The adjoint (GRAD) keeps a record per pair, (dL/dm^2, u) with u = S^-1 R^T e.
 template <bool GRAD>
 struct __align__(16) ShaftSmem {
-    float4 stage[4 * kShaftCands];            // the batch's records, or a step's nodes
+    float4 stage[4 * kShaftCands];            // the batch's records
     float4 ro[kShaftRays];                    // by ray: origin, T (GRAD: by slot: origin, dL/dT T)
     typename std::conditional<GRAD, float4, uint32_t>::type pair[kShaftPairs<GRAD>];  // ray << 6 | Gaussian,
                                               //   then the pair's factor (GRAD: record)
@@ -66,7 +70,7 @@ struct __align__(16) ShaftSmem {
     uint2 mask[kShaftRays];                   // by slot: Gaussians of the batch to evaluate
     float4 fr[5];                             // the shaft's frame (see shaft_cand)
     uint32_t stack[kShaftStack];
-    uint32_t leaf[kShaftCands + 4 * kShaftNodes];  // fewer than a batch left over + one step's
+    uint32_t leaf[kShaftLeaves];
     uint8_t live[kShaftRays];                 // by slot: ray
     uint8_t from[GRAD ? kShaftRays : 1];      // GRAD: by slot: its first pair
 };
@@ -109,14 +113,32 @@ __device__ __forceinline__ float2 dot2(f2x3 a, float4 b) {
     return __ffma2_rn(a.x, dup(b.x), __ffma2_rn(a.y, dup(b.y), __fmul2_rn(a.z, dup(b.z))));
 }
 
-// A box test of shaft_group: planes ordered along the direction, the near
-// planes moved towards the rays by the origins' half extents and the far
-// planes away (cn, cf = c inv +- hh |inv|); otherwise as slab().
-__device__ __forceinline__ bool shaft_slab(float nx, float fx, float ny, float fy, float nz, float fz, float3 inv,
-                                           float3 cn, float3 cf) {
-    const float n = fmaxf(fmaxf(fmaf(nx, inv.x, -cn.x), fmaf(ny, inv.y, -cn.y)), fmaxf(fmaf(nz, inv.z, -cn.z), 0.0f));
-    const float f = fminf(fminf(fmaf(fx, inv.x, -cf.x), fmaf(fy, inv.y, -cf.y)), fmaf(fz, inv.z, -cf.z));
-    return n <= fmaf(fabsf(f), 1e-6f, f);
+// Children 2 h and 2 h + 1 of a 64-byte node against a shaft (see qnode_near):
+// the near planes moved towards the rays by the origins' half extents and the
+// far planes away (cn, cf = c inv +- hh |inv|).
+__device__ __forceinline__ void shaft_qnode(const float4 *__restrict__ q, int h, float3 inv, float3 cn, float3 cf,
+                                            bool &h0, bool &h1, uint32_t &r0, uint32_t &r1) {
+    const float4x2 n0 = ldg_pair(q), n1 = ldg_pair(q + 2);
+    const float ax = n0.a.w * inv.x, ay = n0.b.x * inv.y, az = n0.b.y * inv.z;
+    const float nx = fmaf(n0.a.x, inv.x, -cn.x), ny = fmaf(n0.a.y, inv.y, -cn.y), nz = fmaf(n0.a.z, inv.z, -cn.z);
+    const float fx = fmaf(n0.a.x, inv.x, -cf.x), fy = fmaf(n0.a.y, inv.y, -cf.y), fz = fmaf(n0.a.z, inv.z, -cf.z);
+    const bool sx = inv.x < 0.0f, sy = inv.y < 0.0f, sz = inv.z < 0.0f;
+    const uint32_t lx = __float_as_uint(n0.b.z), hx = __float_as_uint(n0.b.w), ly = __float_as_uint(n1.a.x),
+                   hy = __float_as_uint(n1.a.y), lz = __float_as_uint(n1.a.z), hz = __float_as_uint(n1.a.w);
+    r0 = __float_as_uint(h ? n1.b.z : n1.b.x);
+    r1 = __float_as_uint(h ? n1.b.w : n1.b.y);
+    const uint32_t s0 = h ? 0x7624u : 0x7604u, s1 = s0 + 0x10u;
+    auto dist = [&](uint32_t w, float a, float c) {
+        const float2 k = make_float2(__uint_as_float(__byte_perm(w, 0x3f800000u, s0)),
+                                     __uint_as_float(__byte_perm(w, 0x3f800000u, s1)));
+        return __ffma2_rn(k, make_float2(a, a), make_float2(c, c));
+    };
+    const float2 x0 = dist(sx ? hx : lx, ax, nx), x1 = dist(sx ? lx : hx, ax, fx), y0 = dist(sy ? hy : ly, ay, ny),
+                 y1 = dist(sy ? ly : hy, ay, fy), z0 = dist(sz ? hz : lz, az, nz), z1 = dist(sz ? lz : hz, az, fz);
+    const float na = fmaxf(fmaxf(x0.x, y0.x), fmaxf(z0.x, 0.0f)), fa = fminf(fminf(x1.x, y1.x), z1.x);
+    const float nb = fmaxf(fmaxf(x0.y, y0.y), fmaxf(z0.y, 0.0f)), fb = fminf(fminf(x1.y, y1.y), z1.y);
+    h0 = !(na > fmaf(fabsf(fa), 1e-6f, fa)) && r0 != RT_EMPTY;
+    h1 = !(nb > fmaf(fabsf(fb), 1e-6f, fb)) && r1 != RT_EMPTY;
 }
 
 // Two Gaussians as the rays of a shaft see them (step 2).
@@ -242,7 +264,8 @@ __device__ __forceinline__ void shaft_group(const BvhDev &b, float eps, float3 d
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
     const float inf = __int_as_float(0x7f800000);
-    const float3 inv = safe_inv(d);
+    float3 inv, oi;
+    const bool finite = qnode_ray(make_float3(0.f, 0.f, 0.f), d, inv, oi);
     int live = count;
     if constexpr (GRAD) live = 0;
 #pragma unroll
@@ -312,41 +335,21 @@ __device__ __forceinline__ void shaft_group(const BvhDev &b, float eps, float3 d
             sm.stack[0] = 0u;
         }
     }
-    // step 1: this lane's half node (node lane / 2 of the step): 16-byte row
-    // r of staged node i lies at chunk r ^ (i & 7); rows of the near planes
-    const char *base = reinterpret_cast<const char *>(sm.stage) + 128 * (lane >> 1) + 8 * (lane & 1);
-    const uint32_t swz = (uint32_t)((lane >> 1) & 7);
-    const uint32_t nx = ((inv.x < 0.0f ? 1u : 0u) ^ swz) << 4, ny = ((inv.y < 0.0f ? 3u : 2u) ^ swz) << 4,
-                   nz = ((inv.z < 0.0f ? 5u : 4u) ^ swz) << 4;
-    auto row = [&](uint32_t off) { return *reinterpret_cast<const float2 *>(base + off); };
     // step 2: 16-byte row r of staged record i lies at chunk r ^ ((i >> 1) & 3)
     auto rec = [&](int i, int r) { return sm.stage[4 * i + (r ^ ((i >> 1) & 3))]; };
     const int room = kShaftStack - 4 - 3 * b.levels;  // beyond it, nodes are walked one at a time
-    int bound = live, size = 1, nleaf = 0;
+    int bound = live, size = finite ? 1 : 0, nleaf = 0;  // a direction that is not finite meets nothing
     (void)bound;
     __syncwarp();
     for (;;) {
         while (nleaf < kShaftCands && size > 0) {
-            const int k = min(min(kShaftNodes, size), max(1, (room - size) / 3));
+            const int k = min(min(kShaftNodes, size), min(max(1, (room - size) / 3), (kShaftLeaves - nleaf) / 4));
             size -= k;
-#pragma unroll
-            for (int t = 0; t < kShaftNodes / 4; ++t) {
-                const int i = 4 * t + (lane >> 3);
-                if (i < k)
-                    cp_async16(sm.stage + 8 * i + ((lane ^ i) & 7), b.wide + 8 * (int64_t)sm.stack[size + i] + (lane & 7));
-            }
-            cp_async_done();
+            const uint32_t node = (lane >> 1) < k ? sm.stack[size + (lane >> 1)] : 0u;
             __syncwarp();
             bool h0 = false, h1 = false;
             uint32_t r0 = 0u, r1 = 0u;
-            if ((lane >> 1) < k) {
-                const float2 ax = row(nx), bx = row(nx ^ 16u), ay = row(ny), by = row(ny ^ 16u), az = row(nz),
-                             bz = row(nz ^ 16u), rf = row((6u ^ swz) << 4);
-                h0 = shaft_slab(ax.x, bx.x, ay.x, by.x, az.x, bz.x, inv, cn, cf);
-                h1 = shaft_slab(ax.y, bx.y, ay.y, by.y, az.y, bz.y, inv, cn, cf);
-                r0 = __float_as_uint(rf.x);
-                r1 = __float_as_uint(rf.y);
-            }
+            if ((lane >> 1) < k) shaft_qnode(b.qwide + 4 * (int64_t)node, lane & 1, inv, cn, cf, h0, h1, r0, r1);
             const bool f0 = h0 && (int)r0 < 0, f1 = h1 && (int)r1 < 0;
             h0 = h0 && !f0;
             h1 = h1 && !f1;

@@ -114,3 +114,12 @@ def test_overflowing_inverse_scales(n):
     sc["scale"] = sc["scale"].copy()
     sc["scale"][::3] = 1e-20
     _check(sc, scenes.fibonacci_sphere(11))
+
+
+def test_directions_that_are_not_finite():
+    sc = scenes.uniform_scene(700, 8)
+    dirs = scenes.fibonacci_sphere(6)
+    dirs[1, 0], dirs[3], dirs[4, 2] = np.nan, 0.0, np.inf
+    a, b = (_trace(sc, dirs, k)[0] for k in (1, 3))
+    np.testing.assert_allclose(b, a, rtol=RTOL, atol=0)
+    assert (b[:, [1, 3, 4]] == 1).all()
