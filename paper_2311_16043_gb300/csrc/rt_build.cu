@@ -5,7 +5,7 @@
 // Steps (all kernels below, one stream, one synchronisation at the end):
 //   k_bounds       input check and per-axis min/max of the means
 //   k_morton       30-bit Morton codes, float32 IEEE quantisation (no FMA)
-//   k_sort_small   up to 4096 codes: the whole radix sort in one block
+//   k_sort_small   both for up to 12288 Gaussians, by counting
 //   k_radix_*      stable LSD radix sort of (code, index), 8-bit digits, 4 passes
 //   k_prep         permutation, inverse permutation, 64-bit keys code<<32|index,
 //                  per-Gaussian record (mean, opacity, whitening W = S^-1 R^T)
@@ -105,9 +105,24 @@ __device__ __forceinline__ uint32_t spread10(uint32_t v) {
 
 // Quantisation with separately rounded float32 operations:
 // u = (mu - lo) / (hi - lo), q = clamp(floor(u * 1024), 0, 1023); 0 if hi == lo.
-__global__ void k_morton(const float *__restrict__ mean, int64_t n, const uint32_t *scn,
-                         float *bounds_out, uint32_t *codes, int32_t *vals) {
-    float lo[3], ext[3];
+__device__ __forceinline__ uint32_t morton_code(const float *__restrict__ m, const float (&lo)[3], const float (&ext)[3]) {
+    uint32_t q[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        if (ext[c] == 0.0f) {
+            q[c] = 0;
+            continue;
+        }
+        float u = __fdiv_rn(__fsub_rn(m[c], lo[c]), ext[c]);
+        float v = __fmul_rn(u, 1024.0f);
+        int qi = (int)floorf(v);
+        qi = qi < 0 ? 0 : (qi > 1023 ? 1023 : qi);
+        q[c] = (uint32_t)qi;
+    }
+    return (spread10(q[0]) << 2) | (spread10(q[1]) << 1) | spread10(q[2]);
+}
+// The scene's bounds from the scene words; one thread writes them out.
+__device__ __forceinline__ void scene_bounds(const uint32_t *scn, float *bounds_out, float (&lo)[3], float (&ext)[3]) {
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
         lo[c] = scene_lo(scn, c);
@@ -118,22 +133,14 @@ __global__ void k_morton(const float *__restrict__ mean, int64_t n, const uint32
             bounds_out[3 + c] = hi;
         }
     }
+}
+__global__ void k_morton(const float *__restrict__ mean, int64_t n, const uint32_t *scn,
+                         float *bounds_out, uint32_t *codes, int32_t *vals) {
+    float lo[3], ext[3];
+    scene_bounds(scn, bounds_out, lo, ext);
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
-        uint32_t q[3];
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            if (ext[c] == 0.0f) {
-                q[c] = 0;
-                continue;
-            }
-            float u = __fdiv_rn(__fsub_rn(mean[3 * i + c], lo[c]), ext[c]);
-            float v = __fmul_rn(u, 1024.0f);
-            int qi = (int)floorf(v);
-            qi = qi < 0 ? 0 : (qi > 1023 ? 1023 : qi);
-            q[c] = (uint32_t)qi;
-        }
-        codes[i] = (spread10(q[0]) << 2) | (spread10(q[1]) << 1) | spread10(q[2]);
+        codes[i] = morton_code(mean + 3 * i, lo, ext);
         vals[i] = (int32_t)i;
     }
 }
@@ -276,89 +283,38 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_scatter(
 }
 static_assert(kSortThreads == kRadix, "one digit a thread");
 
-// The radix sort of up to 4096 codes in one block, in place: 32 warps rank
-// 128 consecutive keys each, the keys change places in shared memory.
-constexpr int kSmallSort = 4096;
-__global__ void __launch_bounds__(1024) k_sort_small(uint32_t *keys, int32_t *vals, int n) {
-    constexpr int ITEMS = kSmallSort / 1024;
-    __shared__ uint16_t wcnt16[32][kRadix];
-    __shared__ uint32_t sk[kSmallSort];
-    __shared__ uint16_t sv[kSmallSort];
-    __shared__ uint32_t ws[32];
-    const int t = threadIdx.x, w = t >> 5, lane = t & 31, base = w * (32 * ITEMS) + lane;
-    const uint32_t lt_mask = (1u << lane) - 1u;
-    uint32_t key[ITEMS], val[ITEMS], rank[ITEMS];
-#pragma unroll
-    for (int it = 0; it < ITEMS; ++it) {
-        const int i = base + 32 * it;
-        key[it] = i < n ? keys[i] : 0xffffffffu;  // padding stays behind every 30-bit code
-        val[it] = (uint32_t)i;
+// Morton codes of a small scene in sorted order (ties by index) without a sort:
+// every block forms all codes in shared memory, and the place of one is how
+// many are smaller, or equal with a smaller index; a warp counts for each.
+// n^2 compares, but no chain: four radix passes in one block took 26 us at
+// 4096 Gaussians, and k_morton before them 4 us more; this 10 us (18 with 8
+// threads a code, which form 16 codes each one after the other).
+// Builds of 8192 Gaussians take 112 us so and 154 with the radix sort, of 12288
+// (48 KB of codes) 149 and 157.
+constexpr int kSmallSort = 12288;
+__global__ void __launch_bounds__(1024) k_sort_small(const float *__restrict__ mean, int n, const uint32_t *scn,
+                                                     float *bounds_out, uint32_t *codes, int32_t *vals) {
+    __shared__ uint4 sk4[kSmallSort / 4];
+    uint32_t *sk = reinterpret_cast<uint32_t *>(sk4);
+    float lo[3], ext[3];
+    scene_bounds(scn, bounds_out, lo, ext);
+    const int padded = (n + 127) / 128 * 128;
+#pragma unroll 4
+    for (int i = threadIdx.x; i < padded; i += 1024) sk[i] = i < n ? morton_code(mean + 3 * i, lo, ext) : 0xffffffffu;
+    __syncthreads();
+    const int e = blockIdx.x * 32 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    const uint32_t key = sk[e];
+    int cnt = 0;
+#pragma unroll 4
+    for (int j = lane; j < padded / 4; j += 32) {
+        const uint4 v = sk4[j];
+        const int d = e - 4 * j;  // the first d of the four have a smaller index
+        cnt += (v.x < key + (d > 0)) + (v.y < key + (d > 1)) + (v.z < key + (d > 2)) + (v.w < key + (d > 3));
     }
-    for (int shift = 0; shift < 32; shift += kRadixBits) {
-        for (int j = t; j < 32 * kRadix / 2; j += 1024) reinterpret_cast<uint32_t *>(&wcnt16[0][0])[j] = 0;
-        __syncthreads();
-#pragma unroll
-        for (int it = 0; it < ITEMS; ++it) {
-            const uint32_t d = (key[it] >> shift) & (kRadix - 1), peers = __match_any_sync(0xffffffffu, d);
-            const uint32_t r = __popc(peers & lt_mask), c = wcnt16[w][d];
-            __syncwarp();
-            if (r == 0) wcnt16[w][d] = (uint16_t)(c + __popc(peers));
-            __syncwarp();
-            rank[it] = c + r;
-        }
-        __syncthreads();
-        // exclusive prefix over (digit, warp): thread t takes digit t / 4, warps 8 (t % 4) ...
-        uint32_t v[8], sum = 0;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            v[k] = wcnt16[8 * (t & 3) + k][t >> 2];
-            sum += v[k];
-        }
-        uint32_t inc = sum;
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const uint32_t u = __shfl_up_sync(0xffffffffu, inc, off);
-            if (lane >= off) inc += u;
-        }
-        if (lane == 31) ws[w] = inc;
-        __syncthreads();
-        if (w == 0) {
-            uint32_t x = ws[lane];
-#pragma unroll
-            for (int off = 1; off < 32; off <<= 1) {
-                const uint32_t u = __shfl_up_sync(0xffffffffu, x, off);
-                if (lane >= off) x += u;
-            }
-            ws[lane] = x - ws[lane];
-        }
-        __syncthreads();
-        uint32_t run = ws[w] + inc - sum;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            wcnt16[8 * (t & 3) + k][t >> 2] = (uint16_t)run;  // below 4096
-            run += v[k];
-        }
-        __syncthreads();
-#pragma unroll
-        for (int it = 0; it < ITEMS; ++it) {
-            const uint32_t pos = wcnt16[w][(key[it] >> shift) & (kRadix - 1)] + rank[it];
-            sk[pos] = key[it];
-            sv[pos] = (uint16_t)val[it];
-        }
-        __syncthreads();
-#pragma unroll
-        for (int it = 0; it < ITEMS; ++it) {
-            key[it] = sk[base + 32 * it];
-            val[it] = sv[base + 32 * it];
-        }
-    }
-#pragma unroll
-    for (int it = 0; it < ITEMS; ++it) {
-        const int i = base + 32 * it;
-        if (i < n) {
-            keys[i] = key[it];
-            vals[i] = (int32_t)val[it];
-        }
+    cnt = __reduce_add_sync(0xffffffffu, cnt);
+    if (lane == 0 && e < n) {
+        codes[cnt] = key;
+        vals[cnt] = e;
     }
 }
 
@@ -632,12 +588,32 @@ __device__ __forceinline__ void store_child_box(float4 *nodes, int32_t node, boo
 // costs a fraction of the atomic through L2 and what orders it.  The counts
 // carry the first arrival's height (count in the low 8 bits), so the root's
 // height comes out for free: the levels of the tree.
+// Up to 4096 leaves (CLUSTER) all blocks form one cluster, and the nodes that
+// straddle blocks are in the shared memory of the block their index lies in:
+// 4096 leaves 23.4 us through L2, 15.3 so.
 __device__ __forceinline__ uint32_t atomic_add_acq_rel(uint32_t *p, uint32_t v) {
     uint32_t old;
     asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
     return old;
 }
+// Thread-block clusters: a barrier of all blocks, the address of `p` in block
+// `rank`'s shared memory, and a counter there.
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
+}
+template <class T>
+__device__ __forceinline__ T *cluster_map(T *p, int rank) {
+    uint64_t a;
+    asm volatile("mapa.u64 %0, %1, %2;" : "=l"(a) : "l"((uint64_t)p), "r"(rank));
+    return reinterpret_cast<T *>(a);
+}
+__device__ __forceinline__ uint32_t atomic_add_acq_rel_cluster(uint32_t *p, uint32_t v) {
+    uint32_t old;
+    asm volatile("atom.acq_rel.cluster.add.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
+    return old;
+}
 constexpr int kRefitLeaves = 512;
+template <bool CLUSTER>
 __global__ void __launch_bounds__(kRefitLeaves) k_refit(const float *__restrict__ leafbox,
                                                         const int32_t *__restrict__ parent, int64_t n, float4 *nodes,
                                                         uint32_t *arrivals, uint32_t *levels) {
@@ -646,7 +622,10 @@ __global__ void __launch_bounds__(kRefitLeaves) k_refit(const float *__restrict_
     __shared__ int32_t par[kRefitLeaves];
     __shared__ uint32_t cnt[kRefitLeaves];
     const int t = threadIdx.x;
-    for (int64_t b0 = (int64_t)blockIdx.x * kRefitLeaves; b0 < n; b0 += (int64_t)gridDim.x * kRefitLeaves) {
+    // the grid has no block beyond the leaves, a cluster may: those go round once
+    // too, for its barriers
+    int64_t b0 = (int64_t)blockIdx.x * kRefitLeaves;
+    do {
         const int64_t p = b0 + t, b1 = b0 + kRefitLeaves < n ? b0 + kRefitLeaves : n;
         const float4 none = make_float4(0.f, 0.f, __int_as_float(-1), __int_as_float(0x7fffffff));
         ref[t] = p < n - 1 ? __ldcg(nodes + 4 * p + 3) : none;
@@ -660,6 +639,7 @@ __global__ void __launch_bounds__(kRefitLeaves) k_refit(const float *__restrict_
             node = parent[(n - 1) + p];
         }
         uint32_t child = RT_LEAF_BIT | (uint32_t)p, height = 0u;
+        if constexpr (CLUSTER) cluster_sync();  // every block's slots are ready
         auto local = [&](const float4 &r) { return __float_as_int(r.z) >= b0 && __float_as_int(r.w) < b1; };
         __syncthreads();
         while (node >= 0 && node >= b0 && node < b1) {
@@ -690,24 +670,51 @@ __global__ void __launch_bounds__(kRefitLeaves) k_refit(const float *__restrict_
             if (node == 0) *levels = height;
             node = par[q];
         }
-        while (node >= 0) {
-            const float4 r = __ldcg(nodes + 4 * (int64_t)node + 3);
-            store_child_box(nodes, node, __float_as_uint(r.x) != child, b);
-            const uint32_t old = atomic_add_acq_rel(&arrivals[node], 1u + (height << 8));
-            if (old == 0u) break;
-            height = max(height, old >> 8) + 1u;
-            const float4 *nd = nodes + 4 * (int64_t)node;
-            const float4 x = __ldcg(nd), y = __ldcg(nd + 1), z = __ldcg(nd + 2);
-            // slots: (L.lo.x, L.hi.x, L.lo.y, L.hi.y, L.lo.z, L.hi.z, R.lo.x, ...)
-            b[0] = fminf(x.x, y.z); b[3] = fmaxf(x.y, y.w);
-            b[1] = fminf(x.z, z.x); b[4] = fmaxf(x.w, z.y);
-            b[2] = fminf(y.x, z.z); b[5] = fmaxf(y.y, z.w);
-            child = (uint32_t)node;
-            if (node == 0) *levels = height;
-            node = parent[node];
+        if constexpr (CLUSTER) {
+            while (node >= 0) {
+                const int own = (int)(node / kRefitLeaves), q = (int)(node % kRefitLeaves);
+                const float4 r = *cluster_map(&ref[q], own);
+                const int up = *cluster_map(&par[q], own);
+                float *x = cluster_map(&box[q][0], own), *nd = x + (__float_as_uint(r.x) != child ? 6 : 0);
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    nd[2 * c] = b[c];
+                    nd[2 * c + 1] = b[3 + c];
+                }
+                const uint32_t old = atomic_add_acq_rel_cluster(cluster_map(&cnt[q], own), 1u + (height << 8));
+                if (old == 0u) break;
+                height = max(height, old >> 8) + 1u;
+                const volatile float *l = x;
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    b[c] = fminf(l[2 * c], l[6 + 2 * c]);
+                    b[3 + c] = fmaxf(l[2 * c + 1], l[7 + 2 * c]);
+                }
+                child = (uint32_t)node;
+                if (node == 0) *levels = height;
+                node = up;
+            }
+            cluster_sync();  // no block leaves while another may reach into it
+        } else {
+            while (node >= 0) {
+                const float4 r = __ldcg(nodes + 4 * (int64_t)node + 3);
+                store_child_box(nodes, node, __float_as_uint(r.x) != child, b);
+                const uint32_t old = atomic_add_acq_rel(&arrivals[node], 1u + (height << 8));
+                if (old == 0u) break;
+                height = max(height, old >> 8) + 1u;
+                const float4 *nd = nodes + 4 * (int64_t)node;
+                const float4 x = __ldcg(nd), y = __ldcg(nd + 1), z = __ldcg(nd + 2);
+                // slots: (L.lo.x, L.hi.x, L.lo.y, L.hi.y, L.lo.z, L.hi.z, R.lo.x, ...)
+                b[0] = fminf(x.x, y.z); b[3] = fmaxf(x.y, y.w);
+                b[1] = fminf(x.z, z.x); b[4] = fmaxf(x.w, z.y);
+                b[2] = fminf(y.x, z.z); b[5] = fmaxf(y.y, z.w);
+                child = (uint32_t)node;
+                if (node == 0) *levels = height;
+                node = parent[node];
+            }
         }
         __syncthreads();
-        if (p < n - 1 && local(ref[t])) {
+        if (p < n - 1 && (CLUSTER || local(ref[t]))) {
             const float *l = box[t];
             float4 *nd = nodes + 4 * p;
             nd[0] = make_float4(l[0], l[1], l[2], l[3]);
@@ -715,7 +722,8 @@ __global__ void __launch_bounds__(kRefitLeaves) k_refit(const float *__restrict_
             nd[2] = make_float4(l[8], l[9], l[10], l[11]);
         }
         __syncthreads();
-    }
+        b0 += (int64_t)gridDim.x * kRefitLeaves;
+    } while (!CLUSTER && b0 < n);
 }
 
 // Surface area of a box stored (lo.x, hi.x, lo.y, hi.y, lo.z, hi.z); -1 for NaN.
@@ -960,6 +968,28 @@ int refit_grid(int64_t n) {
     return (int)(g < 1 ? 1 : g < cap ? g : cap);
 }
 
+void launch_refit(const float *leafbox, const int32_t *parent, int64_t n, float4 *nodes, uint32_t *arrivals,
+                  uint32_t *levels, cudaStream_t st) {
+    if (n > 8 * kRefitLeaves) {
+        k_refit<false><<<refit_grid(n), kRefitLeaves, 0, st>>>(leafbox, parent, n, nodes, arrivals, levels);
+        return;
+    }
+    int blocks = 1;  // a power of two: every cluster size of up to 8 is portable
+    while (blocks * kRefitLeaves < n) blocks *= 2;
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3(kRefitLeaves);
+    cfg.stream = st;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = (unsigned)blocks;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, k_refit<true>, leafbox, parent, n, nodes, arrivals, levels);  // rt_check_launch reports
+}
+
 float host_ord2f(uint32_t u) {
     u = (u & 0x80000000u) ? (u & 0x7fffffffu) : ~u;
     float f;
@@ -1083,9 +1113,12 @@ extern "C" rt_status rt_build_bvh(const float *mean, const float *scale, const f
     if (cudaMemsetAsync(scn, 0, SCN_BYTES, st) != cudaSuccess) result = RT_ERR_CUDA;
     if (result == RT_OK) {
         k_bounds<<<bounds_grid(n), 512, 0, st>>>(mean, scale, quat, opacity, n, scn);
-        k_morton<<<grid_for(n, 256), 256, 0, st>>>(mean, n, scn, b->bounds, k0, v0);
-        if (small) k_sort_small<<<1, 1024, 0, st>>>(k0, v0, (int)n);
-        else radix_sort(k0, v0, k1, v1, n, 4, counts, st);
+        if (small) {
+            k_sort_small<<<((int)n + 31) / 32, 1024, 0, st>>>(mean, (int)n, scn, b->bounds, k0, v0);
+        } else {
+            k_morton<<<grid_for(n, 256), 256, 0, st>>>(mean, n, scn, b->bounds, k0, v0);
+            radix_sort(k0, v0, k1, v1, n, 4, counts, st);
+        }
         k_prep<<<grid_for(n, 128), 128, 0, st>>>(mean, scale, quat, opacity, v0, k0, n, prm, scn, b->gauss, leafbox,
                                                  b->perm, b->rank, b->keys);
         const int kb = grid_for(ni, 128), gb = grid_for((n + 63) / 64, 4);
@@ -1094,7 +1127,7 @@ extern "C" rt_status rt_build_bvh(const float *mean, const float *scale, const f
         if (n == 1) {
             if (cudaMemsetAsync(b->parent, 0xff, sizeof(int32_t), st) != cudaSuccess) result = RT_ERR_CUDA;  // -1
         } else {
-            k_refit<<<refit_grid(n), kRefitLeaves, 0, st>>>(leafbox, b->parent, n, b->nodes, arrivals, scn + SCN_LEVELS);
+            launch_refit(leafbox, b->parent, n, b->nodes, arrivals, scn + SCN_LEVELS, st);
             k_wide<<<grid_for(ni, 128), 128, 0, st>>>(b->nodes, ni, b->wide, b->qwide);
             b->n_wide = ni;
         }
@@ -1151,7 +1184,7 @@ extern "C" rt_status rt_bvh_refit(rt_bvh *b, const float *mean, const float *sca
                 result = RT_ERR_CUDA;
                 break;
             }
-            k_refit<<<refit_grid(n), kRefitLeaves, 0, st>>>(leafbox, b->parent, n, b->nodes, arrivals, scn + SCN_LEVELS);
+            launch_refit(leafbox, b->parent, n, b->nodes, arrivals, scn + SCN_LEVELS, st);
         }
         if (b->n_wide > 0)
             k_refit_wide<<<grid_for(4 * ni, 256), 256, 0, st>>>(leafbox, b->nodes, ni, (float *)b->wide,
