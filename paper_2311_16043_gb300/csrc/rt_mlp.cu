@@ -544,11 +544,16 @@ __global__ void __launch_bounds__(128 * INF_WG, 1) k_mlp_infer(MlpDev net, Sampl
 // dX3 and (if another tile follows) W1 -> B0 after dX2; the next tile then
 // finds W1 in B0 and W2 in B1.  Warpgroup 3, which has neither encoding nor
 // dW1 work, draws the next tile's samples into a second sample buffer: the
-// ids while warpgroups 0-2 encode (the sorted position and the target then
-// arrive by asynchronous copies), the mean's copies after its last forward
-// epilogue and the rays while warpgroups 0-2 add the dW1 tile, four MMA
-// phases apart, so the two rounds of dependent global loads do not stall
-// the tile.
+// ids at the top of the tile (the sorted position and the target then arrive
+// by asynchronous copies), the mean's copies after its last forward epilogue
+// and the rays in the last backward epilogue, so the two rounds of dependent
+// global loads do not stall the tile; warpgroups 0-2 encode them while the
+// dW1 products run.
+// Bound: the chain of MMA, TMEM load, epilogue and barrier, eight a tile (0.2 of
+// the tensor pipe, 0.28 of the issue slots; shared memory holds one tile).
+// 262,144 samples: 197 us with dW before dX in one commit and the encoding at
+// the top of the tile, 193.5 with the epilogue of dX over the dW products,
+// 182 with the encoding under the dW1 products too; the same bits.
 constexpr int TR_THREADS = 512;
 constexpr int TR_PSTRIDE = 60040;                // floats per partial (NPARAM + 1 rounded up to 8)
 constexpr int TR_WB0 = 0;                        // 32768: weight buffer 0
@@ -629,9 +634,8 @@ __device__ __forceinline__ void encode_scalar(float xh, float xl, float *f) {
 // product's column 78 becomes the sum over samples of dz1, the gradient of
 // the layer-1 bias; the B operand of the other layers' bias-gradient
 // products is this tile's columns 64..79.
-__device__ __forceinline__ void encode_part(uint8_t *x0, int r, int q, bool valid, float3 p, float3 d,
-                                            const MlpDev &net) {
-    if (q > 2) return;
+__device__ __forceinline__ void encode_part(int q, bool valid, float3 p, float3 d, const MlpDev &net,
+                                            uint32_t (&u)[13]) {
     float xh[2] = {0.0f, 0.0f}, xl[2] = {0.0f, 0.0f};
     if (valid) {
 #pragma unroll
@@ -659,8 +663,11 @@ __device__ __forceinline__ void encode_part(uint8_t *x0, int r, int q, bool vali
         for (int k = 0; k < 26; ++k) f[k] = 0.0f;
     }
 #pragma unroll
-    for (int k = 0; k < 13; ++k)
-        *reinterpret_cast<uint32_t *>(x0 + img_off(r, 26 * q + 2 * k, IN)) = pack_bf16(f[2 * k], f[2 * k + 1]);
+    for (int k = 0; k < 13; ++k) u[k] = pack_bf16(f[2 * k], f[2 * k + 1]);
+}
+__device__ __forceinline__ void store_part(uint8_t *x0, int r, int q, const uint32_t (&u)[13]) {
+#pragma unroll
+    for (int k = 0; k < 13; ++k) *reinterpret_cast<uint32_t *>(x0 + img_off(r, 26 * q + 2 * k, IN)) = u[k];
     if (q == 2) *reinterpret_cast<uint32_t *>(x0 + img_off(r, IN_FEAT, IN)) = 0x3f80u;  // bf16 (1, 0)
 }
 
@@ -693,6 +700,7 @@ __global__ void __launch_bounds__(TR_THREADS, 1) k_mlp_train(MlpDev net, SampleS
     uint64_t *bar = reinterpret_cast<uint64_t *>(smem + TR_BAR);  // MMA commits
     uint64_t *wbar = bar + 1;                                      // [2] weight copies; bar[3]: drain
     uint32_t *tslot = reinterpret_cast<uint32_t *>(smem + TR_BAR + 32);
+    uint64_t *bar_dw = reinterpret_cast<uint64_t *>(smem + TR_BAR + 40);  // commits of the dW products
     float *smp = reinterpret_cast<float *>(smem + TR_SMP);  // [2][7][128]
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
     const int r = t & 127, q = t >> 7, c0 = 32 * q;
@@ -719,6 +727,7 @@ __global__ void __launch_bounds__(TR_THREADS, 1) k_mlp_train(MlpDev net, SampleS
         mbar_init(wbar, 1);
         mbar_init(wbar + 1, 1);
         mbar_init(bar + 3, 1);
+        mbar_init(bar_dw, 1);
     }
     if (warp == 0) tmem_alloc(tslot, 512);
     fence_async_smem();
@@ -739,9 +748,8 @@ __global__ void __launch_bounds__(TR_THREADS, 1) k_mlp_train(MlpDev net, SampleS
     const uint32_t id_dw1 = tc_idesc_bf16(128, IN, true, true);
     const uint32_t id_dx = tc_idesc_bf16(128, 128, false, true);
     const uint32_t id_db = tc_idesc_bf16(128, 16, true, true);
-    uint32_t phase = 0;
+    uint32_t phase = 0, phase_dw = 0;
     bool ok = true;
-
 
     // weight copies (thread 0 only): bit b of `pend` / `wph` is buffer b's
     // pending flag / phase
@@ -834,10 +842,15 @@ __global__ void __launch_bounds__(TR_THREADS, 1) k_mlp_train(MlpDev net, SampleS
         }
     }
     __syncthreads();
-    if (q < 3) {  // the first tile's encoding (the loop encodes the others)
-        const float *smr = smp + r;
-        encode_part(x0, r, q, smr[768] >= 0.0f, make_float3(smr[0], smr[128], smr[256]),
-                    make_float3(smr[384], smr[512], smr[640]), net);
+    // row r's features (warpgroups 0-2) of the tile in sample buffer b
+    uint32_t feat[13];
+    auto encode_row = [&](int b) {
+        const float *o = smp + b * 7 * 128 + r;
+        encode_part(q, o[768] >= 0.0f, make_float3(o[0], o[128], o[256]), make_float3(o[384], o[512], o[640]), net, feat);
+    };
+    if (q < 3) {  // the first tile's encoding (each tile's last phase encodes the next)
+        encode_row(0);
+        store_part(x0, r, q, feat);
     }
     grid_dependency_wait();
     if (t < 128) {
@@ -879,13 +892,8 @@ __global__ void __launch_bounds__(TR_THREADS, 1) k_mlp_train(MlpDev net, SampleS
         const float *smr = smp + sb * 7 * 128 + r;
         const float y = smr[768];
         const bool valid = y >= 0.0f;
-        if (q < 3) {
-            if (!first)
-                encode_part(x0, r, q, valid, make_float3(smr[0], smr[128], smr[256]),
-                            make_float3(smr[384], smr[512], smr[640]), net);
-        } else if (ahead) {
-            draw_ids(more ? tile + 1 : t0, sb ^ 1, more ? S.step : S.step + 1);  // completed in the dW1 phase
-        }
+        // completed in the backward pass
+        if (q == 3 && ahead) draw_ids(more ? tile + 1 : t0, sb ^ 1, more ? S.step : S.step + 1);
         // ---- forward: layer l reads x_l (x0, h1, h2, h3) and W_{l+1} ----
         float h4[32];
 #pragma unroll
@@ -977,13 +985,17 @@ __global__ void __launch_bounds__(TR_THREADS, 1) k_mlp_train(MlpDev net, SampleS
                 need_w(b);
                 if (wok) {
                     const uint32_t s_dzl = l == 3 ? s_dz : s_h(l);
-                    // dW_{l+1} += dz^T x_l : A = dz (MN-major), B = h_l (MN-major), K = samples
-                    issue_mma(tm_dw(l - 1), s_dzl, 2048, 128, 4096, s_h(l - 1), 2048, 128, 4096, id_dw, 128,
-                              !first);
                     // dX_l = dz W_{l+1} : A = dz (K-major), B = W (MN-major), K = units
                     issue_mma(tm_work, s_dzl, 128, 2048, 256, s_wb(b), 2048, 128, 4096, id_dx, 128, false);
                 }
                 tc_commit(bar);
+                if (wok) {
+                    // dW_{l+1} += dz^T x_l : A = dz (MN-major), B = h_l (MN-major), K = samples;
+                    // runs under the epilogue of dX_l until that overwrites h_l
+                    issue_mma(tm_dw(l - 1), l == 3 ? s_dz : s_h(l), 2048, 128, 4096, s_h(l - 1), 2048, 128, 4096, id_dw,
+                              128, !first);
+                }
+                tc_commit(bar_dw);
             }
             wait_mma();
             if (t == 0) {
@@ -1002,6 +1014,9 @@ __global__ void __launch_bounds__(TR_THREADS, 1) k_mlp_train(MlpDev net, SampleS
             load_chunk_raw(hl, r, c0, hp);
 #pragma unroll
             for (int k = 0; k < 16; ++k) hp[k] = pack_bf16(v[2 * k], v[2 * k + 1]) & bf16x2_pos_mask(hp[k]);
+            if (l == 1 && q == 3 && ahead) draw_ray(sb ^ 1);  // the next tile's rays
+            if (!mbar_wait(bar_dw, phase_dw, net.wait_cycles)) ok = false;  // h_l has been read
+            phase_dw ^= 1u;
             store_chunk_raw(hl, r, c0, hp);
         }
         // ---- dW1 = dz1^T x0 (per tile, added to this CTA's partial) and the
@@ -1018,7 +1033,9 @@ __global__ void __launch_bounds__(TR_THREADS, 1) k_mlp_train(MlpDev net, SampleS
             issue_mma(tm_work + 112, s_h(1), 2048, 128, 4096, s_x0 + 1024, 1280, 128, 2560, id_db, 128, false);
             tc_commit(bar);
         }
+        if (q < 3 && more) encode_row(sb ^ 1);  // the next tile, under the MMAs that still read this one
         wait_mma();
+        if (q < 3 && more) store_part(x0, r, q, feat);
         // fire-and-forget vector adds (stores for the first tile): each
         // address of this CTA's partial is only ever written by this thread,
         // in tile order, so the sums are deterministic; warpgroup 3 has no
@@ -1050,7 +1067,6 @@ __global__ void __launch_bounds__(TR_THREADS, 1) k_mlp_train(MlpDev net, SampleS
                 misc[1] += (misc[8] + misc[9]) + (misc[10] + misc[11]);
                 misc[0] += (misc[12] + misc[13]) + (misc[14] + misc[15]);
             }
-            if (ahead) draw_ray(sb ^ 1);  // the next tile's rays, read after its first barrier
         }
         tc_fence_before();
         // the end-of-tile barrier doubles as the vote
