@@ -242,9 +242,13 @@ rt_status rt_materialize_rays(const rt_bvh *bvh, const rt_rayspec *rays, const i
 /* ------------------------------------------------------------------------ */
 
 typedef enum {
-    RT_KERNEL_AUTO = 0,   /* DIRS sets: WIDE where neighbouring Gaussians lie
-                             close together (measured on the tree), else
-                             RAY_WIDE; ENV and HEMI sets: RAY_REFILL; explicit
+    RT_KERNEL_AUTO = 0,   /* small full sets (DIRS up to 2^15 rays, ENV and
+                             HEMI up to 2^20, few per Gaussian): lanes by the
+                             number of rays as in WARP_RAY's lists; DIRS sets:
+                             WIDE where neighbouring Gaussians lie close
+                             together (measured on the tree), else RAY_WIDE;
+                             ENV and HEMI sets: RAY_WIDE up to 2^19 rays,
+                             RAY_REFILL beyond; explicit
                              rays and id lists: WARP_RAY up to 2^22 rays
                              (RAY_WIDE with a hit log), RAY_WIDE beyond (an id
                              list traced in the tree's order); the binary

@@ -126,6 +126,14 @@ __device__ __forceinline__ float4x2 ldg_pair(const float4 *p) {
         : "l"(p));
     return r;
 }
+// The same, not kept in L1.
+__device__ __forceinline__ float4x2 ldg_pair_once(const float4 *p) {
+    float4x2 r;
+    asm("ld.global.nc.L1::no_allocate.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=f"(r.a.x), "=f"(r.a.y), "=f"(r.a.z), "=f"(r.a.w), "=f"(r.b.x), "=f"(r.b.y), "=f"(r.b.z), "=f"(r.b.w)
+        : "l"(p));
+    return r;
+}
 
 // Exact difference a - b = hi + lo (Knuth's TwoSum with b negated).
 __device__ __forceinline__ void two_diff(float a, float b, float &hi, float &lo) {

@@ -134,6 +134,19 @@ int lanes_for(bool full, int64_t m, const BvhDev &b) {
     return m <= 262144 || b.levels > 36 || b.n > (int64_t(1) << 20) ? 8 : 4;
 }
 
+// A full set traced by groups of lanes.  Hemisphere sets, us, lanes against the
+// better of one thread per ray and lane refill: uniform 3k x 8 52 / 152, x 32
+// 139 / 215; 30k x 8 814 / 1,497, x 32 2,786 / 3,148; object 4k x 8 57 / 81, x 16
+// 97 / 85, x 32 112 / 95; 20k x 16 310 / 309; 300k x 4 2,541 / 2,834, x 8 4,987 /
+// 4,520 (environment sets lie 5 % the other way at the ends).  Direction sets
+// against shaft packets or one thread per ray: uniform 3k x 8 52 / 80, x 32
+// 118 / 103; 30k x 1 144 / 247, x 4 398 / 258; object 4k x 8 55 / 90, x 16 94 /
+// 85; 500 x 16 26 / 26, x 64 42 / 28.
+bool small_set_takes_lanes(const rt_bvh *bvh, int32_t kind, int32_t K, int64_t rays) {
+    if (kind == RT_RAYS_DIRS) return rays <= (int64_t(1) << 15) && K <= 16;
+    return rays <= (int64_t(1) << 20) && K <= (rt_shaft_pays(bvh) ? 32 : 16);
+}
+
 template <bool COUNT>
 void launch_lanes(int lanes, const BvhDev &b, const RaySetDev &rs, const TraceJob &job, float *T_out,
                   const TraceAux &aux, cudaStream_t st, unsigned long long *work) {
@@ -226,6 +239,8 @@ rt_status rt_trace_launch(const rt_bvh *bvh, const rt_rayspec *rays, float *T_ou
               : o.kernel == RT_KERNEL_RAY_WIDE ? 4 : o.kernel == RT_KERNEL_WIDE ? 2
               : o.kernel == RT_KERNEL_PACKET ? 1 : 0;
     // AUTO:
+    // - a small full set: a group of lanes per ray (lanes_for), which is bound
+    //   by one ray's latency less than the others (small_set_takes_lanes);
     // - a direction set: shaft packets where the groups are large enough
     //   (rt_shaft_pays), else one thread per ray, farthest child first.  With
     //   counters or a hit log, which shaft packets do not keep: one thread per
@@ -233,13 +248,17 @@ rt_status rt_trace_launch(const rt_bvh *bvh, const rt_rayspec *rays, float *T_ou
     //   18 %, 300k 5 %, 500k 2.7 % in favour of the first; from 1M on the
     //   packets win);
     // - env-map and hemisphere sets (directions differ across a tile): the
-    //   per-ray walk with lane refill;
+    //   per-ray walk with lane refill, up to 2^19 rays one thread per ray, whose
+    //   latency is lower (hemisphere sets, us, thread / refill: object 4k x 64
+    //   118 / 146, 20k x 32 496 / 584, 20k x 64 840 / 814, uniform 3k x 128
+    //   439 / 432);
     // - explicit rays and id lists (scattered rays): a group of lanes per ray
     //   up to 2^22 rays (lanes_for; one thread per ray takes 570 us for 2,000
     //   rays of the 300k scene, 2.4 ms for 600,000), and one thread per ray
     //   over the 4-wide tree for longer lists, which are sorted.
     if (o.kernel == RT_KERNEL_AUTO && job.mode == MODE_FULL)
-        strat = rays->kind != RT_RAYS_DIRS ? 5
+        strat = !o.counters && !o.hit_ids && small_set_takes_lanes(bvh, rays->kind, rs.K, count) ? 6
+                : rays->kind != RT_RAYS_DIRS ? (count <= (int64_t(1) << 19) ? 4 : 5)
                 : o.counters || o.hit_ids  ? (bvh->n <= (int64_t(1) << 19) ? 4 : 2)
                 : rt_shaft_pays(bvh)       ? 2
                                            : 4;
@@ -311,7 +330,7 @@ rt_status rt_trace_launch(const rt_bvh *bvh, const rt_rayspec *rays, float *T_ou
         k_trace<S, C><<<grid, threads, 0, st>>>(b, rs, job, T_out, aux, work);              \
     } while (0)
         if (strat == 6) {
-            const int lanes = lanes_for(job.mode == MODE_FULL, job.n_out, b);
+            const int lanes = lanes_for(o.kernel == RT_KERNEL_WARP_RAY && job.mode == MODE_FULL, job.n_out, b);
             if (count) launch_lanes<true>(lanes, b, rs, job, T_out, aux, st, work);
             else launch_lanes<false>(lanes, b, rs, job, T_out, aux, st, work);
         }

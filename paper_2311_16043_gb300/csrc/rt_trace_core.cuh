@@ -151,10 +151,11 @@ __device__ __forceinline__ bool qnode_ray(float3 o, float3 d, float3 &inv, float
 // 2^15 steps are 0.004 steps, within the 0.1 that quantize_axis adds.  An axis
 // of NaN base does not count.
 // Two 32-byte loads instead of four: the walks of single rays are bound by the
-// L1 data pipe, a wavefront per lane and load.
+// L1 data pipe, a wavefront per lane and load.  Not kept in L1, which these
+// walks hit 0.2 of the time and whose fills cost the same pipe (2 to 2.5 %).
 __device__ __forceinline__ void qnode_near(const float4 *__restrict__ q, float3 inv, float3 oi, float (&tn)[4],
                                            uint32_t (&r)[4]) {
-    const float4x2 n0 = ldg_pair(q), n1 = ldg_pair(q + 2);
+    const float4x2 n0 = ldg_pair_once(q), n1 = ldg_pair_once(q + 2);
     const float ax = n0.a.w * inv.x, ay = n0.b.x * inv.y, az = n0.b.y * inv.z;
     const float cx = fmaf(n0.a.x, inv.x, -oi.x), cy = fmaf(n0.a.y, inv.y, -oi.y), cz = fmaf(n0.a.z, inv.z, -oi.z);
     const bool sx = inv.x < 0.0f, sy = inv.y < 0.0f, sz = inv.z < 0.0f;
@@ -859,6 +860,7 @@ __device__ __forceinline__ void flush_counts(const TraceAux &aux, const WorkCoun
 //   leaf queue, 16 lanes waiting (8: 32.9)        31.0   20.2   12.5
 //   refill from 6 idle lanes instead of 8         30.7   20.2   12.3
 //   lower stack entries shared, 9 blocks for 8    29.3   19.3   11.8
+//   nodes not kept in L1                          28.7   18.9   11.5
 // The quantized boxes cost 1.5 % more nodes and Gaussians, the nodes 64 bytes a
 // Gaussian and 4 us of the build at 4k, 13 at 300k.
 #ifndef RT_REFILL_MIN_BLOCKS

@@ -67,3 +67,45 @@ def test_lane_groups_without_a_tree(n, m):
     out = [rt.rt_trace_visibility(bvh, rs, opts=rt.trace_opts(kernel=k)) for k in (1, 0, 6)]
     torch.cuda.synchronize()
     assert torch.equal(out[0], out[1]) and torch.equal(out[0], out[2])
+
+
+def test_auto_list_with_hit_log():
+    """A hit log needs the one-thread-per-ray walk: AUTO takes it for a list."""
+    from paper_2311_16043_gb300 import rt
+    bvh = build(scene("spread"))
+    rng = np.random.default_rng(2)
+    m = 300
+    ro = torch.as_tensor(rng.uniform(-1, 1, (m, 3)).astype(np.float32)).cuda()
+    rd = rng.normal(size=(m, 3)).astype(np.float32)
+    rd = torch.as_tensor(rd / np.linalg.norm(rd, axis=1, keepdims=True)).cuda()
+    rs = rt.rayspec(rt.RT_RAYS_EXPLICIT, ray_o=ro, ray_d=rd)
+    out = []
+    for kernel in (4, 0):
+        ids = torch.full((m, 64), -1, dtype=torch.int32, device="cuda")
+        cnt = torch.full((m,), -1, dtype=torch.int32, device="cuda")
+        rt.rt_trace_visibility(bvh, rs, opts=rt.trace_opts(kernel=kernel, hit_ids=ids, hit_count=cnt))
+        torch.cuda.synchronize()
+        out.append((ids, cnt))
+    assert int(out[0][1].min()) >= 0
+    assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
+
+
+@pytest.mark.parametrize("n,K", [(3000, 1), (3000, 10), (3000, 16), (3000, 17), (3000, 32), (3000, 33), (500, 16), (500, 17)])
+@pytest.mark.parametrize("kind", ["dirs", "hemi"])
+def test_auto_small_sets(kind, n, K):
+    """Full sets around the sizes where AUTO leaves the lane groups."""
+    from paper_2311_16043_gb300 import rt
+    sc = scenes.uniform_scene(n, 7)
+    bvh = build(sc)
+    if kind == "dirs":
+        rs = rt.rayspec(rt.RT_RAYS_DIRS, dirs=torch.from_numpy(scenes.fibonacci_sphere(K)).cuda())
+    else:
+        nrm = torch.from_numpy(scenes.shortest_axis_normals(sc["scale"], sc["quat"])).cuda()
+        rs = rt.rayspec(rt.RT_RAYS_HEMI, dirs=torch.from_numpy(scenes.fibonacci_hemisphere(K)).cuda(), normals=nrm)
+    ref = rt.rt_trace_visibility(bvh, rs, opts=rt.trace_opts(kernel=1)).double()
+    got = rt.rt_trace_visibility(bvh, rs).double()
+    torch.cuda.synchronize()
+    assert rt.rt_status_last() == 0
+    tol = 2.0 * MAX_HITS * 2.0 ** -24
+    off = (got - ref).abs() > tol * ref
+    assert not bool((off & (torch.maximum(got, ref) > 1e-4 * (1 + tol))).any())
