@@ -9,8 +9,9 @@ Default workload: the 2M-Gaussian object-scale scene (flattened Gaussians on
 directions = 256M rays per step.
 
 Printed (rank 0, one JSON line): traced rays/s of the whole precompute, ms
-per precompute, the roofline of the trace kernel (algorithmic bytes of node
-boxes and Gaussians fetched per ray over the measured HBM peak), the
+per precompute, the roofline of the trace kernel (the bytes it cannot do
+without over the measured HBM peak; the tests a ray needs are listed beside
+it), the
 end-to-end rate through the C ABI from pinned host buffers, the FP64 oracle's
 rate on the host cores (a bounded sample), and SM clocks sampled during the
 timed region.
@@ -50,14 +51,18 @@ WORKLOADS = {
     # under seeded rigid maps, two-level BVH, true inter-object occlusion
     "composed16_objects_k128": ("composed", 2_000_000, 60, 128),
 }
-KERNEL_NAMES = ["auto", "per-ray binary", "packet binary", "packet 4-wide", "per-ray 4-wide",
-                "per-ray 4-wide, lane refill", "warp per ray"]
+KERNEL_NAMES = ["auto", "per-ray binary", "packet binary", "shaft packets", "per-ray 4-wide",
+                "per-ray 4-wide, lane refill", "lanes per ray"]
 ENV_SAMPLES = 512
 METRIC = "traced rays/s & ms per 2M-Gaussian visibility precompute; surrogate speedup at MAE"
-TRACE_SOURCES = ["paper_2311_16043_gb300/csrc/rt_trace.cu", "paper_2311_16043_gb300/csrc/rt_trace_core.cuh"]
-# input check, bounds, morton, 4 x (hist, 3-kernel scan, scatter), perm,
-# prep, karras, refit, and the 4-wide collapse: one launch per level, 63 levels
-BUILD_KERNELS_PER_STEP = 27 + 63
+TRACE_SOURCES = ["paper_2311_16043_gb300/csrc/" + f for f in ("rt_trace.cu", "rt_trace_core.cuh", "rt_shaft.cuh")]
+
+
+def build_kernels(n):
+    """Launches of one tree build: bounds, codes in sorted order, records,
+    topology, boxes, wide nodes; beyond 12,288 Gaussians the codes take one
+    launch and four radix passes of three."""
+    return 6 if n <= 12_288 else 18
 
 
 def parse():
@@ -68,8 +73,8 @@ def parse():
     ap.add_argument("--impl", choices=["ours", "reference"], default="ours")
     ap.add_argument("--workload", choices=sorted(WORKLOADS), default="object_2m_k128")
     ap.add_argument("--kernel", type=int, default=0, choices=range(7),
-                    help="0 auto, 1 per-ray binary, 2 packet binary, 3 packet 4-wide, 4 per-ray 4-wide, "
-                         "5 per-ray 4-wide with lane refill, 6 warp per ray")
+                    help="0 auto, 1 per-ray binary, 2 packet binary, 3 shaft packets, 4 per-ray 4-wide, "
+                         "5 per-ray 4-wide with lane refill, 6 lanes per ray")
     ap.add_argument("--order-block", type=int, default=0)
     ap.add_argument("--cpu-rays", type=int, default=2048, help="oracle sample for cpu_baseline")
     ap.add_argument("--cpu-lbvh-rays", type=int, default=1 << 20, help="sample for the CPU BVH tracer baseline")
@@ -563,9 +568,8 @@ def batch_ray_stats(B, torch, rt, dev, sample=1 << 16):
     """Outside the timed region: per ray kind, the early-exit fraction over
     every output, and per-ray work (child-box tests, Gaussian tests, accepted
     hits) counted on `sample` seeded rays of each job with the per-ray 4-wide
-    traversal, which does each ray's minimal work; the work estimate of the
-    whole batch in the bench's byte model (28 B per box test, 40 B per
-    Gaussian test, 16 B per ray) from those per-job averages."""
+    traversal, which does each ray's minimal work; the bytes the batch cannot
+    do without (44 B per Gaussian of each job, 4 B per ray)."""
     import scenes
     stats, alg_bytes = {}, 0.0
     for kind in ("dirs", "env"):
@@ -580,12 +584,17 @@ def batch_ray_stats(B, torch, rt, dev, sample=1 << 16):
             rt.rt_trace_visibility(bvh, mk(ids), opts=rt.trace_opts(kernel=rt.RT_KERNEL_RAY_WIDE, counters=cnt))
             c = [int(x) for x in cnt.cpu()]
             m = ids.numel()
-            alg_bytes += T.numel() * (28.0 * c[0] / m + 40.0 * c[1] / m + 16.0)
+            alg_bytes += 44.0 * bvh.n + 4.0 * T.numel()
             box, gauss, hits, sampled = box + c[0], gauss + c[1], hits + c[2], sampled + m
         stats[kind] = {"rays": rays, "early_exit_fraction": zeros / max(rays, 1),
                        "box_tests_per_ray": box / max(sampled, 1), "gaussian_tests_per_ray": gauss / max(sampled, 1),
                        "accepted_hits_per_ray": hits / max(sampled, 1)}
     return stats, alg_bytes
+
+
+def batch_kernels(strategies):
+    """Launches of one batch replay: one for each of shaft packets, lane refill and the rest."""
+    return len({"shaft" if k == 3 else "refill" if k == 5 else "items" for k in strategies})
 
 
 def batch_destroy(B):
@@ -621,9 +630,9 @@ def run_batch_section(args, torch, rt, dev):
            "batch_create_s": B["create_s"], "strategy_per_job": info["kernel"], "ray_stats": stats,
            "roofline": {"bound": "hbm", "achieved": alg / (ms / 1000.0) / 1e9, "peak": pk["hbm_gbs"], "unit": "GB/s",
                         "frac": alg / (ms / 1000.0) / 1e9 / pk["hbm_gbs"], "peak_kind": pk_kind,
-                        "algorithmic_bytes_per_launch": alg, "kernel": "k_trace_batch (one persistent launch)",
-                        "bytes_model": "28 B per child-box test + 40 B per Gaussian test + 16 B per ray; per-ray "
-                                       "counts from 2^16 sampled rays per job (per-ray 4-wide traversal)"},
+                        "algorithmic_bytes_per_launch": alg, "kernel": "k_shaft_batch, k_trace_batch, k_refill_batch (one graph)",
+                        "bytes_model": "44 B per Gaussian of each job + 4 B per ray; bound by instruction issue and the "
+                                       "L1 data pipe"},
            "clocks": clk}
     batch_destroy(B)
     return out
@@ -669,10 +678,11 @@ def run_batch(args, rank, world, local, torch, dist, rt):
                     "scene_sizes": [b.n for b, _ in B["bvhs"]], "ray_stats": stats}),
                 "roofline": {"bound": "hbm", "achieved": achieved, "peak": pk["hbm_gbs"], "unit": "GB/s",
                              "frac": achieved / pk["hbm_gbs"], "traffic": None, "peak_kind": pk_kind,
-                             "algorithmic_bytes_per_launch": alg, "kernel": "k_trace_batch (one persistent launch)",
-                             "bytes_model": "28 B per child-box test + 40 B per Gaussian test + 16 B per ray; "
-                                            "per-ray counts from 2^16 sampled rays per job"},
-                "cpu_baseline": None, "e2e": None, "gpu_launches": args.steps, "clocks": clk}
+                             "algorithmic_bytes_per_launch": alg, "kernel": "k_shaft_batch, k_trace_batch, k_refill_batch (one graph)",
+                             "bytes_model": "44 B per Gaussian of each job + 4 B per ray; bound by instruction issue "
+                                            "and the L1 data pipe"},
+                "cpu_baseline": None, "e2e": None, "gpu_launches": batch_kernels(info["kernel"]) * args.steps,
+                "clocks": clk}
         print(json.dumps(line), flush=True)
     batch_destroy(B)
 
@@ -818,7 +828,7 @@ def main():
     bvh.destroy()
     box_tests, gauss_tests, hits, rays_cnt = (int(x) for x in cnt.cpu())
     assert rays_cnt == R, (rays_cnt, R)
-    alg_bytes = 28 * box_tests + 40 * gauss_tests + 16 * R
+    alg_bytes = 44 * n + 4 * R
 
     clocks = ClockSampler(local)
     evs = [[torch.cuda.Event(enable_timing=True) for _ in range(3)] for _ in range(args.steps)]
@@ -923,13 +933,17 @@ def main():
     pk, pk_kind = peaks()
     tr_ms = statistics.mean(trace_ms)
     achieved = alg_bytes / (tr_ms / 1000.0) / 1e9
+    # shaft packets share box tests and fetched records between the rays of a
+    # group, so bytes per ray times rays no longer say what the kernel reads
     roofline = {"bound": "hbm", "achieved": achieved, "peak": pk["hbm_gbs"], "unit": "GB/s",
                 "frac": achieved / pk["hbm_gbs"], "traffic": trace_traffic(),
-                "kernel": "k_trace (visibility trace)", "peak_kind": pk_kind,
+                "kernel": "k_trace_shaft (visibility trace)", "peak_kind": pk_kind,
                 "algorithmic_bytes_per_launch": alg_bytes,
                 "per_ray": {"box_tests": box_tests / R, "gaussian_tests": gauss_tests / R,
-                            "accepted_hits": hits / R},
-                "bytes_model": "28 B per child-box test + 40 B per Gaussian test + 16 B per ray"}
+                            "accepted_hits": hits / R,
+                            "counted_on": "the plain packet walk, whose rays share no test"},
+                "bytes_model": "44 B per Gaussian read once + 4 B per ray written; the kernel is bound by instruction "
+                               "issue (profiles/)"}
 
     cpu = None
     if rank == 0 and world == 1 and not args.no_cpu_baseline:
@@ -948,7 +962,7 @@ def main():
                     "build_ms": statistics.mean(build_ms), "trace_ms": tr_ms,
                     "kernel": KERNEL_NAMES[args.kernel]}),
                 "roofline": roofline, "cpu_baseline": cpu, "e2e": e2e,
-                "gpu_launches": (BUILD_KERNELS_PER_STEP + 1) * args.steps,
+                "gpu_launches": (build_kernels(n) + 1) * args.steps,
                 "clocks": clk, "surrogate": surrogate, "adjoint": adjoint, "pbr": pbr, "refit": refit,
                 "batch": batch_sec}
         print(json.dumps(line), flush=True)

@@ -65,7 +65,7 @@ struct rt_bvh {
     int2 *groups;            // [n_groups] first sorted position and count of each shaft group
     int64_t n_groups;        // (host copy)
     float4 *wide;            // [8 * (n-1)] 4-wide nodes (collapsed binary tree)
-    float4 *qwide;           // [4 * (n-1)] the same nodes in 64 bytes (below)
+    float4 *qwide;           // [4 * (n-1)] the same nodes in 64 bytes
     int64_t n_wide;          // indices of 4-wide nodes: n-1, or 0 for n < 2
     int32_t levels;          // levels of the binary tree, a bound on the 4-wide one's (host copy)
 };

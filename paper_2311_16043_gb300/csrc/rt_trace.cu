@@ -1,16 +1,18 @@
 // rt_trace.cu -- visibility of a ray set (Eq. 13-15, Sec. 4.1-4.2).
 //
-// One persistent launch: each warp repeatedly takes a work item of 32 rays
-// from a device counter.  For a full implicit set (every Gaussian x K
-// directions) an item is 32 Gaussians adjacent in Morton order x one
-// direction, so the warp's rays are nearly parallel and start close together.
-// Items are ordered in sweeps: `order_block` tiles for direction 0, the same
-// tiles for direction 1, ... .  The default, one tile per sweep, hands out a
-// tile's K directions in turn: the rows T[g, 0..K) of a tile are written
-// within a short window (whole sectors merge in L2) and the warps in flight
-// start in the same region of the tree (sweeps of 64 to 62,500 tiles measured
-// 0.6-2 % slower on the 2M-Gaussian object scene).  Explicit ray lists and id
-// subsets are taken in chunks of 32 in the given order.
+// One persistent launch: each warp (or group of lanes) repeatedly takes a work
+// item from a device counter.  For a full implicit set (every Gaussian x K
+// directions) an item is a shaft group x one direction (strategy 3), a ray slot
+// (lane refill, lane groups) or 32 Gaussians adjacent in Morton order x one
+// direction (the other packets and walks), so that a warp's rays start close
+// together and, in a direction set, are parallel.  Items are ordered in
+// sweeps: `order_block` tiles or groups for direction 0, the same for direction
+// 1, ... .  The default, one per sweep, hands out its K directions in turn: the
+// rows T[g, 0..K) are written within a short window (whole sectors merge in L2)
+// and the warps in flight start in the same region of the tree (packets:
+// sweeps of 64 to 62,500 tiles measured 0.6-2 % slower on the 2M-Gaussian object
+// scene; lane refill: no difference from 1 to 4,096).  Explicit ray lists and id
+// subsets are taken in the given order.
 #include <string.h>
 
 #include "rt_shaft.cuh"
