@@ -268,8 +268,9 @@ typedef enum {
     RT_KERNEL_WARP_RAY = 6   /* a group of lanes per ray over the 4-wide tree: they
                               expand as many of the ray's nodes at once (full
                               sets and up to 8192 rays: 32 lanes; lists up to
-                              2^16: 16, up to 2^18: 8, beyond: 4; scattered
-                              rays; no hit log)                              */
+                              2^16: 16, up to 2^18 or over more than 2^20
+                              Gaussians: 8, beyond: 4; scattered rays; no hit
+                              log)                                           */
 } rt_kernel;
 
 typedef struct {
