@@ -153,8 +153,17 @@ struct ShaftCand {
 //   m^2 = (x - (B / C) y)^2 C / det + y^2 / C
 // without a difference of large terms.  t* of a ray from r is q . (mu - r),
 // q = W^T W d / |W d|^2.  p = mu - c - s d is the mean moved along d next to
-// the rays.  Error bound: every term of v is at most |W| reach, mu - c
-// carries |s| ulps, and gauss_eval's own error is within the same terms.
+// the rays.
+// Error bound, in ulps eps = 2^-24, for a ray that gauss_eval may accept (m the
+// largest m it accepts, s_max the longest axis): every term of v is at most
+// |W| (group radius + |p|), and mu - c carries |s| ulps.  f_k is off by eps
+// s_k whatever its size, u by eps |w_k|, so C, B and |W d|^2 are off by up to
+// a few eps s_max |W| of themselves where the projections are small (needles
+// seen nearly end-on, discs edge-on), and v with them, |v| <= m: this does
+// not shrink with the rays' distance.  gauss_eval's peak lies up to m s_max
+// from mu, which puts eps |W| m s_max into its u.  Hence `reach`, the group
+// radius + |p| + m s_max, at 40 eps; the limit of |v|^2 moves by E (2 m + E).
+// The same lengths bound t*, in units of 1 / |W d|.
 // frame: fr[0] = (c, |d|^2), fr[1] = (d, |d|), fr[2] = (d / |d|^2, group
 // radius), fr[3] = (e1, k_sigma^2 log2(e)/2), fr[4] = (e2, log2(alpha_min)).
 template <bool GRAD>
@@ -197,14 +206,18 @@ __device__ __forceinline__ void shaft_cand(const ShaftSmem<GRAD> &sm, const floa
     g.qy = mul(fma2(u0, b0, fma2(u1, b1, mul(u2, b2))), iu);
     const float2 nn = __fadd2_rn(n0, __fadd2_rn(n1, n2));
     const float2 hb = __fadd2_rn(__fadd2_rn(s, pz), fma2(g.qx, px, mul(g.qy, py)));
-    auto lim = [&](float nn1, float px1, float py1, float s1, float iu1, float o, float h1, float &thr, float &h) {
-        const float wn = sqrtf(nn1), reach = F2.w + fabsf(px1) + fabsf(py1), sl = fabsf(s1) * F1.w;
+    auto lim = [&](float nn1, float nmin, float px1, float py1, float s1, float iu1, float o, float h1, float &thr,
+                   float &h) {
+        const float L = fminf(F3.w, __log2f(o) - F4.w), m = sqrtf(fmaxf(L, 0.0f));  // |v| <= m; 1.18 m sigma
+        const float wn = sqrtf(nn1), reach = fmaf(1.18f * m, rsqrtf(nmin), F2.w + fabsf(px1) + fabsf(py1)),
+                    sl = fabsf(s1) * F1.w;
         const float E = wn * fmaf(2.4e-6f, reach, 4e-7f * sl);
-        thr = fmaf(E, 6.0f + E, fminf(F3.w, __log2f(o) - F4.w) + 1e-5f);
+        thr = fmaf(E, fmaf(2.0f, m, E), fmaf(L, 1.000001f, 1e-5f));
         h = fmaf(2e-6f, fmaf(wn * (reach + sl), sqrtf(iu1), fabsf(s1)), h1);
     };
-    lim(nn.x, px.x, py.x, s.x, iu.x, a[0].w, hb.x, g.thr.x, g.h.x);
-    lim(nn.y, px.y, py.y, s.y, iu.y, b[0].w, hb.y, g.thr.y, g.h.y);
+    const float na = fminf(n0.x, fminf(n1.x, n2.x)), nb = fminf(n0.y, fminf(n1.y, n2.y));
+    lim(nn.x, na, px.x, py.x, s.x, iu.x, a[0].w, hb.x, g.thr.x, g.h.x);
+    lim(nn.y, nb, px.y, py.y, s.y, iu.y, b[0].w, hb.y, g.thr.y, g.h.y);
 }
 
 // gauss_eval of two pairs at once, each operation rounded as there.
