@@ -324,10 +324,15 @@ __device__ __forceinline__ void shaft_group(const BvhDev &b, float eps, float3 d
     };
     bounds(live);
     {
-        // plane frame (e1, e2) across d (Duff et al. 2017)
-        const float dd = dot3(d, d), il = rsqrtf(dd);
-        const float3 dn = make_float3(d.x / dd, d.y / dd, d.z / dd);
-        const float x = d.x * il, y = d.y * il, z = d.z * il;
+        // plane frame (e1, e2) across d (Duff et al. 2017); d scaled by a power
+        // of two (exact) to a largest component in [1, 2): |d|^2 is in range, and
+        // all that the rejection test computes is in units of |d|
+        const uint32_t e = __float_as_uint(fmaxf(fmaxf(fabsf(d.x), fabsf(d.y)), fabsf(d.z))) >> 23;
+        const float pw = __uint_as_float((e < 253u ? 254u - e : 1u) << 23);
+        const float3 ds = make_float3(d.x * pw, d.y * pw, d.z * pw);
+        const float dd = dot3(ds, ds), il = rsqrtf(dd);
+        const float3 dn = make_float3(ds.x / dd, ds.y / dd, ds.z / dd);
+        const float x = ds.x * il, y = ds.y * il, z = ds.z * il;
         const float sg = copysignf(1.0f, z), a = -1.0f / (sg + z), q = x * y * a;
         const float3 e1 = make_float3(1.0f + sg * x * x * a, sg * q, -sg * x), e2 = make_float3(q, sg + y * y * a, -y);
 #pragma unroll
@@ -341,7 +346,7 @@ __device__ __forceinline__ void shaft_group(const BvhDev &b, float eps, float3 d
         }
         if (lane == 0) {
             sm.fr[0] = make_float4(c.x, c.y, c.z, dd);
-            sm.fr[1] = make_float4(d.x, d.y, d.z, sqrtf(dd));
+            sm.fr[1] = make_float4(ds.x, ds.y, ds.z, sqrtf(dd));
             sm.fr[2] = make_float4(dn.x, dn.y, dn.z, hh.x + hh.y + hh.z);
             sm.fr[3] = make_float4(e1.x, e1.y, e1.z, 0.72134752f * b.k2);
             sm.fr[4] = make_float4(e2.x, e2.y, e2.z, log2f(b.alpha_min));

@@ -13,6 +13,8 @@ import pytest
 import torch
 from scipy.spatial.transform import Rotation
 
+import scenes
+
 pytestmark = pytest.mark.gpu
 RTOL = 2 * 2304 * 2.0 ** -24
 N_SRC, N, K = 256, 2048, 8
@@ -73,3 +75,20 @@ def test_accepts_what_single_rays_accept(aspect, what, limit):
     assert rt.rt_status_last() == 0
     assert a.max().item() < 0.9  # the needles are met
     assert bool(((b - a).abs() <= RTOL * a + 1e-30).all()), ((b - a).abs() / a).max().item()
+
+
+@pytest.mark.parametrize("length", [1e-21, 1e-19, 1e-12, 1e12, 1e15])
+def test_directions_of_any_length(length):
+    """|d|^2 may underflow or lose its digits where the per-ray walks, which
+    never form it, are exact (h <= 512 factors)."""
+    from paper_2311_16043_gb300 import rt
+    sc = scenes.uniform_scene(1500, 6)
+    sc["mean"] = (0.5 * sc["mean"]).astype(np.float32)
+    dirs = scenes.fibonacci_sphere(6) * length
+    bvh = rt.rt_build_bvh(*(_dev(sc[k]) for k in ("mean", "scale", "quat", "opacity")),
+                          rt.params(t_min=0.0, origin_eps=0.0))
+    a, b = (rt.rt_trace_visibility_dirs(bvh, _dev(dirs), opts=rt.trace_opts(kernel=k)).double() for k in (1, 3))
+    torch.cuda.synchronize()
+    assert rt.rt_status_last() == 0
+    assert a.min().item() < 0.5
+    assert bool(((b - a).abs() <= 2 * 512 * 2.0 ** -24 * a).all()), ((b - a).abs() / a).max().item()
