@@ -284,7 +284,8 @@ typedef struct {
     int32_t *hit_ids;    /* device [R*hit_cap]: original indices of accepted
                             Gaussians per ray, in traversal order (NULL = off) */
     int32_t *hit_count;  /* device [R]: accepted hits per ray (may exceed
-                            hit_cap: the log of that ray is then incomplete)   */
+                            hit_cap: the log of that ray is then incomplete);
+                            0 for every ray if hit_ids is NULL                 */
 } rt_trace_opts;
 
 /* T_out[R] (device float32): visibility of every ray of the set, in ray-id

@@ -323,6 +323,10 @@ rt_status rt_trace_launch(const rt_bvh *bvh, const rt_rayspec *rays, float *T_ou
     }
     rt_status res = RT_OK;
     if (cudaMemsetAsync(work, 0, sizeof(unsigned long long), st) != cudaSuccess) res = RT_ERR_CUDA;
+    // counts without a log: none is kept, and the walks that keep no log write none
+    if (o.hit_count && !o.hit_ids && (strat == 3 || strat >= 5) &&
+        cudaMemsetAsync(o.hit_count, 0, sizeof(int32_t) * (size_t)count, st) != cudaSuccess)
+        res = RT_ERR_CUDA;
     if (res == RT_OK) {
         const int threads = 128;
         const bool count = aux.counters != nullptr;
