@@ -849,8 +849,13 @@ __device__ __forceinline__ void flush_counts(const TraceAux &aux, const WorkCoun
 // A step of a lane is one node visit, which puts the leaves met into a queue of
 // the lane's own (first in first out, so a ray's factors come in the order of
 // its walk whatever its neighbours do); the Gaussians are evaluated, one per
-// lane, once kLeafMin lanes have one waiting: in the visit itself each of the
-// four children had a branch with 6 of 32 lanes busy.
+// lane, once half of the lanes that have a ray (16 at most) have one waiting: in
+// the visit itself each of the four children had a branch with 6 of 32 lanes
+// busy.  With 16 asked for however few lanes still have a ray, a warp's last rays
+// only learn that they are dark when their queues are full: sets that do not
+// fill the lanes many times over took up to 1.5 times as long (hemisphere sets of
+// the 20k object scene, us: x 16 567 -> 330, x 64 964 -> 751; 300k x 64 28.7 ms
+// either way; a third of the lanes instead of half: 349, 778, 31.0 ms).
 // Bound: the L1 data pipe (0.8 of it; a wavefront per lane and 32-byte load, 78
 // nodes and 71 Gaussians a ray, hit rate 0.2), then issue (0.65).  Measured on
 // the way, ms for the 300k object scene's hemisphere set x 64, the 200k's
@@ -870,10 +875,6 @@ __device__ __forceinline__ void flush_counts(const TraceAux &aux, const WorkCoun
 #define RT_REFILL_MIN 6
 #endif
 constexpr int kRefillMin = RT_REFILL_MIN;
-#ifndef RT_LEAF_MIN
-#define RT_LEAF_MIN 16
-#endif
-constexpr int kLeafMin = RT_LEAF_MIN;
 constexpr int kLeafQueue = 8;
 #ifndef RT_STACK_SHARED
 #define RT_STACK_SHARED 24
@@ -930,7 +931,8 @@ __device__ __forceinline__ void refill_walk(Src &from, int *status, unsigned lon
                 }
             }
         }
-        if (__ballot_sync(FULL, has) == 0) {
+        const int n_has = __popc(__ballot_sync(FULL, has));
+        if (n_has == 0) {
             if (exhausted) break;
             continue;
         }
@@ -962,7 +964,7 @@ __device__ __forceinline__ void refill_walk(Src &from, int *status, unsigned lon
         }
         for (;;) {
             const unsigned pend = __ballot_sync(FULL, qn > 0), walk = __ballot_sync(FULL, node >= 0 && qn <= kLeafQueue - 4);
-            if (pend == 0 || (__popc(pend) < kLeafMin && walk != 0)) break;
+            if (pend == 0 || (__popc(pend) < n_has / 2 && walk != 0)) break;
             if (qn > 0) {
                 const int32_t p = queue[qh * 128];
                 qh = (qh + 1) & (kLeafQueue - 1);
