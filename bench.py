@@ -593,8 +593,8 @@ def batch_ray_stats(B, torch, rt, dev, sample=1 << 16):
 
 
 def batch_kernels(strategies):
-    """Launches of one batch replay: one for each of shaft packets, lane refill and the rest."""
-    return len({"shaft" if k == 3 else "refill" if k == 5 else "items" for k in strategies})
+    """Launches of one batch replay: one for the shaft packets, one for all other jobs."""
+    return len({k == 3 for k in strategies})
 
 
 def batch_destroy(B):

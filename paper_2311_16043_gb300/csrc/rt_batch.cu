@@ -12,10 +12,12 @@
 // Batch: the work items of all jobs form virtual queues, job after job in
 // decreasing estimated cost (rays x log2 n), consumed through device counters
 // by persistent grids; each warp finds its job by binary search over the jobs'
-// first item and runs that job's strategy.  Shaft jobs (direction sets), lane
-// refill jobs (env-map and hemisphere sets) and the others have a kernel each
-// (20, 36 and 32 warps a multiprocessor fit), parallel branches of one captured
-// CUDA graph after the counters' reset.
+// first item and runs that job's strategy.  Shaft jobs (direction sets) have a
+// kernel of their own; item jobs and lane refill jobs (env-map and hemisphere
+// sets) share one, in which a warp goes on to the refill queue when the items are
+// out (a batch of refill jobs alone takes a kernel with 36 warps a multiprocessor
+// instead of 32).  The two are parallel branches of one captured CUDA graph after
+// the counters' reset.
 #include <math.h>
 #include <string.h>
 
@@ -121,12 +123,17 @@ __device__ __forceinline__ void batch_refill(const BatchJobDev *__restrict__ job
     refill_walk<false>(from, status, work, wc, rays_done);
 }
 
-// The jobs [0, n_item_jobs) that are consumed as 32-ray items.
+// The jobs [0, n_item_jobs) that are consumed as 32-ray items, then (REFILL) the
+// refill jobs after them.  As two launches the second starts on the first's
+// longest rays: untuned batches of four object scenes of 2 to 7 thousand
+// Gaussians 366 us against 329.
 #ifndef RT_BATCH_MIN_BLOCKS
 #define RT_BATCH_MIN_BLOCKS 8
 #endif
-__global__ void __launch_bounds__(128, RT_BATCH_MIN_BLOCKS) k_trace_batch(const BatchJobDev *__restrict__ jobs, int n_item_jobs,
-                                                     int64_t total_items, int *status, unsigned long long *work) {
+template <bool REFILL>
+__global__ void __launch_bounds__(128, RT_BATCH_MIN_BLOCKS)
+    k_trace_batch(const BatchJobDev *__restrict__ jobs, int n_item_jobs, int64_t total_items, int n_jobs,
+                  int64_t total_slots, int *status, unsigned long long *work) {
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     __shared__ int2 stk_all[4 * RT_WIDE_STACK];
@@ -156,6 +163,10 @@ __global__ void __launch_bounds__(128, RT_BATCH_MIN_BLOCKS) k_trace_batch(const 
         else if (J.strat == 2) trace_item<2, false>(J.b, J.rs, J.job, J.T_out, aux, local, J.job.n_out, wc, rays_done, stk);
         else if (J.strat == 1) trace_item<1, false>(J.b, J.rs, J.job, J.T_out, aux, local, J.job.n_out, wc, rays_done, stk);
         else trace_item<0, false>(J.b, J.rs, J.job, J.T_out, aux, local, J.job.n_out, wc, rays_done, stk);
+    }
+    if (REFILL) {
+        __syncwarp();
+        batch_refill(jobs, n_item_jobs, n_jobs, total_slots, status, work + 1);
     }
 }
 
@@ -362,6 +373,20 @@ extern "C" rt_status rt_batch_create(const rt_batch_job *jobs, int32_t n_jobs, i
         H.job = full_job(J.bvh, rs.K, o.order_block, H.strat == 3);
         cost[j] = (double)count * log2((double)(J.bvh->n > 1 ? J.bvh->n : 2));
     }
+    // a few shaft jobs of less than 2^17 rays together, beside other jobs: one
+    // thread per ray in the others' kernel, since a launch of their own costs more
+    // than they save (the four scenes of 2 to 7 thousand, tuned, the first of them
+    // 48 thousand direction rays: 358 us with it in shafts, 315 without)
+    int64_t shaft_rays = 0, other_rays = 0;
+    for (int j = 0; j < n_jobs; ++j) (host[j].strat == 3 ? shaft_rays : other_rays) += host[j].job.n_out;
+    if (other_rays > 0 && shaft_rays < (int64_t(1) << 17))
+        for (int j = 0; j < n_jobs; ++j)
+            if (host[j].strat == 3) {
+                host[j].strat = 4;
+                host[j].job = full_job(jobs[j].bvh, host[j].rs.K, 1, false);
+                bt->kernel[j] = RT_KERNEL_RAY_WIDE;
+                bt->order_block[j] = 1;
+            }
     // shaft jobs (a queue and kernel of their own), item jobs, then lane-refill
     // jobs; largest estimated cost first in each
     std::vector<int> order(n_jobs);
@@ -406,39 +431,46 @@ extern "C" rt_status rt_batch_create(const rt_batch_job *jobs, int32_t n_jobs, i
         delete bt;
         return RT_ERR_CUDA;
     }
-    // capture: reset the queue counters, then one persistent launch for each
-    // kind of job on a branch of its own, so that each fills the
-    // multiprocessors as the blocks of the one before leave
+    // capture: reset the queue counters, then one persistent launch for the item
+    // and refill jobs and one for the shaft jobs, each on a branch of its own, so
+    // that the second fills the multiprocessors as the blocks of the first leave.
+    // The shaft jobs come second: their longest item is shorter than the others'
+    // longest ray (four uniform scenes of 100 to 686 thousand Gaussians 61.1 ms, the
+    // other way round 64.0)
     const int n_refill_jobs = n_jobs - n_shaft_jobs - n_item_jobs;
-    cudaStream_t cap[3] = {nullptr, nullptr, nullptr};
-    cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};  // fork, the joins
+    cudaStream_t cap[2] = {nullptr, nullptr};
+    cudaEvent_t ev[2] = {nullptr, nullptr};  // fork, join
     bool ok = true;
-    for (int q = 0; q < 3; ++q)
+    for (int q = 0; q < 2; ++q)
         ok = ok && cudaStreamCreateWithFlags(&cap[q], cudaStreamNonBlocking) == cudaSuccess &&
              cudaEventCreateWithFlags(&ev[q], cudaEventDisableTiming) == cudaSuccess;
     int *status = rt_status_ptr();
     if (ok && (ok = cudaStreamBeginCapture(cap[0], cudaStreamCaptureModeThreadLocal) == cudaSuccess)) {
         cudaMemsetAsync(work, 0, 24, cap[0]);
         cudaEventRecord(ev[0], cap[0]);
+        const BatchJobDev *rest = dtab + n_shaft_jobs;
+        const int n_rest = n_item_jobs + n_refill_jobs;
+        if (n_rest > 0) {
+            cudaStreamWaitEvent(cap[1], ev[0], 0);
+            if (n_refill_jobs == 0)
+                k_trace_batch<false><<<persistent_grid((const void *)k_trace_batch<false>), 128, 0, cap[1]>>>(
+                    rest, n_item_jobs, items, n_rest, slots, status, work);
+            else if (n_item_jobs > 0)
+                k_trace_batch<true><<<persistent_grid((const void *)k_trace_batch<true>), 128, 0, cap[1]>>>(
+                    rest, n_item_jobs, items, n_rest, slots, status, work);
+            else
+                k_refill_batch<<<persistent_grid((const void *)k_refill_batch), 128, 0, cap[1]>>>(
+                    rest, n_refill_jobs, slots, status, work + 1);
+            cudaEventRecord(ev[1], cap[1]);
+        }
         if (n_shaft_jobs > 0)
             k_shaft_batch<<<persistent_grid((const void *)k_shaft_batch), 128, 0, cap[0]>>>(dtab, n_shaft_jobs, shafts,
                                                                                             status, work + 2);
-        for (int q = 1; q < 3; ++q) {
-            if ((q == 1 ? n_item_jobs : n_refill_jobs) == 0) continue;
-            cudaStreamWaitEvent(cap[q], ev[0], 0);
-            if (q == 1)
-                k_trace_batch<<<persistent_grid((const void *)k_trace_batch), 128, 0, cap[q]>>>(
-                    dtab + n_shaft_jobs, n_item_jobs, items, status, work);
-            else
-                k_refill_batch<<<persistent_grid((const void *)k_refill_batch), 128, 0, cap[q]>>>(
-                    dtab + n_shaft_jobs + n_item_jobs, n_refill_jobs, slots, status, work + 1);
-            cudaEventRecord(ev[q], cap[q]);
-            cudaStreamWaitEvent(cap[0], ev[q], 0);
-        }
+        if (n_rest > 0) cudaStreamWaitEvent(cap[0], ev[1], 0);
         ok = cudaStreamEndCapture(cap[0], &bt->graph) == cudaSuccess;
     }
     if (ok) ok = cudaGraphInstantiate(&bt->exec, bt->graph, 0) == cudaSuccess;
-    for (int q = 0; q < 3; ++q) {
+    for (int q = 0; q < 2; ++q) {
         if (ev[q]) cudaEventDestroy(ev[q]);
         if (cap[q]) cudaStreamDestroy(cap[q]);
     }
