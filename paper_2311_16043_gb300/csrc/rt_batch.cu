@@ -435,7 +435,7 @@ extern "C" rt_status rt_batch_create(const rt_batch_job *jobs, int32_t n_jobs, i
     // and refill jobs and one for the shaft jobs, each on a branch of its own, so
     // that the second fills the multiprocessors as the blocks of the first leave.
     // The shaft jobs come second: their longest item is shorter than the others'
-    // longest ray (four uniform scenes of 100 to 686 thousand Gaussians 61.1 ms, the
+    // longest ray (four uniform scenes of 30 to 206 thousand Gaussians 61.1 ms, the
     // other way round 64.0)
     const int n_refill_jobs = n_jobs - n_shaft_jobs - n_item_jobs;
     cudaStream_t cap[2] = {nullptr, nullptr};

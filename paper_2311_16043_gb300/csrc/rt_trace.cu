@@ -166,7 +166,8 @@ void launch_lanes(int lanes, const BvhDev &b, const RaySetDev &rs, const TraceJo
 
 }  // namespace
 
-// Launch the single-scene kernel on an explicit job (used by the autotuner).
+// Launch the single-scene kernel of strategy 0 to 5 on an explicit job (used by
+// the autotuner).
 rt_status rt_trace_launch_job(const BvhDev &b, const RaySetDev &rs, const TraceJob &job, float *T_out,
                               int strat, rt_stream_t stream, unsigned long long *work) {
     TraceAux aux;
@@ -175,9 +176,7 @@ rt_status rt_trace_launch_job(const BvhDev &b, const RaySetDev &rs, const TraceJ
     cudaStream_t st = (cudaStream_t)stream;
     if (cudaMemsetAsync(work, 0, sizeof(unsigned long long), st) != cudaSuccess) return RT_ERR_CUDA;
     const int threads = 128;
-    if (strat == 6 && b.wide) {
-        launch_lanes<false>(lanes_for(job.mode == MODE_FULL, job.n_out, b), b, rs, job, T_out, aux, st, work);
-    } else if (strat == 5 && b.wide && job.mode == MODE_FULL) {
+    if (strat == 5 && b.wide && job.mode == MODE_FULL) {
         int grid = persistent_blocks((const void *)k_trace<5, false>, threads);
         k_trace<5, false><<<grid, threads, 0, st>>>(b, rs, job, T_out, aux, work);
     } else if (strat >= 4 && b.wide) {
