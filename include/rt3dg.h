@@ -243,16 +243,21 @@ rt_status rt_materialize_rays(const rt_bvh *bvh, const rt_rayspec *rays, const i
 
 typedef enum {
     RT_KERNEL_AUTO = 0,   /* small full sets (DIRS up to 2^15 rays, ENV and
-                             HEMI up to 2^20, few per Gaussian): lanes by the
-                             number of rays as in WARP_RAY's lists; DIRS sets:
+                             HEMI up to 2^20, few per Gaussian): as WARP_RAY
+                             with 32 lanes to 4 by the number of rays; DIRS sets:
                              WIDE where neighbouring Gaussians lie close
                              together (measured on the tree), else RAY_WIDE;
                              ENV and HEMI sets: RAY_WIDE up to 2^19 rays,
                              RAY_REFILL beyond; explicit
-                             rays and id lists: WARP_RAY up to 2^22 rays
+                             rays and id lists: as WARP_RAY up to 2^22 rays,
+                             32 lanes up to 8192 rays, 16 up to 2^16, 8 up to
+                             2^18 or over more than 2^20 Gaussians, 4 beyond
                              (RAY_WIDE with a hit log), RAY_WIDE beyond (an id
                              list traced in the tree's order); the binary
-                             forms when there is no 4-wide tree              */
+                             forms when there is no 4-wide tree.  The strategies
+                             multiply a ray's factors in different orders, so
+                             the same ray in sets or lists of different sizes
+                             may differ in the last bits of T                */
     RT_KERNEL_RAY = 1,    /* one thread per ray, private stack, binary tree    */
     RT_KERNEL_PACKET = 2, /* one warp per 32 rays of neighbouring Gaussians in
                              one direction, shared stack, binary tree          */
@@ -265,12 +270,10 @@ typedef enum {
     RT_KERNEL_RAY_REFILL = 5, /* as RAY_WIDE, idle lanes refilled with new rays
                               as theirs finish (full implicit sets; otherwise
                               RAY_WIDE)                                       */
-    RT_KERNEL_WARP_RAY = 6   /* a group of lanes per ray over the 4-wide tree: they
-                              expand as many of the ray's nodes at once (full
-                              sets and up to 8192 rays: 32 lanes; lists up to
-                              2^16: 16, up to 2^18 or over more than 2^20
-                              Gaussians: 8, beyond: 4; scattered rays; no hit
-                              log)                                           */
+    RT_KERNEL_WARP_RAY = 6   /* one warp per ray over the 4-wide tree: the lanes
+                              expand up to 32 of the ray's nodes at once (few
+                              or latency-bound rays; no hit log).  T of a ray
+                              is the same bit for bit in any set or list     */
 } rt_kernel;
 
 typedef struct {
@@ -543,7 +546,7 @@ rt_status rt_surrogate_train(rt_surrogate *s, const rt_bvh *bvh, const rt_rayspe
  * network's estimate (= p for w = 1).  If band > 0, rays with
  * |p - 0.5| < band are traced on `bvh` instead (the fallback:
  * RT_KERNEL_WARP_RAY) and T_out holds the traced value, bit-equal to
- * rt_trace_visibility of the same ray set with that kernel; n_fallback (device int64[1], may be
+ * rt_trace_visibility with that kernel; n_fallback (device int64[1], may be
  * NULL) receives their
  * number.  The scene bounds used to normalise origins are the surrogate's.
  * Errors: RT_ERR_INVALID_ARG. */

@@ -121,17 +121,20 @@ int persistent_blocks(const void *kernel, int threads) {
     return per_sm * rt_num_sms();
 }
 
-// Lanes per ray for a list of m rays (a fallback list: the most it can be).
-// 300k object scene, shadow rays in no order, us with 32 / 16 / 8 / 4
+// Lanes per ray that AUTO takes for m rays.  300k object scene, shadow rays in no order, us with 32 / 16 / 8 / 4
 // lanes: 2,000 rays 50 / 69 / 101 / 176; 20,000 122 / 122 / 154 / 230; 100,000
 // 433 / 368 / 325 / 361; 250,000 1,019 / 836 / 683 / 667; 600,000 2,384 /
 // 1,929 / 1,491 / 1,322.  Beyond 2^20 Gaussians nodes and records exceed the L2
 // cache and more lanes hide its misses: 1M rays of the 2M scene 6,138 / 5,724 /
 // 5,302 / 6,443.  4 lanes' stack holds a walk of single nodes through 36 levels.
-// A full set keeps 32, so that a ray of it and of a short id list get the same
-// T bit for bit.
-int lanes_for(bool full, int64_t m, const BvhDev &b) {
-    if (full || m <= 8192) return 32;
+// RT_KERNEL_WARP_RAY asked for by name, and the surrogate's fallback with it, keep
+// 32 whatever the number: the order of a ray's factors follows the lanes, and T
+// of these is to be the same bit for bit in a full set and in any list.  (A
+// fallback list's length is also only known on the device: lanes by its bound took
+// 113 us for the 2,900 of 70,000 rays that fall back on the 200k scene, 32
+// lanes 74; for 134,000 of 2M rays, the other way, 820 and 976.)
+int lanes_for(int64_t m, const BvhDev &b) {
+    if (m <= 8192) return 32;
     if (m <= 65536) return 16;
     return m <= 262144 || b.levels > 36 || b.n > (int64_t(1) << 20) ? 8 : 4;
 }
@@ -335,7 +338,7 @@ rt_status rt_trace_launch(const rt_bvh *bvh, const rt_rayspec *rays, float *T_ou
         k_trace<S, C><<<grid, threads, 0, st>>>(b, rs, job, T_out, aux, work);              \
     } while (0)
         if (strat == 6) {
-            const int lanes = lanes_for(o.kernel == RT_KERNEL_WARP_RAY && job.mode == MODE_FULL, job.n_out, b);
+            const int lanes = o.kernel == RT_KERNEL_WARP_RAY ? 32 : lanes_for(job.n_out, b);
             if (count) launch_lanes<true>(lanes, b, rs, job, T_out, aux, st, work);
             else launch_lanes<false>(lanes, b, rs, job, T_out, aux, st, work);
         }
@@ -388,11 +391,10 @@ rt_status rt_trace_launch_list(const rt_bvh *bvh, const rt_rayspec *rays, const 
     cudaStream_t st = (cudaStream_t)stream;
     if (cudaMemsetAsync(work, 0, sizeof(unsigned long long), st) != cudaSuccess) return RT_ERR_CUDA;
     const int threads = 128;
-    // the listed rays are few and scattered: a group of lanes per ray over the
-    // 4-wide tree, which cuts the latency of the longest traversal
+    // the listed rays are few and scattered: RT_KERNEL_WARP_RAY
     const BvhDev b = bvh_dev(bvh);
     if (bvh->n_wide > 0) {
-        launch_lanes<false>(lanes_for(!rays->ray_ids, max_count, b), b, rs, job, T_out, aux, st, work);
+        launch_lanes<false>(32, b, rs, job, T_out, aux, st, work);
     } else {
         int grid = persistent_blocks((const void *)k_trace<0, false>, threads);
         k_trace<0, false><<<grid, threads, 0, st>>>(b, rs, job, T_out, aux, work);
