@@ -152,10 +152,12 @@ __device__ __forceinline__ bool qnode_ray(float3 o, float3 d, float3 &inv, float
 // of NaN base does not count.
 // Two 32-byte loads instead of four: the walks of single rays are bound by the
 // L1 data pipe, a wavefront per lane and load.  Not kept in L1, which these
-// walks hit 0.2 of the time and whose fills cost the same pipe (2 to 2.5 %).
+// walks hit 0.2 of the time and whose fills cost the same pipe (2 to 2.5 %);
+// CACHED: kept, for walks bound by a ray's latency.
+template <bool CACHED = false>
 __device__ __forceinline__ void qnode_near(const float4 *__restrict__ q, float3 inv, float3 oi, float (&tn)[4],
                                            uint32_t (&r)[4]) {
-    const float4x2 n0 = ldg_pair_once(q), n1 = ldg_pair_once(q + 2);
+    const float4x2 n0 = CACHED ? ldg_pair(q) : ldg_pair_once(q), n1 = CACHED ? ldg_pair(q + 2) : ldg_pair_once(q + 2);
     const float ax = n0.a.w * inv.x, ay = n0.b.x * inv.y, az = n0.b.y * inv.z;
     const float cx = fmaf(n0.a.x, inv.x, -oi.x), cy = fmaf(n0.a.y, inv.y, -oi.y), cz = fmaf(n0.a.z, inv.z, -oi.z);
     const bool sx = inv.x < 0.0f, sy = inv.y < 0.0f, sz = inv.z < 0.0f;
@@ -1082,7 +1084,7 @@ __device__ __forceinline__ void trace_lane_group(const BvhDev &b, const RaySetDe
         uint32_t r[4] = {0u, 0u, 0u, 0u}, pm = 0u;  // internal children to push: a mask over c
         if (sub < k) {
             float tn[4];
-            qnode_near(b.qwide + 4 * (int64_t)node, inv, oi, tn, r);
+            qnode_near<LANES == 32>(b.qwide + 4 * (int64_t)node, inv, oi, tn, r);
             if (COUNT) wc.box += (r[0] != RT_EMPTY) + (r[1] != RT_EMPTY) + (r[2] != RT_EMPTY) + (r[3] != RT_EMPTY);
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
