@@ -247,8 +247,8 @@ typedef enum {
                              with 32 lanes to 4 by the number of rays; DIRS sets:
                              WIDE where neighbouring Gaussians lie close
                              together (measured on the tree), else RAY_WIDE;
-                             ENV and HEMI sets: RAY_WIDE up to 2^19 rays,
-                             RAY_REFILL beyond; explicit
+                             ENV and HEMI sets: RAY_WIDE up to 2^17 or 2^18
+                             rays, RAY_REFILL beyond; explicit
                              rays and id lists: as WARP_RAY up to 2^22 rays,
                              32 lanes up to 8192 rays, 16 up to 2^16, 8 up to
                              2^18 or over more than 2^20 Gaussians, 4 beyond

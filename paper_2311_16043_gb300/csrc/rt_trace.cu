@@ -141,17 +141,30 @@ int lanes_for(int64_t m, const BvhDev &b) {
     return m <= 262144 || b.levels > 36 || b.n > (int64_t(1) << 20) ? 8 : 4;
 }
 
-// A full set traced by groups of lanes.  Hemisphere sets, us, lanes against the
-// better of one thread per ray and lane refill: uniform 3k x 8 52 / 152, x 32
-// 139 / 215; 30k x 8 814 / 1,497, x 32 2,786 / 3,148; object 4k x 8 57 / 81, x 16
-// 97 / 85, x 32 112 / 95; 20k x 16 310 / 309; 300k x 4 2,541 / 2,834, x 8 4,987 /
-// 4,520 (environment sets lie 5 % the other way at the ends).  Direction sets
-// against shaft packets or one thread per ray: uniform 3k x 8 52 / 80, x 32
-// 118 / 103; 30k x 1 144 / 247, x 4 398 / 258; object 4k x 8 55 / 90, x 16 94 /
-// 85; 500 x 16 26 / 26, x 64 42 / 28.
+// A full set traced by groups of lanes.  Hemisphere and environment sets, us,
+// lanes against one thread per ray or lane refill, whichever is less, by the rays
+// per shaft group (how dense the scene is):
+//   uniform 1k: x 16 30 / 66 and 36 / 67; 2k (5): x 32 96 / 138 and 113 / 139
+//   uniform 10 to 28: 4k x 16 122 / 204 and 141 / 211, x 32 205 / 262 and 244 / 268;
+//     20k x 16 (320k rays) 870 / 1,095 and 1,001 / 1,108, x 32 1,625 / 1,690 and
+//     1,897 / 1,725; 60k x 8 (480k) 1,695 / 1,860 and 1,912 / 1,882
+//   object 2 (4k): x 8 57 / 70 and 67 / 72, x 12 78 / 86 and 91 / 78, x 16 99 / 83
+//     and 117 / 83
+//   object 8 (20k): x 8 200 / 242 and 266 / 274, x 16 338 / 330 and 438 / 378, x 32
+//     627 / 471 and 827 / 552
+//   object 11 to 24: 60k x 4 (240k rays) 461 / 490 and 572 / 552, x 8 704 / 670 and
+//     913 / 770; 400k x 2 1,982 / 2,110
+// A lane group works out a ray's direction in every lane, which environment
+// samples make long.  Direction sets against shaft packets or one thread per ray:
+// uniform 3k x 8 52 / 80, x 32 118 / 103; 30k x 1 144 / 247, x 4 398 / 258; object
+// 4k x 8 55 / 90, x 16 94 / 85; 500 x 16 26 / 26, x 64 42 / 28.
 bool small_set_takes_lanes(const rt_bvh *bvh, int32_t kind, int32_t K, int64_t rays) {
     if (kind == RT_RAYS_DIRS) return rays <= (int64_t(1) << 15) && K <= 16;
-    return rays <= (int64_t(1) << 20) && K <= (rt_shaft_pays(bvh) ? 32 : 16);
+    const bool dense = bvh->n >= 9 * bvh->n_groups, denser = bvh->n >= 16 * bvh->n_groups;
+    if (rays > (int64_t(1) << (K <= 2 ? 20 : denser ? 19 : 18))) return false;
+    if (K <= 8 || dense) return K <= 32;
+    if (K <= 16 && (kind == RT_RAYS_HEMI || rays <= (int64_t(1) << 14))) return true;
+    return K <= 32 && rt_shaft_pays(bvh) && rays <= (int64_t(1) << 17);
 }
 
 // No more blocks than the rays need, and with 32 lanes, for few rays, the nodes
@@ -258,17 +271,18 @@ rt_status rt_trace_launch(const rt_bvh *bvh, const rt_rayspec *rays, float *T_ou
     //   18 %, 300k 5 %, 500k 2.7 % in favour of the first; from 1M on the
     //   packets win);
     // - env-map and hemisphere sets (directions differ across a tile): the
-    //   per-ray walk with lane refill, up to 2^19 rays one thread per ray, whose
-    //   latency is lower (hemisphere sets, us, thread / refill: object 4k x 64
-    //   118 / 146, 20k x 32 496 / 584, 20k x 64 840 / 814, uniform 3k x 128
-    //   439 / 432);
+    //   per-ray walk with lane refill, up to 2^18 rays (2^17 in dense scenes)
+    //   one thread per ray, whose latency is lower (environment sets, us, thread /
+    //   refill: object 4k x 32 102 / 125, x 64 143 / 157, 20k x 16 428 / 378; uniform
+    //   4k x 32 280 / 268, x 64 418 / 329);
     // - explicit rays and id lists (scattered rays): a group of lanes per ray
     //   up to 2^22 rays (lanes_for; one thread per ray takes 570 us for 2,000
     //   rays of the 300k scene, 2.4 ms for 600,000), and one thread per ray
     //   over the 4-wide tree for longer lists, which are sorted.
+    const int64_t thread_max = int64_t(1) << (bvh->n >= 9 * bvh->n_groups ? 17 : 18);
     if (o.kernel == RT_KERNEL_AUTO && job.mode == MODE_FULL)
         strat = !o.counters && !o.hit_ids && small_set_takes_lanes(bvh, rays->kind, rs.K, count) ? 6
-                : rays->kind != RT_RAYS_DIRS ? (count <= (int64_t(1) << 19) ? 4 : 5)
+                : rays->kind != RT_RAYS_DIRS ? (count <= thread_max ? 4 : 5)
                 : o.counters || o.hit_ids  ? (bvh->n <= (int64_t(1) << 19) ? 4 : 2)
                 : rt_shaft_pays(bvh)       ? 2
                                            : 4;
