@@ -941,7 +941,7 @@ def main():
                 "algorithmic_bytes_per_launch": alg_bytes,
                 "per_ray": {"box_tests": box_tests / R, "gaussian_tests": gauss_tests / R,
                             "accepted_hits": hits / R,
-                            "counted_on": "the plain packet walk, whose rays share no test"},
+                            "counted_on": "one thread per ray, whose rays share no test"},
                 "bytes_model": "44 B per Gaussian read once + 4 B per ray written; the kernel is bound by instruction "
                                "issue (profiles/)"}
 

@@ -246,7 +246,8 @@ typedef enum {
                              HEMI up to 2^20, few per Gaussian): as WARP_RAY
                              with 32 lanes to 4 by the number of rays; DIRS sets:
                              WIDE where neighbouring Gaussians lie close
-                             together (measured on the tree), else RAY_WIDE;
+                             together (measured on the tree), else RAY_WIDE,
+                             as with counters or a hit log;
                              ENV and HEMI sets: RAY_WIDE up to 2^17 or 2^18
                              rays, RAY_REFILL beyond; explicit
                              rays and id lists: as WARP_RAY up to 2^22 rays,

@@ -26,13 +26,16 @@
 
 namespace {
 
+// Packets of rays with directions of their own take 60 registers where they are
+// let, which costs the ninth block and 2 to 3 %.
 template <int STRAT, bool COUNT>
-__global__ void __launch_bounds__(128, STRAT == 5 ? RT_REFILL_MIN_BLOCKS : RT_TRACE_MIN_BLOCKS)
+__global__ void __launch_bounds__(128, STRAT == 5 ? RT_REFILL_MIN_BLOCKS : STRAT == 2 && !COUNT ? 9 : RT_TRACE_MIN_BLOCKS)
     k_trace(BvhDev b, RaySetDev rs, TraceJob job, float *T_out, TraceAux aux, unsigned long long *work) {
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
-    __shared__ int2 stk_all[STRAT == 2 ? 4 * RT_WIDE_STACK : 1];
-    int2 *stk = stk_all + (STRAT == 2 ? (threadIdx.x >> 5) * RT_WIDE_STACK : 0);
+    constexpr bool packet = STRAT == 2 || STRAT == 3;
+    __shared__ int2 stk_all[packet ? 4 * RT_WIDE_STACK : 1];
+    int2 *stk = stk_all + (packet ? (threadIdx.x >> 5) * RT_WIDE_STACK : 0);
     WorkCounts wc = {0, 0, 0};
     unsigned long long rays_done = 0;
     if constexpr (STRAT == 5) {  // per-ray slots with lane refill (full implicit sets)
@@ -265,11 +268,9 @@ rt_status rt_trace_launch(const rt_bvh *bvh, const rt_rayspec *rays, float *T_ou
     // - a small full set: a group of lanes per ray (lanes_for), which is bound
     //   by one ray's latency less than the others (small_set_takes_lanes);
     // - a direction set: shaft packets where the groups are large enough
-    //   (rt_shaft_pays), else one thread per ray, farthest child first.  With
-    //   counters or a hit log, which shaft packets do not keep: one thread per
-    //   ray up to 2^19 Gaussians, plain packets beyond (object scenes: 100k
-    //   18 %, 300k 5 %, 500k 2.7 % in favour of the first; from 1M on the
-    //   packets win);
+    //   (rt_shaft_pays), else one thread per ray, farthest child first, as with
+    //   counters or a hit log, which shaft packets do not keep (2M object scene x
+    //   8, counted 96 ms, packets 102; 600k x 16 31 / 36);
     // - env-map and hemisphere sets (directions differ across a tile): the
     //   per-ray walk with lane refill, up to 2^18 rays (2^17 in dense scenes)
     //   one thread per ray, whose latency is lower (environment sets, us, thread /
@@ -283,9 +284,8 @@ rt_status rt_trace_launch(const rt_bvh *bvh, const rt_rayspec *rays, float *T_ou
     if (o.kernel == RT_KERNEL_AUTO && job.mode == MODE_FULL)
         strat = !o.counters && !o.hit_ids && small_set_takes_lanes(bvh, rays->kind, rs.K, count) ? 6
                 : rays->kind != RT_RAYS_DIRS ? (count <= thread_max ? 4 : 5)
-                : o.counters || o.hit_ids  ? (bvh->n <= (int64_t(1) << 19) ? 4 : 2)
-                : rt_shaft_pays(bvh)       ? 2
-                                           : 4;
+                : !o.counters && !o.hit_ids && rt_shaft_pays(bvh) ? 2
+                                                                  : 4;
     if (o.kernel == RT_KERNEL_AUTO && job.mode != MODE_FULL) strat = count <= (int64_t(1) << 22) ? 6 : 4;
     // lanes per ray keep no hit log
     if (strat == 6 && o.hit_ids) strat = 4;
@@ -295,7 +295,8 @@ rt_status rt_trace_launch(const rt_bvh *bvh, const rt_rayspec *rays, float *T_ou
     if ((strat == 4 || strat == 6) && bvh->n_wide == 0) strat = 0;  // fewer than two Gaussians
     // a shared direction: shaft packets, which count no single ray's tests and
     // keep no hit log (then the plain packet walk)
-    if (strat == 2 && job.mode == MODE_FULL && rays->kind == RT_RAYS_DIRS && !o.counters && !o.hit_ids) strat = 3;
+    const bool shared_dir = job.mode == MODE_FULL && rays->kind == RT_RAYS_DIRS;
+    if (strat == 2 && shared_dir && !o.counters && !o.hit_ids) strat = 3;
 
     TraceAux aux;
     aux.counters = (unsigned long long *)o.counters;
@@ -372,6 +373,7 @@ rt_status rt_trace_launch(const rt_bvh *bvh, const rt_rayspec *rays, float *T_ou
             int grid = persistent_blocks((const void *)k_trace_shaft, threads);
             k_trace_shaft<<<grid, threads, 0, st>>>(b, rs, job, T_out, aux.status, work);
         }
+        else if (strat == 2 && shared_dir) { if (count) RT_LAUNCH(3, true); else RT_LAUNCH(3, false); }
         else if (strat == 2) { if (count) RT_LAUNCH(2, true); else RT_LAUNCH(2, false); }
         else if (strat == 1) { if (count) RT_LAUNCH(1, true); else RT_LAUNCH(1, false); }
         else { if (count) RT_LAUNCH(0, true); else RT_LAUNCH(0, false); }
