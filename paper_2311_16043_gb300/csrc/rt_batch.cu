@@ -34,10 +34,13 @@ rt_status rt_trace_launch_job(const BvhDev &b, const RaySetDev &rs, const TraceJ
 
 namespace {
 
+// What decides between the strategies: for direction sets also whether shaft
+// groups hold many rays (rt_shaft_pays; two scenes of 4k with 1.8 and 10 a group:
+// shafts 0.5 and 2 times as fast as one thread per ray).
 struct TuneKey {
-    int dev, log2n, kind, K;
+    int dev, log2n, kind, K, shaft;
     bool operator<(const TuneKey &o) const {
-        return std::tie(dev, log2n, kind, K) < std::tie(o.dev, o.log2n, o.kind, o.K);
+        return std::tie(dev, log2n, kind, K, shaft) < std::tie(o.dev, o.log2n, o.kind, o.K, o.shaft);
     }
 };
 std::mutex g_tune_mu;
@@ -221,7 +224,7 @@ extern "C" rt_status rt_trace_autotune(const rt_bvh *bvh, const rt_rayspec *rays
     cudaGetDevice(&dev);
     int log2n = 0;
     while ((1ll << (log2n + 1)) <= bvh->n) ++log2n;
-    const TuneKey key{dev, log2n, rays->kind, rs.K};
+    const TuneKey key{dev, log2n, rays->kind, rs.K, rays->kind == RT_RAYS_DIRS && rt_shaft_pays(bvh)};
     {
         std::lock_guard<std::mutex> g(g_tune_mu);
         auto it = g_tune_cache.find(key);
