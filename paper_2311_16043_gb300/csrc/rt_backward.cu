@@ -521,11 +521,8 @@ struct ShaftGrad {
     }
 };
 
-#ifndef RT_GRAD_MIN_BLOCKS
-#define RT_GRAD_MIN_BLOCKS 4
-#endif
 template <bool DET>
-__global__ void __launch_bounds__(128, RT_GRAD_MIN_BLOCKS) k_shaft_backward(BvhDev b, RaySetDev rs, int64_t n_items,
+__global__ void __launch_bounds__(128, 4) k_shaft_backward(BvhDev b, RaySetDev rs, int64_t n_items,
                                                                             ShaftGrad<DET> init, int *status,
                                                                             unsigned long long *work) {
     __shared__ ShaftSmem<true> sm_all[4];

@@ -51,12 +51,12 @@ constexpr float kTuneMargin = 0.97f;
 
 // The strategy used without tuning: for a direction set over more than 20,000
 // Gaussians shaft packets where they pay (rt_shaft_pays; uniform 30k x 32
-// directions 1.2 ms against 4.4), else one thread per ray on the 4-wide tree
-// (far-first; jobs of up to 20,000 keep the strategy they always reported
-// here, tuning finds the faster one: uniform 4k 0.13 ms against 0.30); one thread per ray on the
-// 4-wide tree with lane refill for env-map and hemisphere rays (their
-// directions differ within a tile); binary variants when there is no 4-wide
-// tree.
+// directions 1.2 ms against 4.4), else one thread per ray on the 4-wide tree,
+// farthest child first.  The line at 20,000 is not where shafts begin to pay
+// (uniform 4k 0.13 ms against 0.30, which tuning finds): smaller jobs are reported
+// as RT_KERNEL_RAY_WIDE, and callers may hold to that (tests/test_gpu_batch.py
+// does).  Env-map and hemisphere rays, whose directions differ within a tile: one
+// thread per ray with lane refill.  Binary variants when there is no 4-wide tree.
 int default_kernel(const rt_bvh *bvh, int32_t kind) {
     if (kind == RT_RAYS_DIRS) {
         if (bvh->n_wide == 0) return RT_KERNEL_PACKET;
@@ -130,11 +130,8 @@ __device__ __forceinline__ void batch_refill(const BatchJobDev *__restrict__ job
 // refill jobs after them.  As two launches the second starts on the first's
 // longest rays: untuned batches of four object scenes of 2 to 7 thousand
 // Gaussians 366 us against 329.
-#ifndef RT_BATCH_MIN_BLOCKS
-#define RT_BATCH_MIN_BLOCKS 8
-#endif
 template <bool REFILL>
-__global__ void __launch_bounds__(128, RT_BATCH_MIN_BLOCKS)
+__global__ void __launch_bounds__(128, 8)
     k_trace_batch(const BatchJobDev *__restrict__ jobs, int n_item_jobs, int64_t total_items, int n_jobs,
                   int64_t total_slots, int *status, unsigned long long *work) {
     const unsigned FULL = 0xffffffffu;
@@ -173,7 +170,7 @@ __global__ void __launch_bounds__(128, RT_BATCH_MIN_BLOCKS)
     }
 }
 
-__global__ void __launch_bounds__(128, RT_REFILL_MIN_BLOCKS) k_refill_batch(const BatchJobDev *__restrict__ jobs, int n_jobs,
+__global__ void __launch_bounds__(128, kRefillBlocks) k_refill_batch(const BatchJobDev *__restrict__ jobs, int n_jobs,
                                                                             int64_t total_slots, int *status,
                                                                             unsigned long long *work) {
     batch_refill(jobs, 0, n_jobs, total_slots, status, work);
@@ -181,7 +178,7 @@ __global__ void __launch_bounds__(128, RT_REFILL_MIN_BLOCKS) k_refill_batch(cons
 
 // The shaft jobs [0, n_jobs) of a batch, their (group, direction) items one
 // queue.
-__global__ void __launch_bounds__(128, RT_SHAFT_MIN_BLOCKS) k_shaft_batch(const BatchJobDev *__restrict__ jobs, int n_jobs,
+__global__ void __launch_bounds__(128, kShaftBlocks) k_shaft_batch(const BatchJobDev *__restrict__ jobs, int n_jobs,
                                                                           int64_t total_items, int *status,
                                                                           unsigned long long *work) {
     __shared__ ShaftSmem<false> sm[4];

@@ -64,13 +64,10 @@ __device__ __forceinline__ bool top_slab(const float *bx, float3 oi, float3 inv)
     return slab(bx[0], bx[3], bx[1], bx[4], bx[2], bx[5], oi, inv);
 }
 
-#ifndef RT_SCENE_MIN_BLOCKS
-#define RT_SCENE_MIN_BLOCKS 8
-#endif
 // rs: an implicit ray set over the scene's rows (row = g_base of the
 // instance + the Gaussian's original index): DIRS, HEMI (world-frame normals
 // per row) or ENV (ray id row * K + k keys the sample).
-__global__ void __launch_bounds__(128, RT_SCENE_MIN_BLOCKS) k_scene_trace(const InstDev *__restrict__ inst, int n_inst,
+__global__ void __launch_bounds__(128, 8) k_scene_trace(const InstDev *__restrict__ inst, int n_inst,
                                                      const TopNode *__restrict__ top, uint32_t root_ref,
                                                      const float *__restrict__ root_box, RaySetDev rs, float t_min,
                                                      int64_t total_items, float *__restrict__ T_out, int *status,

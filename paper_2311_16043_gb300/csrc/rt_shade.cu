@@ -350,7 +350,7 @@ __global__ void __launch_bounds__(128, 8) k_trace_reduce(BvhDev b, RaySetDev rs,
 
 // Ambient occlusion of a direction set: an item is a shaft group, traced
 // along the K directions in turn, each lane summing its (up to two) rays.
-__global__ void __launch_bounds__(128, RT_SHAFT_MIN_BLOCKS) k_shaft_ao(BvhDev b, RaySetDev rs, int64_t n_groups,
+__global__ void __launch_bounds__(128, kShaftBlocks) k_shaft_ao(BvhDev b, RaySetDev rs, int64_t n_groups,
                                                                        float *__restrict__ ao, int *status,
                                                                        unsigned long long *work) {
     __shared__ ShaftSmem<false> sm_all[4];

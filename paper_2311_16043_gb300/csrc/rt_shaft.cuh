@@ -553,6 +553,4 @@ __device__ __forceinline__ void shaft_item(const BvhDev &b, const RaySetDev &rs,
 }
 
 // Resident blocks of 128 threads per SM: 37 KB of shared memory each.
-#ifndef RT_SHAFT_MIN_BLOCKS
-#define RT_SHAFT_MIN_BLOCKS 6
-#endif
+constexpr int kShaftBlocks = 6;

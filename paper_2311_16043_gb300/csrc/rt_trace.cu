@@ -19,17 +19,15 @@
 
 #include "rt_shaft.cuh"
 
-// Resident blocks per SM the trace kernels are compiled for (register cap).
-#ifndef RT_TRACE_MIN_BLOCKS
-#define RT_TRACE_MIN_BLOCKS 8
-#endif
-
 namespace {
+
+// Resident blocks per SM the trace kernels are compiled for (register cap).
+constexpr int kTraceBlocks = 8;
 
 // Packets of rays with directions of their own take 60 registers where they are
 // let, which costs the ninth block and 2 to 3 %.
 template <int STRAT, bool COUNT>
-__global__ void __launch_bounds__(128, STRAT == 5 ? RT_REFILL_MIN_BLOCKS : STRAT == 2 && !COUNT ? 9 : RT_TRACE_MIN_BLOCKS)
+__global__ void __launch_bounds__(128, STRAT == 5 ? kRefillBlocks : STRAT == 2 && !COUNT ? 9 : kTraceBlocks)
     k_trace(BvhDev b, RaySetDev rs, TraceJob job, float *T_out, TraceAux aux, unsigned long long *work) {
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
@@ -61,7 +59,7 @@ __global__ void __launch_bounds__(128, STRAT == 5 ? RT_REFILL_MIN_BLOCKS : STRAT
 
 // Strategy 6: a group of lanes per ray.
 template <int LANES, bool COUNT>
-__global__ void __launch_bounds__(128, RT_TRACE_MIN_BLOCKS) k_trace_lanes(BvhDev b, RaySetDev rs, TraceJob job,
+__global__ void __launch_bounds__(128, kTraceBlocks) k_trace_lanes(BvhDev b, RaySetDev rs, TraceJob job,
                                                                           float *T_out, TraceAux aux,
                                                                           unsigned long long *work) {
     __shared__ uint32_t stk[128 * kLaneStack<LANES>];
@@ -74,7 +72,7 @@ __global__ void __launch_bounds__(128, RT_TRACE_MIN_BLOCKS) k_trace_lanes(BvhDev
 }
 
 // Strategy 3 of a direction set: an item is a shaft group and a direction.
-__global__ void __launch_bounds__(128, RT_SHAFT_MIN_BLOCKS) k_trace_shaft(BvhDev b, RaySetDev rs, TraceJob job,
+__global__ void __launch_bounds__(128, kShaftBlocks) k_trace_shaft(BvhDev b, RaySetDev rs, TraceJob job,
                                                                           float *T_out, int *status,
                                                                           unsigned long long *work) {
     __shared__ ShaftSmem<false> sm[4];

@@ -905,18 +905,10 @@ __device__ __forceinline__ void flush_counts(const TraceAux &aux, const WorkCoun
 //   nodes not kept in L1                          28.7   18.9   11.5
 // The quantized boxes cost 1.5 % more nodes and Gaussians, the nodes 64 bytes a
 // Gaussian and 4 us of the build at 4k, 13 at 300k.
-#ifndef RT_REFILL_MIN_BLOCKS
-#define RT_REFILL_MIN_BLOCKS 9
-#endif
-#ifndef RT_REFILL_MIN
-#define RT_REFILL_MIN 6
-#endif
-constexpr int kRefillMin = RT_REFILL_MIN;
+constexpr int kRefillBlocks = 9;  // resident a multiprocessor
+constexpr int kRefillMin = 6;
 constexpr int kLeafQueue = 8;
-#ifndef RT_STACK_SHARED
-#define RT_STACK_SHARED 24
-#endif
-constexpr int kStackShared = RT_STACK_SHARED;
+constexpr int kStackShared = 24;
 
 // `Src` is what the rays come from: slots(), fetch(slot, o, d, src) (false past
 // a ragged last tile; remembers where the slot's T goes), tree(), far() and
@@ -1063,10 +1055,7 @@ __device__ __forceinline__ void trace_refill(const BvhDev &b, const RaySetDev &r
 // lanes 2.02, 64-byte nodes 1.65, leaf queue (12 lanes waiting) 1.38, stacks of
 // 144 entries instead of 256 (more warps, and an L1 that holds something: hit
 // rate 0.02 before) 1.32; 1M rays of the 2M scene 7.9 -> 6.4 by the last alone.
-#ifndef RT_LANE_LEAF_MIN
-#define RT_LANE_LEAF_MIN 10
-#endif
-constexpr int kLaneLeafMin = RT_LANE_LEAF_MIN;
+constexpr int kLaneLeafMin = 10;
 template <int LANES>
 constexpr int kLaneStack = LANES == 4 ? 36 : LANES == 8 ? 28 : LANES == 16 ? 18 : 12;  // entries per lane
 template <int LANES, bool COUNT>
