@@ -392,7 +392,7 @@ rt_status rt_scene_destroy(rt_scene *scene, rt_stream_t stream);
  *   env[env_h*env_w*3] = the global RGB direct light, equirectangular, row i
  *     over polar angles [i pi/h, (i+1) pi/h] from +z, column j over azimuths
  *     [2 pi j/w, 2 pi (j+1)/w], looked up bilinearly between pixel centres
- *     (azimuth wraps, polar angle clamps); env_h*env_w <= 8192;
+ *     (azimuth wraps, polar angle clamps); env_h*env_w <= 2048;
  *   cam = camera centre, host floats: wo = (cam - mu)/|cam - mu|.           */
 typedef struct {
     const float *albedo;
@@ -414,7 +414,9 @@ typedef struct {
  * k = (r+1)^2/8, normalised half vector, n.wi and n.wo clamped at 0.
  * V[n*K] (device, the visibility of the rays as rt_trace_visibility writes
  * it) or NULL: then the rays are traced in the same kernel and V is never
- * written (one warp per 32 Morton-adjacent Gaussians, all K rays each).
+ * written (one warp per 32 Morton-adjacent Gaussians, all K rays each).  The two
+ * forms sum the SH light in different frames, so they agree up to rounding, not
+ * bit for bit.
  * rgb[n*3] device output.  Errors: RT_ERR_INVALID_ARG (wrong ray kind,
  * missing arrays, map too large). */
 rt_status rt_pbr_shade(const rt_bvh *bvh, const rt_rayspec *rays, const float *V, const rt_pbr_inputs *in,
@@ -600,11 +602,14 @@ typedef struct {
     float *T_out;
 } rt_batch_job;
 
-/* Prepares one persistent launch over all jobs: a device work queue of
- * 32-ray items ordered scene by scene, largest estimated cost first; each
- * job's strategy and work order from rt_trace_autotune (autotune != 0) or the
- * defaults.  The queue reset and the launch are captured once into a CUDA
- * graph.  Jobs' trees, ray sets and outputs must stay alive until
+/* Prepares the launches of all jobs: one over the shaft packets of direction
+ * sets (RT_KERNEL_WIDE), one over all other jobs, as far as there are such; each
+ * drains device work queues ordered job by job, largest estimated cost first.
+ * Each job's strategy and work order come from rt_trace_autotune (autotune != 0)
+ * or the defaults; fewer than 2^17 rays of shaft packets beside other jobs become
+ * RT_KERNEL_RAY_WIDE.  A job's T is what rt_trace_visibility gives with its
+ * reported kernel, bit for bit.  The queues' reset and the launches are captured
+ * once into a CUDA graph.  Jobs' trees, ray sets and outputs must stay alive until
  * rt_batch_destroy.  At most 4096 jobs.  Synchronises `stream`. */
 rt_status rt_batch_create(const rt_batch_job *jobs, int32_t n_jobs, int32_t autotune, rt_stream_t stream,
                           rt_batch **out);

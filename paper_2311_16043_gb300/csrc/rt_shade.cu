@@ -453,10 +453,14 @@ template <int LANES>
 rt_status shade_lanes(const rt_bvh *bvh, const ShadeDev &S, const float *V, float *rgb, size_t smem, cudaStream_t st) {
     const bool vec = S.K % 4 == 0 && ((uintptr_t)V & 15u) == 0;
     smem += 2 * sizeof(float4) * (size_t)(S.K < kShadeChunk ? S.K : kShadeChunk);
+    // a block a multiprocessor always fits, and a small set's call is bound by the
+    // host: the occupancy query is 0.3 us of its 8
     const int64_t blocks = (bvh->n * LANES + 127) / 128;
 #define RT_SHADE(SH, VEC)                                                                            \
     do {                                                                                             \
-        const int64_t cap = grid_for((const void *)k_pbr_shade_v<LANES, SH, VEC>, 128, smem);        \
+        const int64_t cap = blocks <= rt_num_sms()                                                   \
+                                ? blocks                                                             \
+                                : grid_for((const void *)k_pbr_shade_v<LANES, SH, VEC>, 128, smem);  \
         k_pbr_shade_v<LANES, SH, VEC>                                                                \
             <<<(unsigned)(blocks < cap ? blocks : cap), 128, smem, st>>>(bvh_dev(bvh), S, V, rgb);   \
     } while (0)

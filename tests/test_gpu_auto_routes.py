@@ -39,3 +39,21 @@ def test_full_sets(scene, n, k, kind):
     assert bool((((b - a).abs() <= tol * a) | (torch.maximum(a, b) <= 1e-4 * (1 + tol))).all())
     if env is not None:
         env.destroy()
+
+
+@pytest.mark.parametrize("n,k", [(3000, 8), (20_000, 16), (60_000, 16)])
+def test_a_list_and_the_full_set_agree(n, k):
+    """The same ray in a full set and in an id list: AUTO may take different
+    walks, whose factors come in another order, so the last bits may differ."""
+    from paper_2311_16043_gb300 import rt
+    sc = scenes.object_scene(n, 3)
+    bvh = rt.rt_build_bvh(*(_dev(sc[x]) for x in ("mean", "scale", "quat", "opacity")))
+    nrm = scenes.shortest_axis_normals(sc["scale"], sc["quat"])
+    kw = dict(dirs=_dev(scenes.fibonacci_hemisphere(k)), normals=_dev(nrm))
+    ids = _dev(scenes.sample_ray_ids(n * k, 9000, 5))
+    a = rt.rt_trace_visibility(bvh, rt.rayspec(rt.RT_RAYS_HEMI, **kw)).double()[ids]
+    b = rt.rt_trace_visibility(bvh, rt.rayspec(rt.RT_RAYS_HEMI, ray_ids=ids, **kw)).double()
+    torch.cuda.synchronize()
+    assert rt.rt_status_last() == 0
+    tol = 2 * 1024 * 2.0 ** -24
+    assert bool((((b - a).abs() <= tol * a) | (torch.maximum(a, b) <= 1e-4 * (1 + tol))).all())
