@@ -278,7 +278,8 @@ __device__ __forceinline__ void shaft_group(const BvhDev &b, float eps, float3 d
     const unsigned lt = (1u << lane) - 1u;
     const float inf = __int_as_float(0x7f800000);
     float3 inv, oi;
-    const bool finite = qnode_ray(make_float3(0.f, 0.f, 0.f), d, inv, oi);
+    // false: the rays meet nothing (their boxes' tests, all NaN, would let every node pass)
+    const bool finite = qnode_ray(make_float3(eps * d.x, eps * d.y, eps * d.z), d, inv, oi);
     int live = count;
     if constexpr (GRAD) live = 0;
 #pragma unroll
@@ -356,7 +357,7 @@ __device__ __forceinline__ void shaft_group(const BvhDev &b, float eps, float3 d
     // step 2: 16-byte row r of staged record i lies at chunk r ^ ((i >> 1) & 3)
     auto rec = [&](int i, int r) { return sm.stage[4 * i + (r ^ ((i >> 1) & 3))]; };
     const int room = kShaftStack - 4 - 3 * b.levels;  // beyond it, nodes are walked one at a time
-    int bound = live, size = finite ? 1 : 0, nleaf = 0;  // a direction that is not finite meets nothing
+    int bound = live, size = finite ? 1 : 0, nleaf = 0;
     (void)bound;
     __syncwarp();
     for (;;) {

@@ -92,3 +92,16 @@ def test_directions_of_any_length(length):
     assert rt.rt_status_last() == 0
     assert a.min().item() < 0.5
     assert bool(((b - a).abs() <= 2 * 512 * 2.0 ** -24 * a).all()), ((b - a).abs() / a).max().item()
+
+
+@pytest.mark.parametrize("eps", [float("inf"), 3e38])
+def test_origins_that_are_not_finite(eps):
+    """Origins at infinity: nothing is met, and nothing is walked to find that."""
+    from paper_2311_16043_gb300 import rt
+    sc = scenes.uniform_scene(700, 6)
+    dirs = 2.0 * scenes.fibonacci_sphere(6)
+    bvh = rt.rt_build_bvh(*(_dev(sc[k]) for k in ("mean", "scale", "quat", "opacity")), rt.params(origin_eps=eps))
+    a, b = (rt.rt_trace_visibility_dirs(bvh, _dev(dirs), opts=rt.trace_opts(kernel=k)) for k in (1, 3))
+    torch.cuda.synchronize()
+    assert rt.rt_status_last() == 0
+    assert torch.equal(a, torch.ones_like(a)) and torch.equal(a, b)
