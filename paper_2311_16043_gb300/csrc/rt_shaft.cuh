@@ -137,8 +137,8 @@ __device__ __forceinline__ void shaft_qnode(const float4 *__restrict__ q, int h,
                  y1 = dist(sy ? ly : hy, ay, fy), z0 = dist(sz ? hz : lz, az, nz), z1 = dist(sz ? lz : hz, az, fz);
     const float na = fmaxf(fmaxf(x0.x, y0.x), fmaxf(z0.x, 0.0f)), fa = fminf(fminf(x1.x, y1.x), z1.x);
     const float nb = fmaxf(fmaxf(x0.y, y0.y), fmaxf(z0.y, 0.0f)), fb = fminf(fminf(x1.y, y1.y), z1.y);
-    h0 = !(na > fmaf(fabsf(fa), 1e-6f, fa)) && r0 != RT_EMPTY;
-    h1 = !(nb > fmaf(fabsf(fb), 1e-6f, fb)) && r1 != RT_EMPTY;
+    h0 = !(na > kFarMargin * fa) && r0 != RT_EMPTY;
+    h1 = !(nb > kFarMargin * fb) && r1 != RT_EMPTY;
 }
 
 // Two Gaussians as the rays of a shaft see them (step 2).

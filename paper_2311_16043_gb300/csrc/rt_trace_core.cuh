@@ -168,6 +168,10 @@ __device__ __forceinline__ bool qnode_ray(float3 o, float3 d, float3 &inv, float
 // L1 data pipe, a wavefront per lane and load.  Not kept in L1, which these
 // walks hit 0.2 of the time and whose fills cost the same pipe (2 to 2.5 %);
 // CACHED: kept, for walks bound by a ray's latency.
+// kFarMargin: slab's relative allowance on the far distance.  A box behind a ray
+// from so far off that o inv overflows has it at -inf, where fa + 1e-6 |fa| would
+// be NaN and pass: each such ray would walk the whole tree.
+constexpr float kFarMargin = 1.0000011f;
 template <bool CACHED = false>
 __device__ __forceinline__ void qnode_near(const float4 *__restrict__ q, float3 inv, float3 oi, float (&tn)[4],
                                            uint32_t (&r)[4]) {
@@ -197,8 +201,8 @@ __device__ __forceinline__ void qnode_near(const float4 *__restrict__ q, float3 
                      nz2 = dist(nz, az, cz), fz2 = dist(fz, az, cz);
         const float na = fmaxf(fmaxf(nx2.x, ny2.x), fmaxf(nz2.x, 0.0f)), fa = fminf(fminf(fx2.x, fy2.x), fz2.x);
         const float nb = fmaxf(fmaxf(nx2.y, ny2.y), fmaxf(nz2.y, 0.0f)), fb = fminf(fminf(fx2.y, fy2.y), fz2.y);
-        tn[2 * pr] = !(na > fmaf(fabsf(fa), 1e-6f, fa)) && r[2 * pr] != RT_EMPTY ? na : inf;
-        tn[2 * pr + 1] = !(nb > fmaf(fabsf(fb), 1e-6f, fb)) && r[2 * pr + 1] != RT_EMPTY ? nb : inf;
+        tn[2 * pr] = !(na > kFarMargin * fa) && r[2 * pr] != RT_EMPTY ? na : inf;
+        tn[2 * pr + 1] = !(nb > kFarMargin * fb) && r[2 * pr + 1] != RT_EMPTY ? nb : inf;
     }
 }
 

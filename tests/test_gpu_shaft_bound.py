@@ -105,3 +105,25 @@ def test_origins_that_are_not_finite(eps):
     torch.cuda.synchronize()
     assert rt.rt_status_last() == 0
     assert torch.equal(a, torch.ones_like(a)) and torch.equal(a, b)
+
+
+@pytest.mark.parametrize("far", [1e27, -1e30, 3e38])
+def test_rays_from_far_off_walk_no_tree(far):
+    """Axis-parallel rays whose o / d overflows meet no box (at most the root's
+    children are tested, 4 a node)."""
+    from paper_2311_16043_gb300 import rt
+    sc = scenes.uniform_scene(700, 6)
+    bvh = rt.rt_build_bvh(*(_dev(sc[k]) for k in ("mean", "scale", "quat", "opacity")))
+    o = np.zeros((300, 3))
+    o[np.arange(300), np.arange(300) % 3] = far
+    d = np.zeros((300, 3))
+    d[np.arange(300), (np.arange(300) + 1) % 3] = 1.0
+    d[::2] *= -1.0
+    rs = rt.rayspec(rt.RT_RAYS_EXPLICIT, ray_o=_dev(o), ray_d=_dev(d))
+    for kernel in (0, 4, 6):
+        cnt = torch.zeros(4, dtype=torch.int64, device="cuda")
+        T = rt.rt_trace_visibility(bvh, rs, opts=rt.trace_opts(kernel=kernel, counters=cnt))
+        torch.cuda.synchronize()
+        assert rt.rt_status_last() == 0
+        assert bool((T == 1).all())
+        assert int(cnt[0]) <= 4 * 300 and int(cnt[1]) == 0
