@@ -185,6 +185,7 @@ __device__ __forceinline__ void shaft_cand(const ShaftSmem<GRAD> &sm, const floa
     const float2 b0 = dot2(w0, F4), b1 = dot2(w1, F4), b2 = dot2(w2, F4);
     const float2 n0 = dot2(w0, w0), n1 = dot2(w1, w1), n2 = dot2(w2, w2);
     auto rcp = [](float2 v) { return make_float2(__fdividef(1.0f, v.x), __fdividef(1.0f, v.y)); };
+    auto rsq = [](float2 v) { return make_float2(rsqrtf(v.x), rsqrtf(v.y)); };
     auto mul = [](float2 x, float2 y) { return __fmul2_rn(x, y); };
     auto fma2 = [](float2 x, float2 y, float2 z) { return __ffma2_rn(x, y, z); };
     const float2 f0 = mul(b0, rcp(n0)), f1 = mul(b1, rcp(n1)), f2 = mul(b2, rcp(n2));
@@ -192,11 +193,11 @@ __device__ __forceinline__ void shaft_cand(const ShaftSmem<GRAD> &sm, const floa
     const float2 B = fma2(mul(a0, rcp(n0)), f0, fma2(mul(a1, rcp(n1)), f1, mul(mul(a2, rcp(n2)), f2)));
     const float2 C = fma2(f0, f0, fma2(f1, f1, mul(f2, f2)));
     const float2 uu = fma2(u0, u0, fma2(u1, u1, mul(u2, u2)));
-    const float2 iu = rcp(uu), iC = rcp(C);
-    const float kap = 0.84932180f;  // sqrt(log2(e) / 2)
+    const float2 iu = rcp(uu), iC = rcp(C), ru = rsq(uu);
+    const float2 kap = dup(0.84932180f);  // sqrt(log2(e) / 2)
     const float2 r2 = mul(mul(mul(C, n0), mul(mul(n1, iu), n2)), dup(F0.w));
-    g.r11 = make_float2(kap * __fsqrt_rn(r2.x), kap * __fsqrt_rn(r2.y));
-    g.r22 = make_float2(kap * __fsqrt_rn(iC.x), kap * __fsqrt_rn(iC.y));
+    g.r11 = mul(mul(kap, r2), rsq(r2));  // roots to 2 ulps: E holds many times that
+    g.r22 = mul(kap, rsq(C));
     const float2 r12 = mul(mul(B, iC), g.r11);
     g.r12 = make_float2(-r12.x, -r12.y);
     const float2 c1 = fma2(g.r11, px, mul(g.r12, py)), c2 = mul(g.r22, py);
@@ -206,18 +207,18 @@ __device__ __forceinline__ void shaft_cand(const ShaftSmem<GRAD> &sm, const floa
     g.qy = mul(fma2(u0, b0, fma2(u1, b1, mul(u2, b2))), iu);
     const float2 nn = __fadd2_rn(n0, __fadd2_rn(n1, n2));
     const float2 hb = __fadd2_rn(__fadd2_rn(s, pz), fma2(g.qx, px, mul(g.qy, py)));
-    auto lim = [&](float nn1, float nmin, float px1, float py1, float s1, float iu1, float o, float h1, float &thr,
+    auto lim = [&](float nn1, float nmin, float px1, float py1, float s1, float ru1, float o, float h1, float &thr,
                    float &h) {
-        const float L = fminf(F3.w, __log2f(o) - F4.w), m = sqrtf(fmaxf(L, 0.0f));  // |v| <= m; 1.18 m sigma
-        const float wn = sqrtf(nn1), reach = fmaf(1.18f * m, rsqrtf(nmin), F2.w + fabsf(px1) + fabsf(py1)),
+        const float L = fminf(F3.w, __log2f(o) - F4.w), l = fmaxf(L, 1e-20f), m = l * rsqrtf(l);  // |v| <= m; 1.18 m sigma
+        const float wn = nn1 * rsqrtf(nn1), reach = fmaf(1.18f * m, rsqrtf(nmin), F2.w + fabsf(px1) + fabsf(py1)),
                     sl = fabsf(s1) * F1.w;
         const float E = wn * fmaf(2.4e-6f, reach, 4e-7f * sl);
         thr = fmaf(E, fmaf(2.0f, m, E), fmaf(L, 1.000001f, 1e-5f));
-        h = fmaf(2e-6f, fmaf(wn * (reach + sl), sqrtf(iu1), fabsf(s1)), h1);
+        h = fmaf(2e-6f, fmaf(wn * (reach + sl), ru1, fabsf(s1)), h1);
     };
     const float na = fminf(n0.x, fminf(n1.x, n2.x)), nb = fminf(n0.y, fminf(n1.y, n2.y));
-    lim(nn.x, na, px.x, py.x, s.x, iu.x, a[0].w, hb.x, g.thr.x, g.h.x);
-    lim(nn.y, nb, px.y, py.y, s.y, iu.y, b[0].w, hb.y, g.thr.y, g.h.y);
+    lim(nn.x, na, px.x, py.x, s.x, ru.x, a[0].w, hb.x, g.thr.x, g.h.x);
+    lim(nn.y, nb, px.y, py.y, s.y, ru.y, b[0].w, hb.y, g.thr.y, g.h.y);
 }
 
 // gauss_eval of two pairs at once, each operation rounded as there.
