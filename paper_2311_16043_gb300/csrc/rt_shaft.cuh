@@ -28,7 +28,7 @@
 // 182k warp instructions per 32 rays of the 2M-Gaussian object scene (307 per
 // node visit, of which a ray needs half); this takes ~28k, 0.7 of them in
 // steps 1 and 3.  Measured, trace only, against that walk (2M x 64
-// directions: 751 -> 125 ms, 1.0 G rays/s) and the per-ray walk (300k x 128:
+// directions: 751 -> 123 ms, 1.0 G rays/s) and the per-ray walk (300k x 128:
 // 96 -> 26.5 ms, 1.45 G rays/s).  Bound: instruction issue (0.7 of the slots;
 // the rest fixed-latency dependences), with shared memory at 0.65 of its
 // wavefronts; DRAM 0.1 %.  Choices measured on the way (300k / 2M scenes):

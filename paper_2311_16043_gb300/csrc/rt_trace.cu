@@ -125,9 +125,9 @@ int persistent_blocks(const void *kernel, int threads) {
 }
 
 // Lanes per ray that AUTO takes for m rays.  300k object scene, shadow rays in
-// no order, us with 32 / 16 / 8 / 4 lanes: 2,000 rays 50 / 69 / 101 / 176; 20,000 122 / 122 / 154 / 230; 100,000
-// 433 / 368 / 325 / 361; 250,000 1,019 / 836 / 683 / 667; 600,000 2,384 /
-// 1,929 / 1,491 / 1,322.  Beyond 2^20 Gaussians nodes and records exceed the L2
+// no order, us with 32 / 16 / 8 / 4 lanes: 2,000 rays 50 / 69 / 101 / 176; 20,000
+// 122 / 122 / 154 / 230; 100,000 433 / 368 / 325 / 361; 250,000 1,019 / 836 / 683 /
+// 667; 600,000 2,384 / 1,929 / 1,491 / 1,322.  Beyond 2^20 Gaussians nodes and records exceed the L2
 // cache and more lanes hide its misses: 1M rays of the 2M scene 6,138 / 5,724 /
 // 5,302 / 6,443.  4 lanes' stack holds a walk of single nodes through 36 levels.
 // RT_KERNEL_WARP_RAY asked for by name, and the surrogate's fallback with it, keep

@@ -158,6 +158,11 @@ __device__ __forceinline__ bool qnode_ray(float3 o, float3 d, float3 &inv, float
            fabsf(d.z) < inf;
 }
 
+// slab's relative allowance on the far distance, as a factor: a box behind a ray
+// from so far off that o inv overflows has it at -inf, where fa + 1e-6 |fa| is
+// NaN and would pass, and each such ray would walk the whole tree.
+constexpr float kFarMargin = 1.0000011f;
+
 // The four children of a 64-byte node against a ray: child refs, and each
 // box's entry distance (in units of qnode_ray), +inf where the ray misses the
 // box or there is no child.  A plane's distance is (1 + k / 2^15) a + c with
@@ -168,10 +173,6 @@ __device__ __forceinline__ bool qnode_ray(float3 o, float3 d, float3 &inv, float
 // L1 data pipe, a wavefront per lane and load.  Not kept in L1, which these
 // walks hit 0.2 of the time and whose fills cost the same pipe (2 to 2.5 %);
 // CACHED: kept, for walks bound by a ray's latency.
-// kFarMargin: slab's relative allowance on the far distance.  A box behind a ray
-// from so far off that o inv overflows has it at -inf, where fa + 1e-6 |fa| would
-// be NaN and pass: each such ray would walk the whole tree.
-constexpr float kFarMargin = 1.0000011f;
 template <bool CACHED = false>
 __device__ __forceinline__ void qnode_near(const float4 *__restrict__ q, float3 inv, float3 oi, float (&tn)[4],
                                            uint32_t (&r)[4]) {
