@@ -258,7 +258,7 @@ __global__ void __launch_bounds__(128) k_backward(BvhDev b, RaySetDev rs, int64_
 // (bound by those: 17.5M hits of 50k Gaussians x 32, 3.1 ms with fixed-point
 // sums, 1.5 ms float32) and the log itself, which cost the forward 1.2 ms.
 // This takes 1.77 / 1.54 ms with 3.4 hits per Gaussian summed before the
-// atomics.  Bound: instruction issue (0.55 of the slots, 16 warps an SM), then
+// atomics.  Bound: instruction issue (0.52 of the slots, 16 warps an SM), then
 // waits for instructions (the code is long) and memory.  Measured on the way
 // (50k, fixed point): Gaussians hit closed up before their atomics, and those
 // all under way before the first result is looked at 3.05 -> 2.44 ms; 4

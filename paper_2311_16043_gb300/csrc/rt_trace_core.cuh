@@ -898,8 +898,8 @@ __device__ __forceinline__ void flush_counts(const TraceAux &aux, const WorkCoun
 // fill the lanes many times over took up to 1.5 times as long (hemisphere sets of
 // the 20k object scene, us: x 16 567 -> 330, x 64 964 -> 751; 300k x 64 28.7 ms
 // either way; a third of the lanes instead of half: 349, 778, 31.0 ms).
-// Bound: the L1 data pipe (0.8 of it; a wavefront per lane and 32-byte load, 78
-// nodes and 71 Gaussians a ray, hit rate 0.2), then issue (0.65).  Measured on
+// Bound: instruction issue (0.78 of the slots), then the L1 data pipe (0.70 of it;
+// a wavefront per lane and 32-byte load, 78 nodes and 71 Gaussians a ray).  Measured on
 // the way, ms for the 300k object scene's hemisphere set x 64, the 200k's
 // environment set x 64 and a uniform 200k's x 16:
 //   128-byte nodes                                44.9   28.7   17.7
@@ -1055,8 +1055,8 @@ __device__ __forceinline__ void trace_refill(const BvhDev &b, const RaySetDev &r
 // `work` counts slots.  A ray's walk has few nodes at a time: with all 32 lanes
 // on it most idle, with few lanes a single ray takes longer (lanes_for,
 // rt_trace.cu).
-// Bound: issue (0.53) and memory latency at 30 warps an SM, then the L1 data
-// pipe (0.50).  600k shadow rays of the 300k object scene: 32 lanes 3.00 ms, 4
+// Bound: issue (0.71) and memory latency at 30 warps an SM, then the L1 data
+// pipe (0.60).  600k shadow rays of the 300k object scene: 32 lanes 3.00 ms, 4
 // lanes 2.02, 64-byte nodes 1.65, leaf queue (12 lanes waiting) 1.38, stacks of
 // 144 entries instead of 256 (more warps, and an L1 that holds something: hit
 // rate 0.02 before) 1.32; 1M rays of the 2M scene 7.9 -> 6.4 by the last alone.
