@@ -549,8 +549,8 @@ __global__ void __launch_bounds__(128 * INF_WG, 1) k_mlp_infer(MlpDev net, Sampl
 // and the rays in the last backward epilogue, so the two rounds of dependent
 // global loads do not stall the tile; warpgroups 0-2 encode them while the
 // dW1 products run.
-// Bound: the chain of MMA, TMEM load, epilogue and barrier, eight a tile (0.2 of
-// the tensor pipe, 0.28 of the issue slots; shared memory holds one tile).
+// Bound: the chain of MMA, TMEM load, epilogue and barrier, eight a tile (0.28 of
+// the tensor pipe, 0.32 of the issue slots; shared memory holds one tile).
 // 262,144 samples: 197 us with dW before dX in one commit and the encoding at
 // the top of the tile, 193.5 with the epilogue of dX over the dW products,
 // 182 with the encoding under the dW1 products too; the same bits.
